@@ -109,7 +109,8 @@ typedef struct gs_config {
     int32_t persistent;    /* 1: binned raster runs persistent CTAs over tiles in
                               descending span order */
     int32_t repair_in_raster; /* EXACT only, 1 (default): gs_sort_or_bin sorts only
-                              segments longer than 2048 entries and gs_rasterize_fwd
+                              segments longer than 2048 entries (8 x 8 tiles:
+                              512) and gs_rasterize_fwd
                               sorts each segment it reaches in shared memory just
                               before compositing it, so segments past every
                               pixel's termination are never sorted.  The image is
@@ -118,7 +119,9 @@ typedef struct gs_config {
     int32_t chunk_cap;     /* EXACT with repair_in_raster: the most entries of
                               consecutive bins the raster loads and sorts at once
                               (a tile's repair bins; a single longer segment of up
-                              to 2048 forms one on its own); 32..2048, 0 = 256 */
+                              to 2048 forms one on its own; at most one staging
+                              batch, 256 entries or 128 for 8 x 8 tiles, whatever
+                              is set); 32..2048, 0 = 256 */
     int32_t planner;       /* EXACT with repair_in_raster and the tile cull, 1: the
                               bin planner (an MLP over the tile's depth-bin
                               statistics, weights set with gs_planner_set_weights)
@@ -327,9 +330,9 @@ int gs_depth_range_noalloc(const gs_config* cfg, const void* projected, const fl
  *   back sorted, so [span start, tile_end) of every tile is left in
  *   (depth, gid) order (the stream stays valid for any later raster).
  * stream_words is only read otherwise.
- * The GLOBAL kernel is the plain baseline (gsplat-style batch staging); the
- * binned kernel adds the conservative tile-alpha cull and colour staging of
- * the paper's default configuration.  Both give identical images.
+ * GLOBAL streams take the plain raster (every entry of the tile visited by
+ * every warp); binned ones add the conservative tile-alpha cull and per-warp
+ * masks of the paper's default configuration.  Both give identical images.
  */
 int gs_rasterize_fwd(gs_ctx* ctx, const void* projected, int64_t n, const gs_camera* cam,
                      uint64_t* stream_words, const int32_t* offsets, int32_t offsets_stride,

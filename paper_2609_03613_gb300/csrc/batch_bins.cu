@@ -447,7 +447,7 @@ int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m
     gc->launches += 2;
     GS_CUDA_TRY(cudaGetLastError());
     // segments longer than the raster sorts in shared memory
-    return sort_long_segments(gc, NS, gc->r_off, gc->r_stream, kRasterSortCap + 1, st);
+    return sort_long_segments(gc, NS, gc->r_off, gc->r_stream, raster_sort_cap(16) + 1, st);
 }
 
 }  // namespace gs

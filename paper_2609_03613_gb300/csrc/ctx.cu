@@ -407,7 +407,7 @@ extern "C" int gs_sort_or_bin(gs_ctx* ctx, const void* projected, const float* s
         if (r != GS_OK) return r;
         stage_begin(ctx, GS_STAGE_REPAIR, st);
         r = repair_min(ctx, T, m_dev, stream_words, offsets, nullptr,
-                       ctx->cfg.repair_in_raster ? kRasterSortCap + 1 : 2, st);
+                       ctx->cfg.repair_in_raster ? raster_sort_cap(ctx->cfg.tile_size) + 1 : 2, st);
         stage_end(ctx, GS_STAGE_REPAIR, st);
         return r;
     }
@@ -431,10 +431,9 @@ extern "C" int gs_rasterize_fwd(gs_ctx* ctx, const void* projected, int64_t n, c
     if (n > 0 && (!projected || !stream_words)) return GS_ERR_INVALID_ARG;
     if (offsets_stride < 1 || offsets_stride > GS_MAX_K) return GS_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    const bool baseline = baseline_raster(ctx->cfg);
     stage_begin(ctx, GS_STAGE_RASTER, st);
     int r = raster_fwd(ctx, proj_view(const_cast<void*>(projected), n), cam, stream_words, offsets,
-                       offsets_stride, bg, rgb, alpha, last, ntests, baseline, st, final_T, tile_end);
+                       offsets_stride, bg, rgb, alpha, last, ntests, st, final_T, tile_end);
     stage_end(ctx, GS_STAGE_RASTER, st);
     return r;
 }
@@ -466,7 +465,7 @@ extern "C" int gs_rasterize_fwd_plan(gs_ctx* ctx, const void* projected, int64_t
     }
     stage_begin(ctx, GS_STAGE_RASTER, st);
     r = raster_fwd(ctx, proj_view(const_cast<void*>(projected), n), cam, stream_words, offsets, offsets_stride, bg,
-                   rgb, alpha, last, nullptr, false, st, nullptr, nullptr, pl);
+                   rgb, alpha, last, nullptr, st, nullptr, nullptr, pl);
     stage_end(ctx, GS_STAGE_RASTER, st);
     if (r == GS_OK && flags)
         GS_CUDA_TRY(cudaMemcpyAsync(flags, ctx->d_plan + T, (size_t)T, cudaMemcpyDeviceToDevice, st));
@@ -629,7 +628,7 @@ int gs::render_binning(gs_ctx* c, int64_t n, const float* scales, const gs_camer
         if (r != GS_OK) return r;
         stage_begin(c, GS_STAGE_REPAIR, st);
         r = repair_min(c, T, c->r_m, c->r_stream, c->r_off, nullptr,
-                       c->cfg.repair_in_raster ? kRasterSortCap + 1 : 2, st, planned ? 1 : 0);
+                       c->cfg.repair_in_raster ? raster_sort_cap(c->cfg.tile_size) + 1 : 2, st, planned ? 1 : 0);
         stage_end(c, GS_STAGE_REPAIR, st);
     } else {
         r = emit_only(c, pv, n, cam, isect_view(c->r_isect, c->r_m_cap), c->r_m_cap, c->r_m, st);
@@ -665,7 +664,7 @@ int gs::render_after_project(gs_ctx* c, int64_t n, const float* scales, const gs
     // resumes pixels whose stops it does not know: tile ends only)
     int32_t* wend = save && !planned ? c->r_wend : nullptr;
     r = raster_fwd(c, pv, cam, c->r_stream, c->r_off, stride, bg, d_rgb, d_alpha, d_last, nullptr,
-                   baseline_raster(c->cfg), st, save ? c->r_T : nullptr, save ? c->r_tend : nullptr, pl, wend);
+                   st, save ? c->r_T : nullptr, save ? c->r_tend : nullptr, pl, wend);
     stage_end(c, GS_STAGE_RASTER, st);
     if (r != GS_OK) return r;
     if (planned) {
@@ -673,7 +672,7 @@ int gs::render_after_project(gs_ctx* c, int64_t n, const float* scales, const gs
         // segments sorted, the tiles composited on from where they stopped
         stage_begin(c, GS_STAGE_COMPLETE, st);
         r = exact_scatter_rest(c, n, cam, c->r_m_cap, c->r_m, c->r_stream, c->r_off, st);
-        if (r == GS_OK) r = repair_min(c, T, c->r_m, c->r_stream, c->r_off, nullptr, kRasterSortCap + 1, st, 2);
+        if (r == GS_OK) r = repair_min(c, T, c->r_m, c->r_stream, c->r_off, nullptr, raster_sort_cap(c->cfg.tile_size) + 1, st, 2);
         if (r == GS_OK)
             r = raster_listed(c, pv, cam, c->r_stream, c->r_off, stride, bg, d_rgb, d_alpha, d_last, c->d_plan,
                               c->d_plist, st, save ? c->r_T : nullptr, save ? c->r_tend : nullptr);

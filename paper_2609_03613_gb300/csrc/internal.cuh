@@ -468,8 +468,9 @@ int repair_min(gs_ctx* ctx, int32_t n_tiles, const int64_t* m_dev, uint64_t* str
 int sort_long_segments(gs_ctx* ctx, int64_t nseg, const int32_t* offsets, uint64_t* words, int32_t min_len,
                        cudaStream_t st);
 // segments longer than this are sorted before the raster when the raster
-// sorts the segments it reaches
-constexpr int kRasterSortCap = 2048;
+// sorts the segments it reaches (8 x 8 tiles: a smaller buffer, so that more
+// of their one-warp blocks fit an SM)
+__host__ __device__ constexpr int raster_sort_cap(int tile) { return tile == 8 ? 512 : 2048; }
 // Classes of the bin planner: class c < kPlanClasses - 1 gives a tile's first
 // pass the fewest bins from its front that hold at least plan_entries(c)
 // entries; the last class gives it every bin.
@@ -531,10 +532,6 @@ struct PlanView {
 };
 // the configured chunk size of the lazy EXACT raster
 inline int chunk_cap(const gs_config& cfg) { return cfg.chunk_cap > 0 ? cfg.chunk_cap : 256; }
-// The plain baseline raster kernel serves GLOBAL mode without the tile cull;
-// every other configuration (GLOBAL with the cull included) uses the binned
-// kernel, which culls at staging when the stream was not culled when built.
-inline bool baseline_raster(const gs_config& cfg) { return cfg.mode == GS_MODE_GLOBAL_SORT && !cfg.tile_cull; }
 // depth range with samples mapped to gids through the per-Gaussian offsets
 int depth_range_goff(gs_ctx* ctx, const ProjView& pv, const float* scales, int64_t n, int64_t m_cap,
                      const int64_t* m_dev, const gs_camera* cam, cudaStream_t st);
@@ -542,7 +539,7 @@ int depth_range_goff(gs_ctx* ctx, const ProjView& pv, const float* scales, int64
 // raster.cu
 int raster_fwd(gs_ctx* ctx, const ProjView& pv, const gs_camera* cam, uint64_t* stream_words,
                const int32_t* offsets, int32_t stride, const float* bg, float* rgb, float* alpha,
-               int32_t* last, int32_t* ntests, bool baseline, cudaStream_t st, float* final_T = nullptr,
+               int32_t* last, int32_t* ntests, cudaStream_t st, float* final_T = nullptr,
                int32_t* tile_end = nullptr, const PlanView& plan = PlanView(), int32_t* warp_end = nullptr);
 // the completing pass of a planned frame: every tile of list (device {count,
 // tiles...}) composited on from the bin where its first pass stopped (plan

@@ -1,8 +1,8 @@
 // raster.cu -- K6 / K16: front-to-back compositing over each tile's span of
 // the tile-major stream (Sec. 3.4; supplement "Binned raster traversal after
-// repair").  One CTA per tile, one thread per pixel, the span consumed in
-// batches of one entry per thread staged through shared memory, and a
-// block-wide vote ends the tile once every pixel has terminated.
+// repair").  One CTA per tile, two pixels a thread, the span consumed in
+// batches staged through shared memory, and a block-wide vote ends the tile
+// once every pixel has terminated.
 //
 // Per pixel centre (x + 0.5, y + 0.5) and entry in stream order, in this exact
 // float32 order (the same as the compositing definition of the library):
@@ -13,252 +13,382 @@
 //   Tn = T*(1 - alpha); stop before applying if Tn < 1e-4
 //   C = fmaf(col, alpha*T, C); T = Tn; last = gid
 //
-// Two kernels, identical images:
-//   baseline -- the plain kernel of the global-sort path: stages
-//               (mean, conic, opacity) per batch, evaluates exp for every
-//               test, reads colours from global memory when applied;
-//   binned   -- the paper's default raster additions: a conservative
-//               tile-level alpha cull at staging (entries that cannot reach
-//               alpha >= 1/255 anywhere in the tile are dropped, order kept),
-//               colour staging, and a per-entry early-out q > tau with
-//               tau >= ln(255 o), past which alpha < 1/255 is certain.
+// One kernel for every stream.  Binned streams take the paper's default raster
+// additions: a conservative tile-level alpha cull at staging (entries that
+// cannot reach alpha >= 1/255 anywhere in the tile are dropped, order kept;
+// EXACT streams were culled when built) and per-warp masks.  The plain raster
+// of the global-sort path takes neither: every warp visits every entry.  In
+// both an entry's exp is evaluated only where q <= tau matters, tau >= ln(255
+// o), past which alpha < 1/255 is certain.  The images are identical.
 #include <string.h>
 
 #include "raster_common.cuh"
 
 namespace gs {
 
-// Per-thread compositing state.
-struct PixelState {
-    float T, C0, C1, C2;
-    int32_t last, ntests;
-    int32_t stop;  // stream position of the entry that stopped the pixel
-    unsigned long long ops;
-    bool done;
-};
+// A warp's block of pixels and its lanes: 8 x 8 pixels, two a lane, (x, y) and
+// (x + 4, y).  They share dy and the entry's shared-memory reads, and what is
+// done to both runs on packed float32 pairs (each half rounded as the scalar
+// operation).
+constexpr int kBH = 8;
 
-// The binned step at one pixel once q and exp(-q) are known.  exp(-q) is
-// evaluated for every q -- its value is used only when 0 <= q <= tau, where
-// it lies inside the core's range -- and the step has no early exit but the
-// stop, so a warp issues the tests of two entries without diverging around
-// each one (raster 0.296 -> 0.274 ms at 1080p against the form that
-// branched past the exp and the colour update).  Returns true when the pixel
-// stops (the entry is not applied).
-template <bool COUNT>
-__device__ __forceinline__ bool composite_binned(float q, float e, const float4& gb, const float4& col,
-                                                 PixelState& st)
+// ------------------------------------------------------------------ packed float32 pairs
+__device__ __forceinline__ uint64_t pk2(float lo, float hi)
 {
-    // 0 <= q <= tau as one unsigned compare of the float bits
-    // (negative q and NaN compare above any positive tau)
-    const bool inq = __float_as_uint(q) <= __float_as_uint(gb.z);
-    const float alpha = fminf(0.99f, gb.y * e);
-    const bool pass = inq && alpha >= 1.0f / 255.0f;
-    const float Tn = st.T * (1.0f - alpha);
-    if (COUNT) {
-        ++st.ntests;
-        st.ops += 8 + (inq ? 17 : 0) + (pass ? 3 : 0);
-    }
-    if (pass && Tn < 1e-4f) {
-        st.done = true;
-        return true;
-    }
-    if (pass) {
-        if (COUNT) st.ops += 4;
-        const float w = alpha * st.T;
-        st.C0 = fmaf(col.x, w, st.C0);
-        st.C1 = fmaf(col.y, w, st.C1);
-        st.C2 = fmaf(col.z, w, st.C2);
-        st.T = Tn;
-        st.last = __float_as_int(gb.w);
-    }
-    return false;
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void upk2(uint64_t v, float& lo, float& hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t same2(float v) { return pk2(v, v); }
+
+// exp(-q) of two q by spec_exp_core's steps (internal.cuh), bit for bit where
+// its value is used (0 <= q <= 87).  The reduced argument is carried negated
+// (s = -r), which mirrors every rounding: the odd Horner stages come out
+// negated and the last one does not.  2^n is applied to the normal result by
+// adding n to its exponent field: the low 9 bits of the shifter's bits are
+// zero, so bits(k) << 23 is n << 23.
+__device__ __forceinline__ void spec_exp_neg2(float q0, float q1, float& e0, float& e1)
+{
+    const uint64_t q = pk2(q0, q1);
+    const uint64_t k = fma2(q, same2(-1.44269504088896341f), same2(12582912.0f));
+    const uint64_t n = add2(k, same2(-12582912.0f));
+    uint64_t s = fma2(n, same2(0.693145751953125f), q);
+    s = fma2(n, same2(1.42860682030941723e-6f), s);
+    uint64_t p = fma2(same2(-1.0f / 5040.0f), s, same2(1.0f / 720.0f));
+    p = fma2(p, s, same2(-1.0f / 120.0f));
+    p = fma2(p, s, same2(1.0f / 24.0f));
+    p = fma2(p, s, same2(-1.0f / 6.0f));
+    p = fma2(p, s, same2(0.5f));
+    p = fma2(p, s, same2(-1.0f));
+    p = fma2(p, s, same2(1.0f));
+    float p0, p1, k0, k1;
+    upk2(p, p0, p1);
+    upk2(k, k0, k1);
+    e0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(k0) << 23));
+    e1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(k1) << 23));
 }
 
-// One entry at one pixel, q given: the compositing definition's steps.
-// Returns true when the pixel stops (the entry is not applied).
-template <bool BASELINE, bool COUNT, class SH>
-__device__ __forceinline__ bool composite_entry(float q, const float4& ga, const float4& gb, const SH& sh, int k,
-                                                const float4* __restrict__ rgbv, PixelState& st)
+// Per-thread compositing state: two pixels.  A pixel that has stopped (or lies
+// outside the image) has a NaN centre, so that no entry passes it again.
+struct PixelState {
+    float x[2], y;  // pixel centres
+    uint64_t T, C0, C1, C2;  // packed, pixel 0 in the low half
+    int32_t last[2], ntests[2];
+    int32_t stop;   // stream position of the entry that stopped a pixel last
+    int live;       // bit h: pixel h is still compositing
+    unsigned long long ops;
+};
+
+// One staged entry at both pixels: q of each.
+__device__ __forceinline__ void entry_q(const float4& ga, const float4& gb, const PixelState& st, float& q0, float& q1)
 {
-    if constexpr (!BASELINE) {
-        return composite_binned<COUNT>(q, spec_exp_core(-q), gb, sh.c[k], st);
-    } else {
-        if (COUNT) {
-            ++st.ntests;
-            st.ops += 8;
+    const float dy = ga.y - st.y;
+    const uint64_t dx = pk2(ga.x - st.x[0], ga.x - st.x[1]);
+    upk2(fma2(dx, fma2(same2(ga.z), dx, same2(ga.w * dy)), same2((gb.x * dy) * dy)), q0, q1);
+}
+
+// alpha of one entry where the pixel takes it (pass), else 0.  0 <= q <= tau
+// as one unsigned compare of the float bits (negative q and NaN compare above
+// any positive tau).
+struct EntryAlpha {
+    float a0, a1;
+    bool pass0, pass1;
+};
+__device__ __forceinline__ EntryAlpha entry_alpha(float q0, float q1, const float4& gb)
+{
+    float e0, e1;
+    spec_exp_neg2(q0, q1, e0, e1);
+    upk2(mul2(same2(gb.y), pk2(e0, e1)), e0, e1);
+    const float f0 = fminf(0.99f, e0), f1 = fminf(0.99f, e1);
+    const uint32_t tau = __float_as_uint(gb.z);
+    EntryAlpha r;
+    r.pass0 = __float_as_uint(q0) <= tau && f0 >= 1.0f / 255.0f;
+    r.pass1 = __float_as_uint(q1) <= tau && f1 >= 1.0f / 255.0f;
+    r.a0 = r.pass0 ? f0 : 0.0f;
+    r.a1 = r.pass1 ? f1 : 0.0f;
+    return r;
+}
+
+// C = fma(colour, w, C) at both pixels.
+__device__ __forceinline__ void add_colour(const float4& c, uint64_t w, PixelState& st)
+{
+    st.C0 = fma2(same2(c.x), w, st.C0);
+    st.C1 = fma2(same2(c.y), w, st.C1);
+    st.C2 = fma2(same2(c.z), w, st.C2);
+}
+
+// T (1 - alpha) at both pixels, 1 - alpha rounded once.
+__device__ __forceinline__ uint64_t transmit(uint64_t T, uint64_t a)
+{
+    return mul2(T, fma2(a, same2(-1.0f), same2(1.0f)));
+}
+
+// One entry (id g, stream position pos) with its stops: a pixel whose
+// transmittance would fall below 1e-4 stops before it is applied.
+__device__ __forceinline__ void apply_with_stops(const EntryAlpha& e, const float4& c, int32_t g, int32_t pos,
+                                                 PixelState& st)
+{
+    float T[2], t[2], a[2] = {e.a0, e.a1};
+    upk2(st.T, T[0], T[1]);
+    upk2(transmit(st.T, pk2(a[0], a[1])), t[0], t[1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (((st.live >> h) & 1) && t[h] < 1e-4f) {
+            st.live &= ~(1 << h);
+            st.x[h] = __uint_as_float(0x7fc00000u);
+            st.stop = pos;
         }
-        if (!(q >= 0.0f)) return false;
-        // every q >= 0 reaches exp here: the clamped form (exp(-q) for
-        // q > 87 would leave the 2^n range)
-        const float e = spec_exp(-q);
-        const float alpha = fminf(0.99f, gb.y * e);
-        if (COUNT) st.ops += 17;
-        if (alpha < 1.0f / 255.0f) return false;
-        const float Tn = st.T * (1.0f - alpha);
-        if (COUNT) st.ops += 3;
-        if (Tn < 1e-4f) {
-            st.done = true;
-            return true;
+        if (!((st.live >> h) & 1)) {
+            a[h] = 0.0f;
+            t[h] = T[h];
         }
-        if (COUNT) st.ops += 4;
-        const float w = alpha * st.T;
-        const float4 col = __ldg(rgbv + sh.g[k]);
-        st.C0 = fmaf(col.x, w, st.C0);
-        st.C1 = fmaf(col.y, w, st.C1);
-        st.C2 = fmaf(col.z, w, st.C2);
-        st.T = Tn;
-        st.last = __float_as_int(gb.w);
-        return false;
+        if (a[h] > 0.0f) st.last[h] = g;
     }
+    add_colour(c, mul2(pk2(a[0], a[1]), st.T), st);
+    st.T = pk2(t[0], t[1]);
 }
 
 // Composite the cnt staged entries of a batch into the calling thread's
-// pixel (slot k is stream position base + k).  Binned: the warp composites
-// only the entries its warp mask admits.
-template <int TILE, bool BASELINE, bool COUNT>
-__device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE, BASELINE>& sh,
-                                                const float4* __restrict__ rgbv, float pxc, float pyc, PixelState& st,
-                                                int32_t base)
+// pixels (slot k is stream position base + k); the warp visits the entries
+// its mask admits.  The whole warp stays in the loop until all its pixels have
+// stopped (a stopped one passes nothing), so no branch in it diverges.  R
+// entries (2 or 4) go a round: a pixel's transmittance after all of them tells
+// whether any stopped it (it never grows), so one vote a round looks for
+// stops; a round without one (five in six of two at 1080p) is one straight
+// run, the others go entry by entry.
+//
+// What bounds it: register reads and issue together.  A packed multiply-add
+// reads three register pairs and takes 2.3 to 3 cycles of a scheduler where
+// two scalar ones take 2 to 3 (measured), so packing buys issue slots, not
+// arithmetic; a round of two takes about 110 instructions for 2 x 64 tests.  Measured
+// raster times, 1M Gaussians at 1080p / 3M inside a cluster at 1080p / 500k
+// global at 720p: one pixel a lane, scalar, 8 x 4 blocks 254 / 207 / 560 us;
+// this loop with lanes leaving at their stops 250 / 180 / 481 us; with the
+// stops in their own path 235 / 168 / 457 us; with q, opacity and colour
+// packed too 229 / 164 / 446 us, the last 276 with SKIP.  Scalar exps 254 / 178 / 496 us; one pixel a
+// lane with two entries packed 248 / 203 / 516 us.
+//
+// SKIP (the plain raster, whose warps visit entries far from their pixels):
+// a round no pixel of which has q <= tau ends there.
+template <int TILE, bool SKIP, int R>
+__device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE, kBH>& sh, PixelState& st, int32_t base)
 {
     const int warp = threadIdx.x >> 5;
-    int nk = cnt;
-    if constexpr (!BASELINE) nk = __all_sync(0xffffffffu, st.done) ? 0 : warp_strip_list<TILE>(sh, cnt);
-    if (st.done) return;
-    if constexpr (BASELINE) {
-        for (int k = 0; k < nk; ++k) {
-            const float4 ga = sh.a[k];
-            const float4 gb = sh.b[k];
-            const float dx = ga.x - pxc, dy = ga.y - pyc;
-            const float q = fmaf(dx, fmaf(ga.z, dx, ga.w * dy), (gb.x * dy) * dy);
-            if (composite_entry<BASELINE, COUNT>(q, ga, gb, sh, k, rgbv, st)) {
-                st.stop = base + k;
-                break;
-            }
+    if (__all_sync(0xffffffffu, st.live == 0)) return;
+    const int nk = warp_strip_list<TILE, kBH>(sh, cnt);
+    const char* pa = reinterpret_cast<const char*>(sh.a);
+    const char* pb = reinterpret_cast<const char*>(sh.b);
+    const char* pc = reinterpret_cast<const char*>(sh.c);
+    for (int i = 0; i < nk; i += R) {
+        uint32_t k[R];
+#pragma unroll
+        for (int j = 0; j < R; j += 2) {
+            const uint32_t pair = *reinterpret_cast<const uint32_t*>(&sh.list[warp][i + j]);
+            k[j] = pair & 0xffffu;
+            k[j + 1] = pair >> 16;
         }
-    } else {
-        // two entries a round: both q and exp(-q) first (independent), then
-        // the two compositing steps in stream order
-        int i = 0;
-        for (; i + 1 < nk; i += 2) {
-            const int k0 = sh.list[warp][i], k1 = sh.list[warp][i + 1];
-            const float4 ga0 = sh.a[k0], gb0 = sh.b[k0];
-            const float4 ga1 = sh.a[k1], gb1 = sh.b[k1];
-            const float dx0 = ga0.x - pxc, dy0 = ga0.y - pyc;
-            const float dx1 = ga1.x - pxc, dy1 = ga1.y - pyc;
-            const float q0 = fmaf(dx0, fmaf(ga0.z, dx0, ga0.w * dy0), (gb0.x * dy0) * dy0);
-            const float q1 = fmaf(dx1, fmaf(ga1.z, dx1, ga1.w * dy1), (gb1.x * dy1) * dy1);
-            const float e0 = spec_exp_core(-q0), e1 = spec_exp_core(-q1);
-            if (composite_binned<COUNT>(q0, e0, gb0, sh.c[k0], st)) {
-                st.stop = base + k0;
-                break;
-            }
-            if (composite_binned<COUNT>(q1, e1, gb1, sh.c[k1], st)) {
-                st.stop = base + k1;
-                break;
-            }
+        float4 gb[R];
+        float q[R][2];
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            gb[j] = *reinterpret_cast<const float4*>(pb + k[j]);
+            entry_q(*reinterpret_cast<const float4*>(pa + k[j]), gb[j], st, q[j][0], q[j][1]);
         }
-        if (!st.done && i < nk) {
-            const int k = sh.list[warp][i];
-            const float4 ga = sh.a[k], gb = sh.b[k];
-            const float dx = ga.x - pxc, dy = ga.y - pyc;
-            const float q = fmaf(dx, fmaf(ga.z, dx, ga.w * dy), (gb.x * dy) * dy);
-            if (composite_entry<BASELINE, COUNT>(q, ga, gb, sh, k, rgbv, st)) st.stop = base + k;
+        if constexpr (SKIP) {
+            bool any = false;
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                any |= min(__float_as_uint(q[j][0]), __float_as_uint(q[j][1])) <= __float_as_uint(gb[j].z);
+            if (!__any_sync(0xffffffffu, any)) continue;
+        }
+        EntryAlpha e[R];
+        uint64_t A[R], T[R + 1];
+        T[0] = st.T;
+#pragma unroll
+        for (int j = 0; j < R; ++j) e[j] = entry_alpha(q[j][0], q[j][1], gb[j]);
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            A[j] = pk2(e[j].a0, e[j].a1);
+            T[j + 1] = transmit(T[j], A[j]);
+        }
+        float t0, t1;
+        upk2(T[R], t0, t1);
+        if (__any_sync(0xffffffffu, fminf(t0, t1) < 1e-4f)) {
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                apply_with_stops(e[j], *reinterpret_cast<const float4*>(pc + k[j]), __float_as_int(gb[j].w),
+                                 base + (int32_t)(k[j] >> 4), st);
+            if (__all_sync(0xffffffffu, st.live == 0)) break;
+        } else {
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                add_colour(*reinterpret_cast<const float4*>(pc + k[j]), mul2(A[j], T[j]), st);
+                const int32_t g = __float_as_int(gb[j].w);
+                st.last[0] = e[j].pass0 ? g : st.last[0];
+                st.last[1] = e[j].pass1 ? g : st.last[1];
+            }
+            st.T = T[R];
         }
     }
 }
 
-// Composite n_entries stream words from src (global or shared memory) into
-// every pixel of the tile, in batches.  Returns -1 after the last entry, or,
-// block-uniformly, the offset of the first batch left unprocessed once every
-// pixel of the tile has terminated.
-// cullmode bit 1: tile-alpha cull at staging; bit 2: per-warp strip mask.
-template <int TILE, bool BASELINE, bool COUNT>
-__device__ __forceinline__ int32_t raster_span(const uint64_t* src, int32_t n_entries,
-                                            RasterShared<TILE, BASELINE>& sh, const float4* __restrict__ xy_ab,
-                                            const float4* __restrict__ c_o_z, const float4* __restrict__ rgbv,
-                                            int cullmode, int tx, int ty, float pxc, float pyc, PixelState& st,
-                                            bool checked, int32_t base)
+// The counting twin: one pixel and one entry at a time, the same values.
+template <int TILE>
+__device__ __forceinline__ void composite_batch_count(int cnt, RasterShared<TILE, kBH>& sh, PixelState& st,
+                                                      int32_t base)
 {
-    using SH = RasterShared<TILE, BASELINE>;
-    constexpr int BS = SH::BS, BATCH = SH::BATCH;
-    for (int32_t b0 = 0; b0 < n_entries; b0 += BATCH) {
-        // checked: the caller has just counted the terminated pixels (block
-        // barrier included) with nothing composited since
-        if (!(checked && b0 == 0) && __syncthreads_count(st.done) == BS) return b0;
-        const int cnt = stage_batch<TILE, BASELINE>(src, b0, n_entries, sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty);
-        __syncthreads();
-        composite_batch<TILE, BASELINE, COUNT>(cnt, sh, rgbv, pxc, pyc, st, base + b0);
+    const int warp = threadIdx.x >> 5;
+    const int nk = warp_strip_list<TILE, kBH>(sh, cnt);
+    float T[2], C0[2], C1[2], C2[2];
+    upk2(st.T, T[0], T[1]);
+    upk2(st.C0, C0[0], C0[1]);
+    upk2(st.C1, C1[0], C1[1]);
+    upk2(st.C2, C2[0], C2[1]);
+    for (int i = 0; i < nk && st.live; ++i) {
+        const int k = sh.list[warp][i] >> 4;
+        const float4 ga = sh.a[k], gb = sh.b[k], col = sh.c[k];
+        const float dy = ga.y - st.y;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (!((st.live >> h) & 1)) continue;
+            const float dx = ga.x - st.x[h];
+            const float q = fmaf(dx, fmaf(ga.z, dx, ga.w * dy), (gb.x * dy) * dy);
+            const bool inq = __float_as_uint(q) <= __float_as_uint(gb.z);
+            const float alpha = inq ? fminf(0.99f, gb.y * spec_exp_core(-q)) : 0.0f;
+            const bool pass = alpha >= 1.0f / 255.0f;
+            ++st.ntests[h];
+            st.ops += 8 + (inq ? 17 : 0) + (pass ? 3 : 0);
+            if (!pass) continue;
+            const float Tn = T[h] * (1.0f - alpha);
+            if (Tn < 1e-4f) {
+                st.live &= ~(1 << h);
+                st.x[h] = __uint_as_float(0x7fc00000u);
+                st.stop = base + k;
+                continue;
+            }
+            st.ops += 4;
+            const float w = alpha * T[h];
+            C0[h] = fmaf(col.x, w, C0[h]);
+            C1[h] = fmaf(col.y, w, C1[h]);
+            C2[h] = fmaf(col.z, w, C2[h]);
+            T[h] = Tn;
+            st.last[h] = __float_as_int(gb.w);
+        }
     }
-    return -1;
+    st.T = pk2(T[0], T[1]);
+    st.C0 = pk2(C0[0], C0[1]);
+    st.C1 = pk2(C1[0], C1[1]);
+    st.C2 = pk2(C2[0], C2[1]);
 }
 
-template <int TILE, bool BASELINE, bool COUNT>
+// A run of entries composited into the tile's pixels: what the walk hands its
+// runs and staged chunks to (raster_common.cuh).
+template <int TILE, bool COUNT, bool LAZY, int R>
 struct FwdSpan {
-    RasterShared<TILE, BASELINE>& sh;
+    using SH = RasterShared<TILE, kBH>;
+    static constexpr int kBatch = SH::BATCH;
+    SH& sh;
     const float4* __restrict__ xy_ab;
     const float4* __restrict__ c_o_z;
     const float4* __restrict__ rgbv;
     int cullmode, tx, ty;
-    float pxc, pyc;
     PixelState& st;
+    // n entries from src (global or shared memory) in batches: -1 after the
+    // last, or the offset of the first batch left once every pixel of the
+    // tile has terminated
     __device__ __forceinline__ int32_t operator()(const uint64_t* src, int32_t n, bool checked, int32_t base)
     {
-        return raster_span<TILE, BASELINE, COUNT>(src, n, sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty, pxc, pyc, st,
-                                                  checked, base);
+        for (int32_t b0 = 0; b0 < n; b0 += kBatch) {
+            // checked: the caller has just counted the terminated pixels (block
+            // barrier included) with nothing composited since
+            if (!(checked && b0 == 0) && __syncthreads_count(done()) == SH::TB::NT) return b0;
+            const int cnt = stage_batch<TILE, kBH>(src, b0, n, sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty);
+            __syncthreads();
+            composite_staged(cnt, base + b0);
+        }
+        return -1;
     }
-    __device__ __forceinline__ bool done() const { return st.done; }
-    // binned: a chunk of one batch is staged slot by slot by the walk
-    static constexpr bool kStageAtRank = !BASELINE;
-    static constexpr int kBatch = RasterShared<TILE, BASELINE>::BATCH;
+    __device__ __forceinline__ bool done() const { return st.live == 0; }
     __device__ __forceinline__ void stage_at(int slot, uint32_t g)
     {
-        if constexpr (!BASELINE) {
-            float4 A, B, C;
-            stage_record<TILE>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
-            sh.a[slot] = A;
-            sh.b[slot] = B;
-            sh.c[slot] = C;
-        }
+        float4 A, B, C;
+        stage_record<TILE, kBH>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
+        sh.a[slot] = A;
+        sh.b[slot] = B;
+        sh.c[slot] = C;
     }
     __device__ __forceinline__ void composite_staged(int cnt, int32_t base)
     {
-        composite_batch<TILE, BASELINE, COUNT>(cnt, sh, rgbv, pxc, pyc, st, base);
+        if constexpr (COUNT) {
+            composite_batch_count<TILE>(cnt, sh, st, base);
+        } else {
+            if constexpr (!LAZY)
+                if (cullmode & kPlain) return composite_batch<TILE, true, R>(cnt, sh, st, base);
+            composite_batch<TILE, false, R>(cnt, sh, st, base);
+        }
     }
 };
 
 // LAZY (EXACT mode with the repair in the raster): the tile's segments are
-// walked front to back; each segment of 2..kRasterSortCap entries is loaded
-// into shared memory and sorted by (depth bits, gid) right before it is
+// walked front to back; each segment of 2..raster_sort_cap(TILE) entries is
+// loaded into shared memory and sorted by (depth bits, gid) right before it is
 // composited (longer ones were sorted eagerly), so segments after every
 // pixel's termination are never sorted.
-// One tile t by the whole block (the body of both raster kernels below).
-template <int TILE, bool BASELINE, bool COUNT, bool LAZY>
+// One tile t by the whole block (the body of the raster kernels below).
+template <int TILE, bool COUNT, bool LAZY, int R>
 __device__ __forceinline__ void raster_tile(
-    int t, RasterShared<TILE, BASELINE>& sh, WalkShared<LAZY>& ws, const float4* __restrict__ xy_ab,
+    int t, RasterShared<TILE, kBH>& sh, WalkShared<TILE, LAZY>& ws, const float4* __restrict__ xy_ab,
     const float4* __restrict__ c_o_z, const float4* __restrict__ rgbv, uint64_t* words,
     const int32_t* __restrict__ off, const RasterArgs& a, int cullmode, float* __restrict__ out_rgb,
     float* __restrict__ out_alpha, int32_t* __restrict__ out_last, int32_t* __restrict__ out_ntests,
     unsigned long long* __restrict__ ops_total, float* __restrict__ out_T, int32_t* __restrict__ out_end,
     const PlanView& pl, int cap, int32_t* __restrict__ out_wend = nullptr)
 {
+    using TB = TileBlocks<TILE, kBH>;
     const int tx = t % a.tiles_x, ty = t / a.tiles_x;
-    const int lx = WarpBlocks<TILE>::lx(), ly = WarpBlocks<TILE>::ly();
-    const int px = tx * TILE + lx, py = ty * TILE + ly;
-    const bool inside = px < a.width && py < a.height;
-    const float pxc = (float)px + 0.5f, pyc = (float)py + 0.5f;
+    const int lane = threadIdx.x & 31;
+    // the lane's first pixel; the second is four to its right
+    const int px = tx * TILE + TB::x0() + (lane & 3), py = ty * TILE + TB::y0() + (lane >> 2);
+    const int inside = py < a.height ? (px < a.width ? 1 : 0) | (px + 4 < a.width ? 2 : 0) : 0;
 
     // float32 operations of the compositing definition each pixel executes
     // (COUNT builds): 8 per visit (offsets, q, sign test), 17 more when exp is
     // evaluated (exp, o*e, clamp, threshold), 3 when alpha passes (1-alpha,
     // T*, stop test), 4 when applied (alpha*T and three colour fmas)
     PixelState st;
-    st.T = 1.0f;
-    st.C0 = st.C1 = st.C2 = 0.0f;
-    st.last = -1;
-    st.ntests = 0;
+    st.y = (float)py + 0.5f;
+    st.T = same2(1.0f);
+    st.C0 = st.C1 = st.C2 = 0ull;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        st.last[h] = -1;
+        st.ntests[h] = 0;
+    }
     st.stop = -1;
     st.ops = 0;
-    st.done = !inside;
+    st.live = inside;
 
     const int K = a.stride;
     int kbegin = 0, kend = K;
@@ -267,42 +397,54 @@ __device__ __forceinline__ void raster_tile(
         if (pl.resume) kbegin = B;
         else kend = B;
     }
-    if (pl.resume && inside) {
-        const int64_t p = (int64_t)py * a.width + px;
-        // the first pass's state: C in rgb, T in alpha (negative once the
-        // pixel stopped), last
-        const float Ts = out_alpha[p];
-        st.T = fabsf(Ts);
-        st.done = signbit(Ts);
-        st.C0 = out_rgb[3 * p];
-        st.C1 = out_rgb[3 * p + 1];
-        st.C2 = out_rgb[3 * p + 2];
-        st.last = out_last[p];
+    if (pl.resume) {
+        float T[2] = {1.0f, 1.0f}, C[3][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if ((inside >> h) & 1) {
+                const int64_t p = (int64_t)py * a.width + px + 4 * h;
+                // the first pass's state: C in rgb, T in alpha (negative once the
+                // pixel stopped), last
+                const float Ts = out_alpha[p];
+                T[h] = fabsf(Ts);
+                if (signbit(Ts)) st.live &= ~(1 << h);
+                C[0][h] = out_rgb[3 * p];
+                C[1][h] = out_rgb[3 * p + 1];
+                C[2][h] = out_rgb[3 * p + 2];
+                st.last[h] = out_last[p];
+            }
+        st.T = pk2(T[0], T[1]);
+        st.C0 = pk2(C[0][0], C[0][1]);
+        st.C1 = pk2(C[1][0], C[1][1]);
+        st.C2 = pk2(C[2][0], C[2][1]);
     }
-    FwdSpan<TILE, BASELINE, COUNT> span{sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty, pxc, pyc, st};
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        st.x[h] = (st.live >> h) & 1 ? (float)(px + 4 * h) + 0.5f : __uint_as_float(0x7fc00000u);
+    sh.init_pad();
+    FwdSpan<TILE, COUNT, LAZY, R> span{sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty, st};
     // saving for the backward: the sorted chunks go back into the stream
     const int32_t end =
-        walk_tile<TILE, LAZY>(words, off, t, K, kbegin, kend, cap, ws, span, out_end ? words : nullptr);
+        walk_tile<TILE, LAZY, TB::NT>(words, off, t, K, kbegin, kend, cap, ws, span, out_end ? words : nullptr);
     if (out_end && threadIdx.x == 0) out_end[t] = end;
     if (out_wend) {
-        // per warp, the stream position past the entry that stopped its last
-        // pixel (the tile's end when one of its pixels never stopped): the
-        // backward has nothing to do for the warp at or beyond it
-        const int32_t wv = !inside ? INT32_MIN : (st.done ? st.stop + 1 : end);
-        const int32_t m = __reduce_max_sync(0xffffffffu, wv);
-        if ((threadIdx.x & 31) == 0)
-            out_wend[(int64_t)t * (TILE * TILE / 32) + (threadIdx.x >> 5)] = m == INT32_MIN ? 0 : min(m, end);
+        // per 8 x 4 block of pixels, the stream position past the entry that
+        // stopped its last pixel (the tile's end when one of its pixels never
+        // stopped): the backward has nothing to do for it at or beyond it.
+        // Lanes 0..15 hold the upper four rows of the warp's block.
+        int32_t m = !inside ? INT32_MIN : (st.live ? end : st.stop + 1);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        const int col = TB::x0() / 8, row = TB::y0() / 4 + (lane >> 4);
+        if ((lane & 15) == 0)
+            out_wend[(int64_t)t * (TILE * TILE / 32) + row * TB::COLS + col] = m == INT32_MIN ? 0 : min(m, end);
     }
-    // the pixel's index formed again after the walk: kept live across it,
-    // it cost the kernel a spill at its register budget (raster 0.274 ->
-    // 0.264 ms at 1080p)
-    const int64_t p = (int64_t)(ty * TILE + WarpBlocks<TILE>::ly()) * a.width + (tx * TILE + WarpBlocks<TILE>::lx());
     bool unfinished = false;
     if (pl.flag && kend < K) {
         // a planned first pass: a tile with a pixel still compositing when its
         // bins ran out, and entries in later bins, is left to the completing
         // pass with its pixels' state in the outputs
-        const bool all_done = __syncthreads_count(st.done) == TILE * TILE;
+        const bool all_done = __syncthreads_count(st.live == 0) == TB::NT;
         unfinished = !all_done && off[(int64_t)t * K + K] > off[(int64_t)t * K + kend];
         if (unfinished && threadIdx.x == 0) {
             pl.flag[t] = 1;
@@ -317,7 +459,7 @@ __device__ __forceinline__ void raster_tile(
         const int32_t s0 = off[(int64_t)t * K], s1 = off[(int64_t)t * K + K];
         if (threadIdx.x == 0) s_end = s0;
         __syncthreads();
-        if (inside) atomicMax(&s_end, st.done ? st.stop + 1 : s1);
+        if (inside) atomicMax(&s_end, st.live ? s1 : st.stop + 1);
         __syncthreads();
         if (threadIdx.x == 0) {
             int need = 0;
@@ -333,21 +475,55 @@ __device__ __forceinline__ void raster_tile(
             pl.needed[t] = need;
         }
     }
-    if (inside && unfinished) {
-        out_rgb[3 * p] = st.C0;
-        out_rgb[3 * p + 1] = st.C1;
-        out_rgb[3 * p + 2] = st.C2;
-        out_alpha[p] = st.done ? -st.T : st.T;
-        out_last[p] = st.last;
-    } else if (inside) {
-        // the image is not read again on the device: streaming stores
-        __stcs(out_rgb + 3 * p, fmaf(st.T, a.bg0, st.C0));
-        __stcs(out_rgb + 3 * p + 1, fmaf(st.T, a.bg1, st.C1));
-        __stcs(out_rgb + 3 * p + 2, fmaf(st.T, a.bg2, st.C2));
-        __stcs(out_alpha + p, 1.0f - st.T);
-        __stcs(out_last + p, st.last >= 0 ? st.last - a.gid_base : st.last);
-        if (out_T) out_T[p] = st.T;
-        if (COUNT && out_ntests) out_ntests[p] = st.ntests;
+    float T[2], C0[2], C1[2], C2[2];
+    upk2(st.T, T[0], T[1]);
+    upk2(st.C0, C0[0], C0[1]);
+    upk2(st.C1, C1[0], C1[1]);
+    upk2(st.C2, C2[0], C2[1]);
+    if (unfinished) {  // the transmittance signed by termination
+        T[0] = st.live & 1 ? T[0] : -T[0];
+        T[1] = st.live & 2 ? T[1] : -T[1];
+    }
+    // The lanes of two neighbouring rows exchange one pixel each, so that
+    // eight lanes hold eight neighbouring pixels of one row (96 bytes of rgb)
+    // in each of the two store rounds: a lane of an even row then holds its
+    // pixel x of that row and of the next, one of an odd row its pixel x + 4
+    // of the row before and of its own.
+    const bool odd = (lane & 4) != 0;
+    auto pair_rows = [&](auto& v) {
+        const auto mine = odd ? v[0] : v[1];
+        const auto other = __shfl_xor_sync(0xffffffffu, mine, 4);
+        if (odd) v[0] = other;
+        else v[1] = other;
+    };
+    pair_rows(T);
+    pair_rows(C0);
+    pair_rows(C1);
+    pair_rows(C2);
+    pair_rows(st.last);
+    if (COUNT) pair_rows(st.ntests);
+    const int ox = tx * TILE + TB::x0() + (lane & 3) + (odd ? 4 : 0);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int oy = ty * TILE + TB::y0() + ((lane >> 2) & ~1) + h;
+        if (ox >= a.width || oy >= a.height) continue;
+        const int64_t p = (int64_t)oy * a.width + ox;
+        if (unfinished) {
+            out_rgb[3 * p] = C0[h];
+            out_rgb[3 * p + 1] = C1[h];
+            out_rgb[3 * p + 2] = C2[h];
+            out_alpha[p] = T[h];
+            out_last[p] = st.last[h];
+        } else {
+            // the image is not read again on the device: streaming stores
+            __stcs(out_rgb + 3 * p, fmaf(T[h], a.bg0, C0[h]));
+            __stcs(out_rgb + 3 * p + 1, fmaf(T[h], a.bg1, C1[h]));
+            __stcs(out_rgb + 3 * p + 2, fmaf(T[h], a.bg2, C2[h]));
+            __stcs(out_alpha + p, 1.0f - T[h]);
+            __stcs(out_last + p, st.last[h] >= 0 ? st.last[h] - a.gid_base : st.last[h]);
+            if (out_T) out_T[p] = T[h];
+            if (COUNT && out_ntests) out_ntests[p] = st.ntests[h];
+        }
     }
     if (COUNT) {
         // block reduction of the op count, one atomic per block
@@ -360,9 +536,19 @@ __device__ __forceinline__ void raster_tile(
     }
 }
 
+// Threads of a tile's block and the blocks an SM holds: 16 x 16 tiles' seven
+// blocks of 128 threads fill the shared memory (31.8 KB each).
+template <int TILE>
+constexpr int raster_threads() { return TileBlocks<TILE, kBH>::NT; }
+template <int TILE>
+constexpr int raster_min_blocks() { return TILE == 16 ? 7 : TILE == 8 ? 16 : 2; }
+// ... and with rounds of four
+template <int TILE>
+constexpr int raster_wide_blocks() { return TILE == 16 ? 4 : TILE == 8 ? 16 : 1; }
 
-template <int TILE, bool BASELINE, bool COUNT, bool LAZY>
-__global__ void __launch_bounds__(TILE * TILE, TILE == 16 ? 5 : 1)
+template <int TILE, bool COUNT, bool LAZY, int R>
+__global__ void __launch_bounds__(raster_threads<TILE>(),
+                                  COUNT ? 1 : R == 4 ? raster_wide_blocks<TILE>() : raster_min_blocks<TILE>())
 k_raster(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o_z, const float4* __restrict__ rgbv,
          uint64_t* words, const int32_t* __restrict__ off, RasterArgs a, int cullmode,
          float* __restrict__ out_rgb, float* __restrict__ out_alpha, int32_t* __restrict__ out_last,
@@ -370,18 +556,17 @@ k_raster(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o_z, con
          int32_t* __restrict__ out_end, const PlanView pl, int cap, int32_t* __restrict__ out_wend)
 {
     grid_dependency_sync();
-    __shared__ RasterShared<TILE, BASELINE> sh;
-    __shared__ WalkShared<LAZY> ws;
-    raster_tile<TILE, BASELINE, COUNT, LAZY>(blockIdx.x, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode, out_rgb,
-                                             out_alpha, out_last, out_ntests, ops_total, out_T, out_end, pl, cap,
-                                             out_wend);
+    __shared__ RasterShared<TILE, kBH> sh;
+    __shared__ WalkShared<TILE, LAZY> ws;
+    raster_tile<TILE, COUNT, LAZY, R>(blockIdx.x, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode, out_rgb, out_alpha,
+                                   out_last, out_ntests, ops_total, out_T, out_end, pl, cap, out_wend);
 }
 
 // The completing pass of a planned frame: persistent blocks take the listed
 // tiles ({count, tiles...}) one at a time and composite each on from the bin
 // where its first pass stopped, from the pixel state that pass left.
 template <int TILE>
-__global__ void __launch_bounds__(TILE * TILE, TILE == 16 ? 5 : 1)
+__global__ void __launch_bounds__(raster_threads<TILE>(), raster_min_blocks<TILE>())
 k_raster_listed(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o_z, const float4* __restrict__ rgbv,
                 uint64_t* words, const int32_t* __restrict__ off, RasterArgs a, int cullmode,
                 float* __restrict__ out_rgb, float* __restrict__ out_alpha, int32_t* __restrict__ out_last,
@@ -389,15 +574,15 @@ k_raster_listed(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o
                 const int32_t* __restrict__ list, int cap)
 {
     grid_dependency_sync();
-    __shared__ RasterShared<TILE, false> sh;
-    __shared__ WalkShared<true> ws;
+    __shared__ RasterShared<TILE, kBH> sh;
+    __shared__ WalkShared<TILE, true> ws;
     PlanView pl;
     pl.bins = plan;
     pl.resume = 1;
     const int32_t nl = list[0];
     for (int32_t k = blockIdx.x; k < nl; k += gridDim.x) {
         const int t = list[1 + k];
-        raster_tile<TILE, false, false, true>(t, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode, out_rgb,
+        raster_tile<TILE, false, true, TILE == 8 ? 4 : 2>(t, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode, out_rgb,
                                               out_alpha, out_last, nullptr, nullptr, out_T, out_end, pl, cap);
         __syncthreads();  // the next tile reuses the shared memory
     }
@@ -465,12 +650,12 @@ __global__ void k_view_order(const __grid_constant__ ViewRasterSet vs, int32_t* 
 }
 
 template <int TILE, bool LAZY>
-__global__ void __launch_bounds__(TILE * TILE, TILE == 16 ? 5 : 1)
+__global__ void __launch_bounds__(raster_threads<TILE>(), raster_min_blocks<TILE>())
 k_raster_views(const __grid_constant__ ViewRasterSet vs, const int32_t* __restrict__ order,
                int32_t* __restrict__ counter)
 {
-    __shared__ RasterShared<TILE, false> sh;
-    __shared__ WalkShared<LAZY> ws;
+    __shared__ RasterShared<TILE, kBH> sh;
+    __shared__ WalkShared<TILE, LAZY> ws;
     __shared__ int32_t s_item;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -482,39 +667,37 @@ k_raster_views(const __grid_constant__ ViewRasterSet vs, const int32_t* __restri
         __syncthreads();
         if (item >= vs.total) break;
         const ViewRasterSet::View& V = vs.v[view_of(vs, item)];
-        raster_tile<TILE, false, false, LAZY>(item - V.item0, sh, ws, V.xy_ab, V.c_o_z, V.rgbv, V.words, V.off, V.a,
+        raster_tile<TILE, false, LAZY, 2>(item - V.item0, sh, ws, V.xy_ab, V.c_o_z, V.rgbv, V.words, V.off, V.a,
                                               V.cullmode, V.rgb, V.alpha, V.last, nullptr, nullptr, nullptr, nullptr,
                                               PlanView(), V.cap);
     }
 }
 
 template <int TILE>
-static cudaError_t launch_tile(const gs_ctx* ctx, bool baseline, bool count, bool lazy, unsigned grid,
-                               cudaStream_t st, const ProjView& pv, uint64_t* words, const int32_t* off,
-                               const RasterArgs& a, int cull, float* rgb, float* alpha, int32_t* last,
-                               int32_t* ntests, unsigned long long* ops, float* final_T, int32_t* tile_end,
-                               const PlanView& pl, int cap, int32_t* warp_end)
+static cudaError_t launch_tile(const gs_ctx* ctx, bool count, bool lazy, unsigned grid, cudaStream_t st,
+                               const ProjView& pv, uint64_t* words, const int32_t* off, const RasterArgs& a, int cull,
+                               float* rgb, float* alpha, int32_t* last, int32_t* ntests, unsigned long long* ops,
+                               float* final_T, int32_t* tile_end, const PlanView& pl, int cap, int32_t* warp_end)
 {
-    constexpr int BS = TILE * TILE;
-#define GS_RASTER_LAUNCH(B, CNT, LZ)                                                                          \
-    return launch_k(ctx, k_raster<TILE, B, CNT, LZ>, grid, BS, 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, off, a, \
-                    (B) ? 0 : cull, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end)
-    if (baseline) {
-        if (count) GS_RASTER_LAUNCH(true, true, false);
-        else GS_RASTER_LAUNCH(true, false, false);
-    } else if (lazy) {
-        if (count) GS_RASTER_LAUNCH(false, true, true);
-        else GS_RASTER_LAUNCH(false, false, true);
-    } else {
-        if (count) GS_RASTER_LAUNCH(false, true, false);
-        else GS_RASTER_LAUNCH(false, false, false);
-    }
-#undef GS_RASTER_LAUNCH
+    // Rounds of four when all the frame's tiles are resident at once (each
+    // SM's few warps wait for their own results, and a wide round has twice as
+    // many of them in flight): 256 tiles of 16 x 16, 20.4 us against 22.4;
+    // past that rounds of two, whose smaller register share holds seven blocks
+    // an SM instead of four (8160 tiles: 229 us against 244; 3600 tiles, global:
+    // 276 against 331).  8 x 8 tiles have one warp a block, as many blocks
+    // either way, and always go by four (2646 tiles: 63.4 us against 69.5).
+    const bool wide = TILE == 8 || grid <= (unsigned)(ctx->num_sms * raster_wide_blocks<TILE>());
+    constexpr int RN = TILE == 8 ? 4 : 2;
+    const auto kern = count  ? (lazy ? k_raster<TILE, true, true, RN> : k_raster<TILE, true, false, RN>)
+                      : wide ? (lazy ? k_raster<TILE, false, true, 4> : k_raster<TILE, false, false, 4>)
+                             : (lazy ? k_raster<TILE, false, true, RN> : k_raster<TILE, false, false, RN>);
+    return launch_k(ctx, kern, grid, raster_threads<TILE>(), 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, off, a, cull,
+                    rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end);
 }
 
 int raster_fwd(gs_ctx* ctx, const ProjView& pv, const gs_camera* cam, uint64_t* words,
                const int32_t* offsets, int32_t stride, const float* bg, float* rgb, float* alpha,
-               int32_t* last, int32_t* ntests, bool baseline, cudaStream_t st, float* final_T, int32_t* tile_end,
+               int32_t* last, int32_t* ntests, cudaStream_t st, float* final_T, int32_t* tile_end,
                const PlanView& pl, int32_t* warp_end)
 {
     const int tile = ctx->cfg.tile_size;
@@ -527,12 +710,14 @@ int raster_fwd(gs_ctx* ctx, const ProjView& pv, const gs_camera* cam, uint64_t* 
     a.bg0 = bg[0];
     a.bg1 = bg[1];
     a.bg2 = bg[2];
-    const int cull = ctx->cfg.tile_cull ? 1 : 0;
     const bool count = ntests != nullptr || pl.needed != nullptr;
-    const bool lazy = !baseline && ctx->cfg.mode == GS_MODE_BINNED_EXACT && ctx->cfg.repair_in_raster;
+    const bool lazy = ctx->cfg.mode == GS_MODE_BINNED_EXACT && ctx->cfg.repair_in_raster;
     // EXACT streams are culled when they are built: no second tile test at
-    // staging, only the per-warp strip mask
-    const int cull_here = !cull ? 0 : (ctx->cfg.mode == GS_MODE_BINNED_EXACT ? 2 : 3);
+    // staging, only the per-warp mask.  GLOBAL without the cull is the plain
+    // raster.
+    const bool exact = ctx->cfg.mode == GS_MODE_BINNED_EXACT;
+    const int cull_here = ctx->cfg.tile_cull ? (exact ? kCullWarp : kCullTile | kCullWarp)
+                                             : (ctx->cfg.mode == GS_MODE_GLOBAL_SORT ? kPlain : 0);
     const int cap = chunk_cap(ctx->cfg);
     const unsigned grid = (unsigned)a.n_tiles;
     if (grid == 0) return GS_OK;
@@ -540,9 +725,9 @@ int raster_fwd(gs_ctx* ctx, const ProjView& pv, const gs_camera* cam, uint64_t* 
     if (count) GS_CUDA_TRY(cudaMemsetAsync(ops, 0, sizeof(unsigned long long), st));
     cudaError_t e;
     switch (tile) {
-        case 8: e = launch_tile<8>(ctx, baseline, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end); break;
-        case 32: e = launch_tile<32>(ctx, baseline, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end); break;
-        default: e = launch_tile<16>(ctx, baseline, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end); break;
+        case 8: e = launch_tile<8>(ctx, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end); break;
+        case 32: e = launch_tile<32>(ctx, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end); break;
+        default: e = launch_tile<16>(ctx, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end); break;
     }
     GS_CUDA_TRY(e);
     ctx->launches += 1;
@@ -566,12 +751,12 @@ int raster_listed(gs_ctx* ctx, const ProjView& pv, const gs_camera* cam, uint64_
     a.bg2 = bg[2];
     if (a.n_tiles == 0) return GS_OK;
     // EXACT streams are culled when built: the strip mask only
-    const int cull = ctx->cfg.tile_cull ? 2 : 0;
+    const int cull = ctx->cfg.tile_cull ? kCullWarp : 0;
     const int cap = chunk_cap(ctx->cfg);
     switch (tile) {
-        case 8: GS_CUDA_TRY(launch_k(ctx, k_raster_listed<8>, (unsigned)ctx->num_sms, 64, 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, offsets, a, cull, rgb, alpha, last, final_T, tile_end, plan, list, cap)); break;
-        case 32: GS_CUDA_TRY(launch_k(ctx, k_raster_listed<32>, (unsigned)ctx->num_sms, 1024, 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, offsets, a, cull, rgb, alpha, last, final_T, tile_end, plan, list, cap)); break;
-        default: GS_CUDA_TRY(launch_k(ctx, k_raster_listed<16>, (unsigned)ctx->num_sms * 5, 256, 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, offsets, a, cull, rgb, alpha, last, final_T, tile_end, plan, list, cap)); break;
+        case 8: GS_CUDA_TRY(launch_k(ctx, k_raster_listed<8>, (unsigned)ctx->num_sms * 8, raster_threads<8>(), 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, offsets, a, cull, rgb, alpha, last, final_T, tile_end, plan, list, cap)); break;
+        case 32: GS_CUDA_TRY(launch_k(ctx, k_raster_listed<32>, (unsigned)ctx->num_sms, raster_threads<32>(), 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, offsets, a, cull, rgb, alpha, last, final_T, tile_end, plan, list, cap)); break;
+        default: GS_CUDA_TRY(launch_k(ctx, k_raster_listed<16>, (unsigned)ctx->num_sms * raster_min_blocks<16>(), raster_threads<16>(), 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, offsets, a, cull, rgb, alpha, last, final_T, tile_end, plan, list, cap)); break;
     }
     ctx->launches += 1;
     GS_CUDA_TRY(cudaGetLastError());
@@ -601,7 +786,7 @@ int raster_views(gs_ctx* ctx, const RasterView* views, int nv, int32_t* sched, i
         V.a.bg0 = r.bg[0];
         V.a.bg1 = r.bg[1];
         V.a.bg2 = r.bg[2];
-        V.cullmode = r.cull ? 2 : 0;
+        V.cullmode = r.cull ? kCullWarp : 0;
         V.cap = r.cap;
         V.rgb = r.rgb;
         V.alpha = r.alpha;
@@ -619,8 +804,9 @@ int raster_views(gs_ctx* ctx, const RasterView* views, int nv, int32_t* sched, i
     k_view_buckets<<<gi, 256, 0, st>>>(vs, sched);
     k_view_bucket_starts<<<1, 32, 0, st>>>(sched);
     k_view_order<<<gi, 256, 0, st>>>(vs, sched, order);
-    const unsigned grid = (unsigned)(ctx->num_sms * 5 < total ? ctx->num_sms * 5 : total);
-    k_raster_views<16, true><<<grid, 256, 0, st>>>(vs, order, sched + 64);
+    const int resident = ctx->num_sms * raster_min_blocks<16>();
+    const unsigned grid = (unsigned)(resident < total ? resident : total);
+    k_raster_views<16, true><<<grid, raster_threads<16>(), 0, st>>>(vs, order, sched + 64);
     ctx->launches += 4;
     GS_CUDA_TRY(cudaGetLastError());
     return GS_OK;

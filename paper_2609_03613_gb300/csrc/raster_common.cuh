@@ -3,7 +3,7 @@
 // memory (with the conservative tile-alpha cull and the per-warp strip mask)
 // and the walk over a tile's span -- either the whole span at once, or, for
 // EXACT streams whose repair runs in the raster, chunk by chunk with each
-// segment of 2..kRasterSortCap entries sorted in shared memory by (depth bits,
+// segment of 2..raster_sort_cap(TILE) entries sorted in shared memory by (depth bits,
 // gid) right before it is composited (Sec. 3.5 selective repair; supplement,
 // binned raster traversal after repair).  A forward that saves its state for
 // the backward stores the sorted chunks back, so the backward walks the same
@@ -19,23 +19,45 @@ struct RasterArgs {
     int32_t gid_base = 0;  // stream words hold gid_base + gid (the last-id output subtracts it)
 };
 
-template <int TILE, bool BASELINE>
+// A warp owns a block of 8 x BH pixels of the tile (BH = 4: a pixel a lane;
+// BH = 8: two).  Blocks are laid out TILE/8 wide and TILE/BH tall, warps
+// row-major over them; the block of the tile has one warp for each.
+template <int TILE, int BH>
+struct TileBlocks {
+    static constexpr int COLS = TILE / 8, ROWS = TILE / BH;
+    static constexpr int NW = COLS * ROWS;    // warps of the tile
+    static constexpr int NT = 32 * NW;        // threads of the tile
+    __device__ static int x0() { return ((threadIdx.x >> 5) % COLS) * 8; }
+    __device__ static int y0() { return ((threadIdx.x >> 5) / COLS) * BH; }
+};
+
+// Entries staged per batch.
+template <int TILE>
+constexpr int raster_batch() { return TILE == 8 ? 128 : 256; }
+
+template <int TILE, int BH>
 struct RasterShared {
-    static constexpr int BS = TILE * TILE;
-    static constexpr int BATCH = BS < 256 ? BS : 256;  // entries staged per batch
-    static constexpr int NW = BATCH / 32;              // warps that load a batch
-    static constexpr int NWT = BS / 32;                // warps of the tile
-    float4 a[BATCH];                       // {mx, my, a/2, b}
-    float4 b[BATCH];                       // {c/2, o, tau, gid bits}
-    float4 c[BASELINE ? 1 : BATCH];        // colour (binned)
-    uint32_t g[BASELINE ? BATCH : 1];      // gid (baseline colour lookup)
-    uint8_t list[BASELINE ? 1 : NWT][BASELINE ? 1 : BATCH];  // per warp: staged entries its warp mask admits
+    using TB = TileBlocks<TILE, BH>;
+    static constexpr int BATCH = raster_batch<TILE>();
+    float4 a[BATCH + 1];  // {mx, my, a/2, b}; the last slot of each array is a
+    float4 b[BATCH + 1];  // {c/2, o, tau, gid bits}        zero record, which no
+    float4 c[BATCH + 1];  // colour, warp mask              pixel ever passes
+    // per warp: the slots its mask admits, as byte offsets into a, b, c; read
+    // two at a time
+    alignas(8) uint16_t list[TB::NW][BATCH + 4];
+
+    // The zero record (before the first block barrier of the kernel).
+    __device__ __forceinline__ void init_pad()
+    {
+        if (threadIdx.x == 0) a[BATCH] = b[BATCH] = c[BATCH] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 };
 
 // The staged entries (of cnt) whose warp mask admits the calling warp, in
-// stage order, into sh.list[warp]; returns their count.  Whole warp.
-template <int TILE>
-__device__ __forceinline__ int warp_strip_list(RasterShared<TILE, false>& sh, int cnt)
+// stage order, into sh.list[warp], followed by three references to the zero
+// record (a whole round of two or four); returns their count.  Whole warp.
+template <int TILE, int BH>
+__device__ __forceinline__ int warp_strip_list(RasterShared<TILE, BH>& sh, int cnt)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int nw = 0;
@@ -43,40 +65,30 @@ __device__ __forceinline__ int warp_strip_list(RasterShared<TILE, false>& sh, in
         const int j = j0 + lane;
         const bool mine = j < cnt && ((__float_as_uint(sh.c[j].w) >> warp) & 1u);
         const unsigned bal = __ballot_sync(0xffffffffu, mine);
-        if (mine) sh.list[warp][nw + __popc(bal & ((1u << lane) - 1u))] = (uint8_t)j;
+        if (mine) sh.list[warp][nw + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(16 * j);
         nw += __popc(bal);
     }
+    if (lane < 3) sh.list[warp][nw + lane] = (uint16_t)(16 * RasterShared<TILE, BH>::BATCH);
     __syncwarp();
     return nw;
 }
 
-// A warp owns an 8 x 4 pixel block of the tile: blocks are laid out TILE/8
-// wide and TILE/4 tall (16x16: 2 x 4 blocks for the 8 warps; 8x8: 1 x 2;
-// 32x32: 4 x 8), lanes row-major inside the block.
-template <int TILE>
-struct WarpBlocks {
-    static constexpr int COLS = TILE / 8, ROWS = TILE / 4;
-    static_assert(COLS * ROWS == TILE * TILE / 32, "one 8x4 block per warp");
-    __device__ static int lx() { return ((threadIdx.x >> 5) % COLS) * 8 + (threadIdx.x & 7); }
-    __device__ static int ly() { return ((threadIdx.x >> 5) / COLS) * 4 + ((threadIdx.x & 31) >> 3); }
-};
-
 // Warp mask of an entry: bit w is set when the entry's alpha >= 1/255
 // ellipse (the tile cull's bound Q(d) <= tau / margin, d = mean - pixel
-// centre, widened as there) reaches a pixel centre of warp w's 8 x 4 block of
-// the tile (origin x0, y0).  Per band of four pixel rows the ellipse's
+// centre, widened as there) reaches a pixel centre of warp w's 8 x BH block of
+// the tile (origin x0, y0).  Per band of BH pixel rows the ellipse's
 // x-extent over the band's centre rows (the row-span geometry of the bin
 // stage: band ends and the ellipse's leftmost / rightmost points) is widened
 // by 5e-3 relative + 0.05 px and tested against each block's centre columns,
 // so a warp never skips a pixel the entry can reach.  The geometry takes the
 // hardware's approximate division and square root (relative errors near
 // 2^-22, far inside the widening).
-template <int TILE>
+template <int TILE, int BH>
 __device__ __forceinline__ uint32_t strip_mask(float mx, float my, float ha, float hb, float hc, float tau,
                                                float margin, float x0, float y0)
 {
-    using WB = WarpBlocks<TILE>;
-    constexpr int NWT = TILE * TILE / 32;
+    using WB = TileBlocks<TILE, BH>;
+    constexpr int NWT = WB::NW;
     const uint32_t all = NWT >= 32 ? 0xffffffffu : ((1u << NWT) - 1u);
     if (!(margin > 0.0f)) return all;
     const float D = 4.0f * ha * hc - hb * hb;
@@ -93,7 +105,7 @@ __device__ __forceinline__ uint32_t strip_mask(float mx, float my, float ha, flo
     uint32_t m = 0u;
 #pragma unroll
     for (int by = 0; by < WB::ROWS; ++by) {
-        float yl = my - (y0 + (float)(4 * by) + 3.5f), yh = my - (y0 + (float)(4 * by) + 0.5f);
+        float yl = my - (y0 + (float)(BH * by) + ((float)BH - 0.5f)), yh = my - (y0 + (float)(BH * by) + 0.5f);
         yl = yl - (0.05f + 5e-3f * fabsf(yl));
         yh = yh + (0.05f + 5e-3f * fabsf(yh));
         const float ya = fmaxf(yl, -dymax), yb = fminf(yh, dymax);
@@ -116,84 +128,79 @@ __device__ __forceinline__ uint32_t strip_mask(float mx, float my, float ha, flo
     return m & all;
 }
 
-// The staged record of binned entry g from its projected fields p = xy_ab[g],
+// How a stream's entries are staged (bits of cullmode).
+constexpr int kCullTile = 1;   // the tile-alpha cull
+constexpr int kCullWarp = 2;   // per-warp masks
+constexpr int kPlain = 4;      // neither: the plain raster
+
+// The staged record of entry g from its projected fields p = xy_ab[g],
 // q = c_o_z[g] and colour c = rgbv[g]: {mx, my, a/2, b}, {c/2, o, tau, gid
 // bits} and the colour with the warp mask in .w (zero when the tile cull
 // drops the entry: no warp's list admits it).
-template <int TILE>
+template <int TILE, int BH>
 __device__ __forceinline__ void stage_record(uint32_t g, const float4& p, const float4& q, float4 c, int cullmode,
                                              int tx, int ty, float4& A, float4& B, float4& C)
 {
     A = make_float4(p.x, p.y, 0.5f * p.z, p.w);
-    B = make_float4(0.5f * q.x, q.y, q.w, __uint_as_float(g));
+    // the plain raster takes nothing from the record's cull fields: its
+    // early-out bound comes from the opacity itself, within the exp's range
+    const float tau = (cullmode & kPlain) ? fminf(fmaxf(logf(255.0f * q.y) + 2e-4f, 0.0f), 87.0f) : q.w;
+    B = make_float4(0.5f * q.x, q.y, tau, __uint_as_float(g));
     bool keep = true;
-    if (cullmode & 1)
+    if (cullmode & kCullTile)
         keep = !tile_culled(A.x, A.y, A.z, A.w, B.x, q.w, c.w, (float)(tx * TILE), (float)(ty * TILE), (float)TILE);
-    const uint32_t m = (cullmode & 2)
-                           ? strip_mask<TILE>(A.x, A.y, A.z, A.w, B.x, q.w, c.w, (float)(tx * TILE), (float)(ty * TILE))
-                           : 0xffffffffu;
+    const uint32_t m = (cullmode & kCullWarp) ? strip_mask<TILE, BH>(A.x, A.y, A.z, A.w, B.x, q.w, c.w,
+                                                                     (float)(tx * TILE), (float)(ty * TILE))
+                                              : 0xffffffffu;
     c.w = __uint_as_float(keep ? m : 0u);
     C = c;
 }
 
 // Stage the batch [b0, b0 + BATCH) of n_entries stream words from src (global
-// or shared memory): per entry {mx, my, a/2, b}, {c/2, o, tau, gid bits} and,
-// binned, the colour with the strip mask in .w (zero for an entry the tile
-// cull drops).  Returns the number staged (block-uniform); the caller
+// or shared memory): per entry {mx, my, a/2, b}, {c/2, o, tau, gid bits} and
+// the colour with the warp mask in .w (zero for an entry the tile cull
+// drops).  Returns the number staged (block-uniform); the caller
 // synchronises the block before reading sh.
-template <int TILE, bool BASELINE>
+template <int TILE, int BH>
 __device__ __forceinline__ int stage_batch(const uint64_t* src, int32_t b0, int32_t n_entries,
-                                           RasterShared<TILE, BASELINE>& sh, const float4* __restrict__ xy_ab,
+                                           RasterShared<TILE, BH>& sh, const float4* __restrict__ xy_ab,
                                            const float4* __restrict__ c_o_z, const float4* __restrict__ rgbv,
                                            int cullmode, int tx, int ty)
 {
-    using SH = RasterShared<TILE, BASELINE>;
-    constexpr int BATCH = SH::BATCH;
-    const int32_t idx = b0 + threadIdx.x;
-    const bool valid = threadIdx.x < BATCH && idx < n_entries;
-    float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A, Cc = A;
-    uint32_t g = 0;
-    if (valid) {
-        g = (uint32_t)(src[idx] & 0xffffffffull);
-        const float4 p = __ldg(xy_ab + g);
-        const float4 q = __ldg(c_o_z + g);
-        if constexpr (BASELINE) {
-            A = make_float4(p.x, p.y, 0.5f * p.z, p.w);
-            B = make_float4(0.5f * q.x, q.y, q.w, __uint_as_float(g));
-        } else {
-            stage_record<TILE>(g, p, q, __ldg(rgbv + g), cullmode, tx, ty, A, B, Cc);
-        }
-    }
-    // entry i of the batch goes to slot i: the tile cull and the strip mask
+    using SH = RasterShared<TILE, BH>;
+    const int cnt = min(SH::BATCH, n_entries - b0);
+    // entry i of the batch goes to slot i: the tile cull and the warp mask
     // leave a zero mask, which no warp's list admits (stream order is kept
     // without a compaction pass)
-    const int cnt = min(BATCH, n_entries - b0);
-    const int pos = threadIdx.x;
-    if (valid) {
-        sh.a[pos] = A;
-        sh.b[pos] = B;
-        if (BASELINE) sh.g[pos] = g;
-        else sh.c[pos] = Cc;
+    auto put = [&](int i) {
+        const uint32_t g = (uint32_t)(src[b0 + i] & 0xffffffffull);
+        float4 A, B, C;
+        stage_record<TILE, BH>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
+        sh.a[i] = A;
+        sh.b[i] = B;
+        sh.c[i] = C;
+    };
+    if constexpr (SH::TB::NT >= SH::BATCH) {
+        if ((int)threadIdx.x < cnt) put(threadIdx.x);
+    } else {
+        for (int i = threadIdx.x; i < cnt; i += SH::TB::NT) put(i);
     }
     return cnt;
 }
 
 // Shared memory of the tile walk.
-template <bool LAZY>
+template <int TILE, bool LAZY>
 struct WalkShared {
-    uint64_t sort[LAZY ? kRasterSortCap : 1];
+    uint64_t sort[LAZY ? raster_sort_cap(TILE) : 1];
     int32_t off[LAZY ? GS_MAX_K + 1 : 1];
-    int big[LAZY ? GS_MAX_K : 1];  // segments sorted by the whole block
-    int nsort;
 };
 
 // The sorted position of word `key`, entry i of the chunk held in ws.sort
 // (bins bfirst..e-1 from stream position c0): the start of its segment plus
 // the number of smaller words in the segment (the words are distinct, their
 // low half being the gid).
-template <bool LAZY>
-__device__ __forceinline__ int chunk_rank(const WalkShared<LAZY>& ws, int i, uint64_t key, int32_t c0, int bfirst,
-                                          int e)
+template <class WS>
+__device__ __forceinline__ int chunk_rank(const WS& ws, int i, uint64_t key, int32_t c0, int bfirst, int e)
 {
     int lo = bfirst, hi = e - 1;  // the last bin starting at or before i
     while (lo < hi) {
@@ -207,157 +214,127 @@ __device__ __forceinline__ int chunk_rank(const WalkShared<LAZY>& ws, int i, uin
     return r;
 }
 
-// Load the chunk [c0, c0 + len) (bins bfirst..e-1) into ws.sort and sort each
-// of its segments by (depth bits, gid).  A chunk of at most one entry per
-// thread is sorted by rank: each thread counts the smaller words of its own
-// segment (the words are distinct, their low half being the gid), so one
-// pass of comparisons and one scatter place every word.  Longer chunks: each
-// segment of up to 64 entries in registers by one warp, up to 256 in shared
-// memory by one warp, longer ones by the whole block (ws.big[base..] collects
-// the long ones).
-template <int TILE, bool LAZY>
-__device__ __forceinline__ void load_sort_chunk(const uint64_t* words, int32_t c0, int32_t len,
-                                                int bfirst, int e, WalkShared<LAZY>& ws, int base = 0)
-{
-    constexpr int BS = TILE * TILE;
-    constexpr int NWB = BS / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (len <= BS) {
-        // one entry a thread: its rank in its segment is the segment start
-        // plus the number of smaller words there (words are unique: gid)
-        const int i = threadIdx.x;
-        uint64_t key = 0;
-        if (i < len) key = __ldcs(reinterpret_cast<const unsigned long long*>(words) + c0 + i);
-        if (i < len) ws.sort[i] = key;
-        __syncthreads();
-        const int r = i < len ? chunk_rank(ws, i, key, c0, bfirst, e) : 0;
-        __syncthreads();
-        if (i < len) ws.sort[r] = key;
-        __syncthreads();
-        return;
-    }
-    // the stream is read once: streamed past L2 (evict first)
-    for (int i = threadIdx.x; i < len; i += BS)
-        ws.sort[i] = __ldcs(reinterpret_cast<const unsigned long long*>(words) + c0 + i);
-    if (threadIdx.x == 0) ws.nsort = 0;
-    __syncthreads();
-    for (int j = bfirst + warp; j < e; j += NWB) {
-        const int l = ws.off[j + 1] - ws.off[j];
-        uint64_t* seg = ws.sort + (ws.off[j] - c0);
-        if (l < 2) continue;
-        if (l <= 32) {
-            uint64_t v = lane < l ? seg[lane] : ~0ull;
-            v = warp_bitonic32(v);
-            if (lane < l) seg[lane] = v;
-        } else if (l <= 64) {
-            warp_bitonic64(seg, l);
-        } else if (l <= 256) {
-            bitonic_mem(seg, l, lane, 32, SyncWarp{});
-        } else if (lane == 0) {
-            ws.big[atomicAdd(&ws.nsort, 1)] = j;
-        }
-    }
-    __syncthreads();
-    const int nbig = ws.nsort;
-    for (int k = 0; k < nbig; ++k) {
-        const int j = ws.big[k];
-        bitonic_mem(ws.sort + (ws.off[j] - c0), ws.off[j + 1] - ws.off[j], threadIdx.x, BS, SyncBlock{});
-    }
-}
-
-// Walk tile t's span of the stream front to back, handing runs of entries to
-// span(src, n, checked, base) (src[0] is stream position base; returns -1
-// after consuming all n, or, block-uniformly, the offset within the run at
-// which every pixel of the tile had terminated; span.done() is the calling
-// thread's termination flag; a Span with kStageAtRank also takes a chunk of
-// at most kBatch entries staged slot by slot, span.stage_at(slot, gid), and
-// composites it with span.composite_staged(n, base)).  Only bins [kbegin, kend) of the tile's K are
-// walked (a planned frame's passes; 0, K: the whole span).
+// Walk tile t's span of the stream front to back by NT threads, handing runs
+// of entries to span(src, n, checked, base) (src[0] is stream position base;
+// returns -1 after consuming all n, or, block-uniformly, the offset within the
+// run at which every pixel of the tile had terminated; span.done() is true
+// when the calling thread's pixels have terminated; span.stage_at(slot, gid)
+// stages one entry of a run of at most kBatch, which span.composite_staged(n,
+// base) then composites).  Only bins [kbegin, kend) of the tile's K are walked
+// (a planned frame's passes; 0, K: the whole span).
 // Not LAZY: one run, [off[t*K], off[t*K + kend]).  LAZY: chunks of
-// consecutive segments of at most `cap` entries (a single segment of up to
-// kRasterSortCap entries forms a chunk of its own) are loaded into shared
-// memory and every segment of the chunk is sorted; a segment longer than
-// kRasterSortCap was sorted before the raster and is handed over in place.
-// The chunks are the tile's repair bins.  ws.off holds all K + 1 bin offsets
-// of the tile on return (LAZY).
+// consecutive segments of at most `cap` entries (and at most one batch), whose
+// words are loaded into shared memory, ranked within their segments and
+// staged straight at their sorted slots; a single longer segment of up to
+// raster_sort_cap(TILE) entries is sorted there by the block and handed over
+// as a run, one beyond that was sorted before the raster and is handed over
+// in place.  The chunks are the tile's repair bins.  ws.off holds all K + 1
+// bin offsets of the tile on return (LAZY).
 // Returns the stream index at which the walk ended: the end of the walked
 // bins, or the position (in the composited order) where every pixel had
 // terminated.  With writeback (the stream itself), every sorted chunk is also
 // stored back in place, so the tile's composited prefix is left in (depth,
 // gid) order.
-template <int TILE, bool LAZY, class Span>
+template <int TILE, bool LAZY, int NT, class Span>
 __device__ __forceinline__ int32_t walk_tile(const uint64_t* words, const int32_t* __restrict__ off, int t, int K,
-                                             int kbegin, int kend, int cap, WalkShared<LAZY>& ws, Span& span,
+                                             int kbegin, int kend, int cap, WalkShared<TILE, LAZY>& ws, Span& span,
                                              uint64_t* writeback = nullptr)
 {
-    constexpr int BS = TILE * TILE;
-    if (!LAZY) {
+    if constexpr (!LAZY) {
         const int32_t s0 = off[(int64_t)t * K + kbegin], s1 = off[(int64_t)t * K + kend];
         const int32_t r = span(words + s0, s1 - s0, false, s0);
         return r < 0 ? s1 : s0 + r;
-    }
-    for (int b = threadIdx.x; b <= K; b += BS) ws.off[b] = off[(int64_t)t * K + b];
-    __syncthreads();
-    int b = kbegin;
-    while (b < kend) {
-        const int32_t c0 = ws.off[b];
-        if (ws.off[b + 1] - c0 > kRasterSortCap) {  // sorted before the raster
-            const int32_t r = span(words + c0, ws.off[b + 1] - c0, false, c0);
-            if (r >= 0) return c0 + r;
-            ++b;
-            continue;
-        }
-        // the chunk ends before the first bin j > b whose end passes c0 + cap
-        // (bin ends are nondecreasing, so the bins that fit are a prefix):
-        // counted 32 bins a ballot by every warp, in place of a serial walk
-        int e = b + 1;
-        {
-            const int lane = threadIdx.x & 31;
-            for (int j0 = b + 1; j0 < kend; j0 += 32) {
-                const int j = j0 + lane;
-                const int fit = __popc(__ballot_sync(0xffffffffu, j < kend && ws.off[j + 1] - c0 <= cap));
-                e += fit;
-                if (fit < 32) break;
+    } else {
+        const unsigned long long* wl = reinterpret_cast<const unsigned long long*>(words);
+        cap = min(cap, Span::kBatch);
+        for (int b = threadIdx.x; b <= K; b += NT) ws.off[b] = off[(int64_t)t * K + b];
+        __syncthreads();
+        constexpr int PER = (Span::kBatch + NT - 1) / NT;
+        // the chunk that starts with bin b: it ends before the first bin j > b
+        // whose end passes the start + cap (bin ends are nondecreasing, so the
+        // bins that fit are a prefix): counted 32 bins a ballot by every warp,
+        // in place of a serial walk.  Bins without entries are passed over.
+        // Its words, when they fit a batch, are loaded at once (the stream is
+        // read once: streamed past L2): the next chunk's while this one is
+        // staged and composited.
+        int b = kbegin, e;
+        int32_t c0, len;
+        uint64_t key[PER];
+        auto find = [&]() {
+            len = 0;
+            while (b < kend && len == 0) {
+                c0 = ws.off[b];
+                e = b + 1;
+                if (ws.off[b + 1] - c0 <= cap) {
+                    const int lane = threadIdx.x & 31;
+                    for (int j0 = b + 1; j0 < kend; j0 += 32) {
+                        const int j = j0 + lane;
+                        const int fit = __popc(__ballot_sync(0xffffffffu, j < kend && ws.off[j + 1] - c0 <= cap));
+                        e += fit;
+                        if (fit < 32) break;
+                    }
+                }
+                len = ws.off[e] - c0;
+                if (len == 0) b = e;
             }
-        }
-        const int32_t len = ws.off[e] - c0;
-        const int bfirst = b;
-        b = e;
-        if (len == 0) continue;
-        if (__syncthreads_count(span.done()) == BS) return c0;
-        if constexpr (Span::kStageAtRank) {
             if (len <= Span::kBatch) {
-                // a chunk of one batch: each thread loads one word, finds
-                // its rank in its segment and stages its entry straight at
-                // that slot -- no sorted copy of the chunk, two block
-                // barriers and a shared-memory round fewer than sorting
-                // first and staging after (raster 0.264 -> 0.259 ms at
-                // 1080p; gathering the entry's fields before the rank count
-                // instead held them across it and spilled: 0.291 ms)
-                const int i = threadIdx.x;
-                uint64_t key = 0;
-                if (i < len) {
-                    key = __ldcs(reinterpret_cast<const unsigned long long*>(words) + c0 + i);
-                    ws.sort[i] = key;
+#pragma unroll
+                for (int u = 0; u < PER; ++u) {
+                    const int i = threadIdx.x + u * NT;
+                    if (i < len) key[u] = __ldcs(wl + c0 + i);
+                }
+            }
+        };
+        find();
+        while (len > 0) {
+            const int32_t at = c0, n = len;
+            const int bfirst = b, bend = e;
+            b = e;
+            if (__syncthreads_count(span.done()) == NT) return at;
+            if (n <= Span::kBatch) {
+                // each thread finds its words' ranks in their segments and
+                // stages each entry straight at its sorted slot: no sorted
+                // copy of the chunk (raster 0.264 -> 0.259 ms at 1080p;
+                // gathering the entry's fields before the rank count instead
+                // held them across it and spilled: 0.291 ms)
+                uint64_t mine[PER];
+#pragma unroll
+                for (int u = 0; u < PER; ++u) {
+                    const int i = threadIdx.x + u * NT;
+                    mine[u] = key[u];
+                    if (i < n) ws.sort[i] = mine[u];
                 }
                 __syncthreads();
-                if (i < len) {
-                    const int r = chunk_rank(ws, i, key, c0, bfirst, e);
-                    if (writeback) writeback[c0 + r] = key;
-                    span.stage_at(r, (uint32_t)key);
+                find();
+#pragma unroll
+                for (int u = 0; u < PER; ++u) {
+                    const int i = threadIdx.x + u * NT;
+                    if (i < n) {
+                        const int r = chunk_rank(ws, i, mine[u], at, bfirst, bend);
+                        if (writeback) writeback[at + r] = mine[u];
+                        span.stage_at(r, (uint32_t)mine[u]);
+                    }
                 }
                 __syncthreads();
-                span.composite_staged(len, c0);  // termination just counted above
+                span.composite_staged(n, at);  // termination just counted above
                 continue;
             }
+            // one long segment: sorted in shared memory by the block, or before
+            // the raster
+            const bool sorted = n > raster_sort_cap(TILE);
+            if (!sorted) {
+                for (int i = threadIdx.x; i < n; i += NT) ws.sort[i] = __ldcs(wl + at + i);
+                __syncthreads();
+                bitonic_mem(ws.sort, n, threadIdx.x, NT, SyncBlock{});
+                if (writeback)
+                    for (int i = threadIdx.x; i < n; i += NT) writeback[at + i] = ws.sort[i];
+            }
+            const int32_t r = span(sorted ? words + at : ws.sort, n, true, at);  // termination just counted above
+            if (r >= 0) return at + r;
+            find();
         }
-        load_sort_chunk<TILE>(words, c0, len, bfirst, e, ws);  // ends with a block barrier
-        if (writeback)
-            for (int i = threadIdx.x; i < len; i += BS) writeback[c0 + i] = ws.sort[i];
-        const int32_t r = span(ws.sort, len, true, c0);  // termination just counted above
-        if (r >= 0) return c0 + r;
+        return ws.off[kend];
     }
-    return ws.off[kend];
 }
 
 // The walk of walk_tile in reverse over the entries before stream index

@@ -1,0 +1,55 @@
+"""The forward raster where its work split can go wrong: images one pixel past
+and one short of a warp's 8 x 8 block and of its two pixels a lane (x and
+x + 4), frames on both sides of the rule that picks the round width (tiles
+resident at once or not), and segments on both sides of a staging batch and of
+the in-raster sort's buffer, against the oracle bit for bit."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2609_03613_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2609_03613_gb300 import tilegs as G  # noqa: E402
+
+
+def assert_image(mode, sc, cam, tile, K, ref, **cfg):
+    ctx = G.Context(mode, tile_size=tile, K=K, **cfg)
+    rgb, alpha, last = (t.cpu().numpy() for t in ctx.render(G.DeviceScene.from_numpy(sc), cam, (0.1, 0.2, 0.3)))
+    assert ctx.error() == 0
+    np.testing.assert_array_equal(rgb.view(np.uint32), ref[0].view(np.uint32))
+    np.testing.assert_array_equal(alpha.view(np.uint32), ref[1].view(np.uint32))
+    np.testing.assert_array_equal(last, ref[2])
+
+
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("w,h", [(1, 1), (4, 7), (5, 8), (9, 17), (36, 33), (512, 304), (513, 304)])
+def test_ragged_sizes_and_round_widths(w, h, tile):
+    sc = scenes.mixture_scene(3000, 91)
+    cam = scenes.hd_camera(width=w, height=h, f=max(w, h) * 0.6)
+    ref = O.render(sc, cam, tile, bg=(0.1, 0.2, 0.3))[3]
+    for mode in ("exact", "global"):
+        assert_image(mode, sc, cam, tile, 64 if mode == "exact" else 1, ref)
+
+
+@pytest.mark.parametrize("tile", [8, 16])
+@pytest.mark.parametrize("count", [127, 128, 129, 255, 256, 257, 511, 512, 513, 2047, 2048, 2049])
+def test_segments_at_batch_and_sort_limits(count, tile):
+    # one bin a tile holding `count` entries (all inside one tile, none
+    # terminating it): staged at rank, sorted by the block, or sorted before
+    # the raster
+    rng = np.random.default_rng(count)
+    cam = scenes.tiny_camera()
+    z = rng.uniform(-0.4, 0.4, count)
+    xy = (132.0 + rng.uniform(-1.0, 1.0, (count, 2)) - cam.cx) * (3.0 - z)[:, None] / cam.fx
+    sc = scenes.Scene(np.column_stack([xy, z]).astype(np.float32), np.full((count, 3), 0.002, np.float32),
+                      np.tile(np.array([1, 0, 0, 0], np.float32), (count, 1)),
+                      np.full(count, 0.0045, np.float32), rng.uniform(0, 1, (count, 1, 3)).astype(np.float32), 0)
+    P, ent, (off, stream), ref = O.render(sc, cam, tile, bg=(0.1, 0.2, 0.3))
+    assert np.diff(off).max() == count
+    assert_image("exact", sc, cam, tile, 1, ref)
