@@ -10,7 +10,7 @@
 //   counts and row counts of every item, one scan     (as a single frame)
 //   per-view entry counts, samples and depth range    (Alg. 2, a block a view)
 //   row spans, per-row difference counts per view     (Alg. 3's histogram)
-//   per-view layer prefixes, transposition, one scan  (bin offsets)
+//   one pass over every view's tile rows              (bin offsets)
 //   the scatter of every view's row records           (one cursor per segment)
 //   the eager sort of segments over 2048 entries
 // and the persistent multi-view raster composites every view's tiles from
@@ -20,6 +20,7 @@
 #include <string.h>
 
 #include "depth_range.cuh"
+#include "offsets.cuh"
 #include "rows.cuh"
 #include "scan.cuh"
 
@@ -225,68 +226,69 @@ k_group_transpose(const int32_t* __restrict__ D, const GroupViews gv, int32_t* _
     }
 }
 
+// The group's tile rows (offsets.cuh): view by view.
+struct GroupRows {
+    const int32_t* D;
+    GroupViews gv;
+    __device__ __forceinline__ OffsetRow operator()(int row) const
+    {
+        int v = 0;
+        while (v + 1 < gv.nv && gv.row_base[v + 1] <= row) ++v;
+        const int y = row - gv.row_base[v], tx = gv.tiles_x[v], K = gv.K[v];
+        return OffsetRow{D + gv.d_base[v] + (int64_t)y * (tx + 1), (int64_t)gv.tiles_y[v] * (tx + 1), tx, K,
+                         gv.seg_base[v] + (int64_t)y * tx * K, gv.seg_base[v] + (int64_t)y * tx,
+                         (int64_t)tx * gv.tiles_y[v]};
+    }
+};
+
+int group_offsets_prepare()
+{
+    GS_CUDA_TRY(cudaFuncSetAttribute(k_bin_offsets<GroupRows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kOffMaxSmem));
+    return GS_OK;
+}
+
+// The cursors from the segment offsets, where the scan wrote those alone.
+__global__ void __launch_bounds__(256)
+k_group_cursors(const int32_t* __restrict__ off, const __grid_constant__ GroupViews gv, int32_t* __restrict__ cur)
+{
+    const int64_t n = gv.seg_base[gv.nv];
+    int v = 0;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
+        while (v + 1 < gv.nv && gv.seg_base[v + 1] <= q) ++v;
+        const int64_t l = q - gv.seg_base[v], t = l / gv.K[v], b = l - t * gv.K[v];
+        cur[gv.seg_base[v] + b * gv.tiles_x[v] * gv.tiles_y[v] + t] = off[q];
+    }
+}
+
 // The scatter of k_bin_scatter_rows (tiles.cu) for the group: a record's
-// item gives its view, whose tile grid, bin count and first segment place the
-// entry; four entries a lane in flight.
+// item gives its view, whose tile grid and first segment place its entries
+// (cursors bin by bin inside their view).
 __global__ void __launch_bounds__(256)
 k_group_scatter(const uint32_t* __restrict__ rs_g, const uint32_t* __restrict__ rs_ya, const uint32_t* __restrict__ rs_w,
-                const uint32_t* __restrict__ rs_z, const int32_t* __restrict__ roff, const GroupViews gv,
+                const uint32_t* __restrict__ rs_z, const int32_t* __restrict__ roff, const __grid_constant__ GroupViews gv,
                 const int64_t* __restrict__ m_dev, int64_t m_cap, int32_t* __restrict__ cur,
                 uint64_t* __restrict__ words)
 {
+    __shared__ ScatterShared s_sc[8];
     if (*m_dev > m_cap) return;
     const int64_t R = roff[gv.n * gv.nv];
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nchunks = (R + 31) / 32;
     const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < nchunks; c += wstride) {
+    for (int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; c < nchunks; c += wstride) {
         const int64_t k = c * 32 + lane;
-        uint32_t w = 0, g = 0, ya = 0, z = 0;
-        int view = 0;
+        uint32_t w = 0, g = 0, z = 0, slot = 0;
         if (k < R) {  // read once: streamed past L2
+            const uint32_t ya = __ldcs(rs_ya + k);
             w = __ldcs(rs_w + k);
             g = __ldcs(rs_g + k);
-            ya = __ldcs(rs_ya + k);
             z = __ldcs(rs_z + k);
-            view = gv.view_of(g);
+            const int v = gv.view_of(g), tx = gv.tiles_x[v];
+            slot = (uint32_t)(gv.seg_base[v] + (int64_t)(ya >> 24) * tx * gv.tiles_y[v] +
+                              (int)(ya & 0xfffu) * tx + (int)((ya >> 12) & 0xfffu));
         }
-        uint32_t incl = w;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += u;
-        }
-        const uint32_t excl = incl - w;
-        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        for (uint32_t e0 = 0; e0 < total; e0 += 32 * 4) {
-            int32_t pos[4];
-            uint64_t word[4];
-            bool live[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t e = e0 + 32 * u + lane;
-                int o = 0;
-#pragma unroll
-                for (int s = 16; s > 0; s >>= 1) {
-                    const uint32_t vv = __shfl_sync(0xffffffffu, excl, (o + s) & 31);
-                    if (o + s < 32 && vv <= e) o += s;
-                }
-                const uint32_t oex = __shfl_sync(0xffffffffu, excl, o);
-                const uint32_t og = __shfl_sync(0xffffffffu, g, o), oya = __shfl_sync(0xffffffffu, ya, o);
-                const uint32_t oz = __shfl_sync(0xffffffffu, z, o);
-                const int ov = __shfl_sync(0xffffffffu, view, o);
-                live[u] = e < total;
-                if (live[u]) {
-                    const int ty = (int)(oya & 0xfffu), tx = (int)((oya >> 12) & 0xfffu) + (int)(e - oex);
-                    const int64_t q = gv.seg_base[ov] + ((int64_t)ty * gv.tiles_x[ov] + tx) * gv.K[ov] + (oya >> 24);
-                    pos[u] = atomicAdd(&cur[q], 1);
-                    word[u] = ((uint64_t)oz << 32) | og;
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (live[u]) words[pos[u]] = word[u];
-        }
+        scatter_row_records(w, g, z, slot, 1u, cur, words, s_sc[warp], KeepAll());
     }
 }
 
@@ -379,7 +381,9 @@ int group_reserve(gs_ctx* gc, const GroupViews* gvp, int64_t m_cap)
         return r;
     gc->d_tiles = (int32_t*)tp;
     if ((r = goff_reserve(gc, N)) != GS_OK) return r;
-    return scan_reserve(gc, N > NS ? N : NS);
+    if ((r = scan_reserve(gc, N > NS ? N : NS)) != GS_OK) return r;
+    // ... and one flag word a tile row (the offsets' pass)
+    return ensure(&gc->d_scan, &gc->scan_bytes, ((size_t)gv.row_base[gv.nv] + 2) * sizeof(uint64_t));
 }
 
 int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m_views, cudaStream_t st)
@@ -418,8 +422,7 @@ int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m
     a.K = 0;  // set per view
     k_group_depth_range<<<(unsigned)gv.nv, kDrThreads, 0, st>>>(pv.c_o_z, gv, s.vc, s.samples, a, s.bp);
     gc->launches += N > 0 ? 3 : 2;
-    // row spans and per-row difference counts, per-view prefixes, the counts
-    // transposed into the group's segment order, one scan
+    // row spans and per-row difference counts, then the offsets
     GS_CUDA_TRY(cudaMemsetAsync(s.D, 0, (size_t)gv.d_base[gv.nv] * 4, st));
     const CullArgs ca{pv.xy_ab, pv.c_o_z, pv.rgb, 16};
     const int64_t warps = (N + 31) / 32;
@@ -427,24 +430,42 @@ int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m
         k_group_row_spans<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(pv.rect, roff, ca, gv, s.bp, gc->r_m,
                                                                        gc->r_m_cap, s.D, s.rs_g, s.rs_ya, s.rs_w,
                                                                        s.rs_z);
-    k_group_layer_prefix<<<(unsigned)gv.layer_base[gv.nv], 1024, 0, st>>>(s.D, gv);
     int max_tx = 1, max_k = 1;
+    size_t osm = 0;
     for (int v = 0; v < gv.nv; ++v) {
         max_tx = gv.tiles_x[v] > max_tx ? gv.tiles_x[v] : max_tx;
         max_k = gv.K[v] > max_k ? gv.K[v] : max_k;
+        const size_t need = bin_offsets_smem(gv.tiles_x[v], gv.K[v]);
+        osm = need > osm ? need : osm;
     }
-    k_group_transpose<<<dim3((unsigned)((max_tx + 31) / 32), (unsigned)((max_k + 31) / 32), (unsigned)gv.row_base[gv.nv]),
-                        256, 0, st>>>(s.D, gv, s.cur);
-    gc->launches += 3;
-    if ((r = scan_impl(gc, LoadI32{s.cur}, NS, gc->r_off, nullptr, st)) != GS_OK) return r;
     const unsigned g_sm = (unsigned)gc->num_sms * 8;
-    k_zero_if_over<<<g_sm, 256, 0, st>>>(gc->r_m, gc->r_m_cap, gc->r_off, NS + 1, gc->d_err);
+    const int n_rows = gv.row_base[gv.nv];
+    gc->launches += 1;
+    if (osm <= kOffMaxSmem) {
+        // one pass over every view's tile rows, cursors included (prefixes, a
+        // transposition, a scan, the over-capacity pass and a copy before:
+        // 57 us of kernels for 16 views of 1M Gaussians; the scatter with its
+        // cursors in segment order and four entries in flight 947 us)
+        uint64_t* flags;
+        if ((r = scan_flags(gc, n_rows, &flags, st)) != GS_OK) return r;
+        GS_CUDA_TRY(launch_k(gc, k_bin_offsets<GroupRows>, (unsigned)n_rows, kOffThreads, osm, st, GroupRows{s.D, gv},
+                             n_rows, gc->r_m, gc->r_m_cap, flags, gc->d_scan_done, gc->r_off, s.cur, gc->d_err));
+        gc->launches += 1;
+    } else {
+        // a view's tile rows too wide for one block's shared memory
+        k_group_layer_prefix<<<(unsigned)gv.layer_base[gv.nv], 1024, 0, st>>>(s.D, gv);
+        k_group_transpose<<<dim3((unsigned)((max_tx + 31) / 32), (unsigned)((max_k + 31) / 32), (unsigned)n_rows), 256, 0,
+                            st>>>(s.D, gv, s.cur);
+        if ((r = scan_impl(gc, LoadI32{s.cur}, NS, gc->r_off, nullptr, st)) != GS_OK) return r;
+        k_zero_if_over<<<g_sm, 256, 0, st>>>(gc->r_m, gc->r_m_cap, gc->r_off, NS + 1, gc->d_err);
+        k_group_cursors<<<g_sm, 256, 0, st>>>(gc->r_off, gv, s.cur);
+        gc->launches += 4;
+    }
     // the scatter: every entry a slot in its view's (tile, bin) segment
-    GS_CUDA_TRY(cudaMemcpyAsync(s.cur, gc->r_off, (size_t)NS * 4, cudaMemcpyDeviceToDevice, st));
     if (N > 0)
         k_group_scatter<<<g_sm * 2, 256, 0, st>>>(s.rs_g, s.rs_ya, s.rs_w, s.rs_z, roff, gv, gc->r_m, gc->r_m_cap,
                                                   s.cur, gc->r_stream);
-    gc->launches += 2;
+    gc->launches += 1;
     GS_CUDA_TRY(cudaGetLastError());
     // segments longer than the raster sorts in shared memory
     return sort_long_segments(gc, NS, gc->r_off, gc->r_stream, raster_sort_cap(16) + 1, st);

@@ -16,6 +16,7 @@
 // every segment, or the raster's in-shared-memory sort of each segment it
 // reaches (segments too long for its buffer are sorted here, eagerly).
 #include "device.cuh"
+#include "offsets.cuh"
 #include "rows.cuh"
 #include "scan.cuh"
 
@@ -197,35 +198,22 @@ k_layer_rows_prefix(int32_t* __restrict__ D, int tiles_x, int tiles_y, int64_t l
     }
 }
 
-// Warp-cooperative over the entries of 64 consecutive row records, two a
-// lane: a warp scans the lanes' record widths and keeps its records (gid,
-// tile row | first tile | bin, depth bits, first entry) in shared memory;
-// then, a window of 384 entries at a time, each record marks the window's
-// entries that are its own in a per-warp owner map, and each lane takes
-// every 32nd entry, reads its record through the map and takes a slot in the
-// entry's (tile, bin) segment -- the cursors start at the segment offsets, so
-// the atomic returns the slot itself.  Twelve entries per lane are in flight:
-// the kernel waits on its atomics' returns.  Measured at 1080p against a
-// binary search over the warp's prefix with the fields shuffled from the
-// owning lane: one record a lane and four in flight 13.6 us slower, two
-// records and twelve in flight 6.7 us slower (short-scoreboard stalls on
-// the shuffles); with the owner map, four records a lane were slower.  The
-// records carry the Gaussian's bin and depth bits, so nothing is gathered.
-//
-// The cursors of one bin lie tile by tile (Cursors): the entries of a record,
-// which neighbouring lanes hold, take their slots from neighbouring words, so
-// that a warp's atomic instruction reaches the L2 as a few sectors instead of
-// one a lane (bin stage at 1080p, 1M Gaussians: 203 -> 182 us).
-struct Cursors {
-    int32_t* p;
-    int64_t tile, bin;  // strides
-    __device__ __forceinline__ int32_t* at(int64_t t, int b) const { return p + t * tile + b * bin; }
+// The tile a pass keeps of a record (ScatterPass::keep), from the lane that
+// holds it in the warp's shared copy of the row words.
+struct KeepPlanned {
+    const ScatterPass& sp;
+    const uint32_t* ya;
+    int tiles_x;
+    __device__ __forceinline__ bool operator()(int o, uint32_t d) const
+    {
+        const uint32_t r = ya[o];
+        return sp.keep((int64_t)(r & 0xfffu) * tiles_x + ((r >> 12) & 0xfffu) + d, (int)(r >> 24));
+    }
 };
 
-constexpr int kScatRL = 2;                 // row records a lane
-constexpr int kScatIF = 12;                // entries a lane has in flight
-constexpr int kScatWin = 32 * kScatIF;     // entries a warp places a round
-
+// The scatter of a frame's row records (rows.cuh).  PLANNED: one pass of a
+// planned frame, which drops the records and entries it does not take.
+template <bool PLANNED>
 __global__ void __launch_bounds__(256)
 k_bin_scatter_rows(const uint32_t* __restrict__ rs_g, const uint32_t* __restrict__ rs_ya, const uint32_t* __restrict__ rs_w,
                    const uint32_t* __restrict__ rs_z, const int32_t* __restrict__ roff, int64_t n, int tiles_x,
@@ -233,84 +221,35 @@ k_bin_scatter_rows(const uint32_t* __restrict__ rs_g, const uint32_t* __restrict
                    uint64_t* __restrict__ words, const ScatterPass sp, const int32_t* __restrict__ flagged)
 {
     grid_dependency_sync();
-    // per warp: its 64 records {gid, tile row | first tile | bin, depth bits,
-    // first entry}, and for a round's window of entries the record of each
-    __shared__ uint4 s_rec[8][32 * kScatRL];
-    __shared__ uint8_t s_own[8][kScatWin];
+    __shared__ ScatterShared s_sc[8];
+    __shared__ uint32_t s_ya[PLANNED ? 8 : 1][32];
     if (*m_dev > m_cap) return;
-    if (sp.pass == 2 && flagged[0] == 0) return;  // no tile to complete
+    if (PLANNED && sp.pass == 2 && flagged[0] == 0) return;  // no tile to complete
     const int64_t R = roff[n];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint4* rec = s_rec[warp];
-    uint8_t* own = s_own[warp];
-    const int64_t nchunks = (R + 32 * kScatRL - 1) / (32 * kScatRL);
+    const int64_t nchunks = (R + 31) / 32;
     const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; c < nchunks; c += wstride) {
-        uint32_t w[kScatRL], g[kScatRL], ya[kScatRL], z[kScatRL];
-#pragma unroll
-        for (int h = 0; h < kScatRL; ++h) {
-            w[h] = g[h] = ya[h] = z[h] = 0;
-            const int64_t k = c * (32 * kScatRL) + kScatRL * lane + h;
-            if (k < R) {  // read once: streamed past L2
-                ya[h] = __ldcs(rs_ya + k);
-                w[h] = __ldcs(rs_w + k);
-                g[h] = __ldcs(rs_g + k);
-                z[h] = __ldcs(rs_z + k);
-                if (sp.row_live((int)(ya[h] & 0xfffu))) sp.trim(ya[h], w[h], tiles_x);
-                else w[h] = 0;
+        uint32_t w = 0, g = 0, ya = 0, z = 0;
+        const int64_t k = c * 32 + lane;
+        if (k < R) {  // read once: streamed past L2
+            ya = __ldcs(rs_ya + k);
+            if (!PLANNED || sp.row_live((int)(ya & 0xfffu))) {
+                w = __ldcs(rs_w + k);
+                g = __ldcs(rs_g + k);
+                z = __ldcs(rs_z + k);
+                if (PLANNED) sp.trim(ya, w, tiles_x);
             }
         }
-        uint32_t wl = 0;
-#pragma unroll
-        for (int h = 0; h < kScatRL; ++h) wl += w[h];
-        uint32_t incl = wl;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += u;
+        const uint32_t slot = (uint32_t)(((int64_t)(ya & 0xfffu) * tiles_x + ((ya >> 12) & 0xfffu)) * cur.tile +
+                                         (int64_t)(ya >> 24) * cur.bin);
+        if constexpr (PLANNED) {
+            s_ya[warp][lane] = ya;  // read after the warp barriers of the scatter
+            scatter_row_records(w, g, z, slot, (uint32_t)cur.tile, cur.p, words, s_sc[warp],
+                                KeepPlanned{sp, s_ya[warp], tiles_x});
+        } else {
+            scatter_row_records(w, g, z, slot, (uint32_t)cur.tile, cur.p, words, s_sc[warp], KeepAll());
         }
-        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        uint32_t st[kScatRL];
-        st[0] = incl - wl;
-#pragma unroll
-        for (int h = 1; h < kScatRL; ++h) st[h] = st[h - 1] + w[h - 1];
-#pragma unroll
-        for (int h = 0; h < kScatRL; ++h) rec[kScatRL * lane + h] = make_uint4(g[h], ya[h], z[h], st[h]);
-        for (uint32_t e0 = 0; e0 < total; e0 += kScatWin) {
-            // each record marks the entries of this window that are its own
-#pragma unroll
-            for (int h = 0; h < kScatRL; ++h) {
-                const uint32_t lo = st[h] > e0 ? st[h] : e0;
-                const uint32_t end = st[h] + w[h], wend = e0 + kScatWin;
-                const uint32_t hi = end < wend ? end : wend;
-                for (uint32_t x = lo; x < hi; ++x) own[x - e0] = (uint8_t)(kScatRL * lane + h);
-            }
-            __syncwarp();
-            int32_t p[kScatIF];
-            uint64_t word[kScatIF];
-            bool live[kScatIF];
-#pragma unroll
-            for (int u = 0; u < kScatIF; ++u) {
-                const uint32_t e = e0 + 32 * u + lane;
-                live[u] = e < total;
-                if (live[u]) {
-                    const uint4 r = rec[own[e - e0]];
-                    const uint32_t oya = r.y;
-                    const int ty = (int)(oya & 0xfffu), tx = (int)((oya >> 12) & 0xfffu) + (int)(e - r.w);
-                    const int64_t t = (int64_t)ty * tiles_x + tx;
-                    live[u] = sp.keep(t, (int)(oya >> 24));
-                    if (live[u]) {
-                        p[u] = atomicAdd(cur.at(t, (int)(oya >> 24)), 1);
-                        word[u] = ((uint64_t)r.z << 32) | r.x;
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kScatIF; ++u)
-                if (live[u]) words[p[u]] = word[u];
-            __syncwarp();  // the window's owner map is read before the next one is written
-        }
-        __syncwarp();  // the records are read before the next chunk's are written
     }
 }
 
@@ -504,126 +443,17 @@ k_transpose_counts(const int32_t* __restrict__ D, int tiles_x, int tiles_y, int 
     }
 }
 
-// The (tile, bin) segment offsets from the layered row differences
-// D[b][ty][x] in one pass, tile-major (t = ty tiles_x + x, bins inside): one
-// block per tile row (taken in ticket order) forms its counts by a prefix
-// along x per bin, scans them in tile-major order, finds the rows before it
-// by decoupled look-back over the rows' published totals (bounded waits),
-// and writes offsets and, when given, the scatter cursors.  Over capacity
-// (or past INT32_MAX) every offset is written 0 and GS_ERR_CAPACITY raised,
-// so nothing downstream reads out of bounds.  Replaces a per-layer prefix,
-// a transposition, a device-wide scan and the over-capacity pass.
-constexpr int kOffThreads = 1024;
-constexpr size_t kOffMaxSmem = 160 * 1024;
-__host__ __device__ inline size_t bin_offsets_smem(int tiles_x, int K) { return (size_t)tiles_x * (K + 1) * 4; }
-
-__global__ void __launch_bounds__(kOffThreads)
-k_bin_offsets(const int32_t* __restrict__ D, int tiles_x, int tiles_y, int K, int64_t layer,
-              const int64_t* __restrict__ m_dev, int64_t m_cap, uint64_t* flags, unsigned int* ticket,
-              int32_t* __restrict__ off, int32_t* __restrict__ cur, int* err)
-{
-    grid_dependency_sync();
-    extern __shared__ int32_t s_c[];  // [tiles_x][K + 1]: counts, then exclusive offsets in the row
-    __shared__ int32_t s_warp[kOffThreads / 32];
-    __shared__ int64_t s_pre;
-    __shared__ int s_row;
-    if (threadIdx.x == 0) {
-        const unsigned t = atomicAdd(ticket, 1u);
-        s_row = (int)t;
-        if ((int)t == tiles_y - 1) *ticket = 0u;  // every ticket is out: ready for the next scan
-    }
-    __syncthreads();
-    const int ty = s_row;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int KP = K + 1;
-    // counts: per bin, the inclusive prefix of the row's differences
-    for (int b = warp; b < K; b += kOffThreads / 32) {
-        const int32_t* row = D + (int64_t)b * layer + (int64_t)ty * (tiles_x + 1);
-        int32_t carry = 0;
-        for (int x0 = 0; x0 < tiles_x; x0 += 32) {
-            const int x = x0 + lane;
-            int32_t v = x < tiles_x ? row[x] : 0;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int32_t u = __shfl_up_sync(0xffffffffu, v, d);
-                if (lane >= d) v += u;
-            }
-            if (x < tiles_x) s_c[x * KP + b] = carry + v;
-            carry += __shfl_sync(0xffffffffu, v, 31);
-        }
-    }
-    __syncthreads();
-    // the row's exclusive scan in tile-major order: a run of items a thread
-    const int items = tiles_x * K;
-    const int per = (items + kOffThreads - 1) / kOffThreads;
-    const int j0 = threadIdx.x * per;
-    int32_t run = 0;
+// The tile rows of one frame (offsets.cuh).
+struct FrameRows {
+    const int32_t* D;
+    int tiles_x, tiles_y, K;
+    int64_t layer;
+    __device__ __forceinline__ OffsetRow operator()(int y) const
     {
-        int x = j0 / K, b = j0 - (j0 / K) * K;
-        for (int k = 0; k < per && j0 + k < items; ++k) {
-            run += s_c[x * KP + b];
-            if (++b == K) { b = 0; ++x; }
-        }
+        return OffsetRow{D + (int64_t)y * (tiles_x + 1), layer, tiles_x, K, (int64_t)y * tiles_x * K,
+                         (int64_t)y * tiles_x, (int64_t)tiles_x * tiles_y};
     }
-    int32_t incl = run;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int32_t u = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += u;
-    }
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        constexpr int NW = kOffThreads / 32;
-        int32_t w = lane < NW ? s_warp[lane] : 0;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int32_t u = __shfl_up_sync(0xffffffffu, w, d);
-            if (lane >= d) w += u;
-        }
-        if (lane < NW) s_warp[lane] = w;  // inclusive warp totals
-    }
-    __syncthreads();
-    const int64_t total = s_warp[kOffThreads / 32 - 1];
-    int32_t e = (warp > 0 ? s_warp[warp - 1] : 0) + incl - run;
-    {
-        int x = j0 / K, b = j0 - (j0 / K) * K;
-        for (int k = 0; k < per && j0 + k < items; ++k) {
-            const int32_t c = s_c[x * KP + b];
-            s_c[x * KP + b] = e;
-            e += c;
-            if (++b == K) { b = 0; ++x; }
-        }
-    }
-    // the rows before: publish this row's total, look back over theirs
-    volatile uint64_t* vf = flags;
-    if (threadIdx.x == 0) vf[ty] = (ty == 0 ? kScanFlagP : kScanFlagA) | (uint64_t)total;
-    if (warp == 0) {
-        const int64_t pre = ty > 0 ? scan_lookback(vf, ty, err) : 0;
-        if (lane == 0) {
-            if (ty > 0) vf[ty] = kScanFlagP | (uint64_t)(pre + total);
-            s_pre = pre;
-        }
-    }
-    __syncthreads();
-    const int64_t pre = s_pre;
-    const bool over = *m_dev > m_cap || pre + total > (int64_t)INT32_MAX - 1;
-    if (over && threadIdx.x == 0) raise_error(err, GS_ERR_CAPACITY);
-    const int64_t base = (int64_t)ty * items;
-    for (int j = threadIdx.x; j < items; j += kOffThreads) {
-        const int x = j / K, b = j - x * K;
-        const int32_t v = over ? 0 : (int32_t)(pre + s_c[x * KP + b]);
-        off[base + j] = v;
-    }
-    if (cur) {  // bin by bin, tiles inside
-        const int64_t T = (int64_t)tiles_x * tiles_y;
-        for (int j = threadIdx.x; j < items; j += kOffThreads) {
-            const int b = j / tiles_x, x = j - b * tiles_x;
-            cur[b * T + (int64_t)ty * tiles_x + x] = over ? 0 : (int32_t)(pre + s_c[x * KP + b]);
-        }
-    }
-    if (ty == tiles_y - 1 && threadIdx.x == 0) off[(int64_t)tiles_y * items] = over ? 0 : (int32_t)(pre + total);
-}
+};
 
 struct LoadPlainCount {
     const int32_t* C;
@@ -761,7 +591,7 @@ static int exact_scatter(gs_ctx* ctx, const ExactScratch& v, int64_t n, int32_t 
             GS_CUDA_TRY(launch_k(ctx, k_flagged_cursors, (unsigned)ctx->num_sms * 2, 256, 0, st, flagged, offsets, K, cur));
             ctx->launches += 1;
         }
-        GS_CUDA_TRY(launch_k(ctx, k_bin_scatter_rows, g_sm * 2, 256, 0, st, v.rs_g, v.rs_ya, v.rs_w, v.rs_z, v.roff, n, tiles_x, m_dev,
+        GS_CUDA_TRY(launch_k(ctx, sp.pass ? k_bin_scatter_rows<true> : k_bin_scatter_rows<false>, g_sm * 2, 256, 0, st, v.rs_g, v.rs_ya, v.rs_w, v.rs_z, v.roff, n, tiles_x, m_dev,
                                                      m_cap, cur, words, sp, flagged));
         ctx->launches += 1;
     }
@@ -818,8 +648,9 @@ int exact_frame_zero(gs_ctx* ctx, int64_t n, const gs_camera* cam, int64_t m_cap
 // context, on its device.
 int bin_offsets_prepare()
 {
-    GS_CUDA_TRY(cudaFuncSetAttribute(k_bin_offsets, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOffMaxSmem));
-    return GS_OK;
+    GS_CUDA_TRY(cudaFuncSetAttribute(k_bin_offsets<FrameRows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kOffMaxSmem));
+    return group_offsets_prepare();
 }
 
 int exact_scatter_rest(gs_ctx* ctx, int64_t n, const gs_camera* cam, int64_t m_cap, const int64_t* m_dev,
@@ -877,9 +708,9 @@ int exact_bins(gs_ctx* ctx, const ProjView& pv, int64_t n, const gs_camera* cam,
             // one pass: counts, tile-major scan, look-back over tile rows
             uint64_t* flags;
             if ((r = scan_flags(ctx, tiles_y, &flags, st)) != GS_OK) return r;
-            GS_CUDA_TRY(launch_k(ctx, k_bin_offsets, (unsigned)tiles_y, kOffThreads, osm, st, v.D, tiles_x, tiles_y,
-                                 K, rlayer, m_dev, m_cap, flags, ctx->d_scan_done, offsets,
-                                 want_cur ? v.cur : nullptr, ctx->d_err));
+            GS_CUDA_TRY(launch_k(ctx, k_bin_offsets<FrameRows>, (unsigned)tiles_y, kOffThreads, osm, st,
+                                 FrameRows{v.D, tiles_x, tiles_y, K, rlayer}, (int)tiles_y, m_dev, m_cap, flags,
+                                 ctx->d_scan_done, offsets, want_cur ? v.cur : nullptr, ctx->d_err));
             ctx->launches += 1;
         } else {
             // rows too wide for one block's shared memory: per-layer prefix,
