@@ -580,7 +580,7 @@ int gs::render_save_buffers(gs_ctx* c, int32_t W, int32_t H, int32_t T)
     c->r_tend = (int32_t*)p;
     p = c->r_wend;
     const int ts = c->cfg.tile_size;
-    if ((r = ensure(&p, &c->r_wend_cap, (size_t)T * (ts * ts / 32) * 4 + 4)) != GS_OK) return r;
+    if ((r = ensure(&p, &c->r_wend_cap, (size_t)T * (ts * ts / 64) * 4 + 4)) != GS_OK) return r;
     c->r_wend = (int32_t*)p;
     return GS_OK;
 }

@@ -26,69 +26,9 @@
 
 namespace gs {
 
-// A warp's block of pixels and its lanes: 8 x 8 pixels, two a lane, (x, y) and
-// (x + 4, y).  They share dy and the entry's shared-memory reads, and what is
-// done to both runs on packed float32 pairs (each half rounded as the scalar
-// operation).
-constexpr int kBH = 8;
-
-// ------------------------------------------------------------------ packed float32 pairs
-__device__ __forceinline__ uint64_t pk2(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void upk2(uint64_t v, float& lo, float& hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t same2(float v) { return pk2(v, v); }
-
-// exp(-q) of two q by spec_exp_core's steps (internal.cuh), bit for bit where
-// its value is used (0 <= q <= 87).  The reduced argument is carried negated
-// (s = -r), which mirrors every rounding: the odd Horner stages come out
-// negated and the last one does not.  2^n is applied to the normal result by
-// adding n to its exponent field: the low 9 bits of the shifter's bits are
-// zero, so bits(k) << 23 is n << 23.
-__device__ __forceinline__ void spec_exp_neg2(float q0, float q1, float& e0, float& e1)
-{
-    const uint64_t q = pk2(q0, q1);
-    const uint64_t k = fma2(q, same2(-1.44269504088896341f), same2(12582912.0f));
-    const uint64_t n = add2(k, same2(-12582912.0f));
-    uint64_t s = fma2(n, same2(0.693145751953125f), q);
-    s = fma2(n, same2(1.42860682030941723e-6f), s);
-    uint64_t p = fma2(same2(-1.0f / 5040.0f), s, same2(1.0f / 720.0f));
-    p = fma2(p, s, same2(-1.0f / 120.0f));
-    p = fma2(p, s, same2(1.0f / 24.0f));
-    p = fma2(p, s, same2(-1.0f / 6.0f));
-    p = fma2(p, s, same2(0.5f));
-    p = fma2(p, s, same2(-1.0f));
-    p = fma2(p, s, same2(1.0f));
-    float p0, p1, k0, k1;
-    upk2(p, p0, p1);
-    upk2(k, k0, k1);
-    e0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(k0) << 23));
-    e1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(k1) << 23));
-}
+// A lane's two pixels of its warp's 8 x 8 block: (x, y) and (x + 4, y).  They
+// share dy and the entry's shared-memory reads, and what is done to both runs
+// on packed float32 pairs (each half rounded as the scalar operation).
 
 // Per-thread compositing state: two pixels.  A pixel that has stopped (or lies
 // outside the image) has a NaN centre, so that no entry passes it again.
@@ -100,14 +40,6 @@ struct PixelState {
     int live;       // bit h: pixel h is still compositing
     unsigned long long ops;
 };
-
-// One staged entry at both pixels: q of each.
-__device__ __forceinline__ void entry_q(const float4& ga, const float4& gb, const PixelState& st, float& q0, float& q1)
-{
-    const float dy = ga.y - st.y;
-    const uint64_t dx = pk2(ga.x - st.x[0], ga.x - st.x[1]);
-    upk2(fma2(dx, fma2(same2(ga.z), dx, same2(ga.w * dy)), same2((gb.x * dy) * dy)), q0, q1);
-}
 
 // alpha of one entry where the pixel takes it (pass), else 0.  0 <= q <= tau
 // as one unsigned compare of the float bits (negative q and NaN compare above
@@ -193,11 +125,11 @@ __device__ __forceinline__ void apply_with_stops(const EntryAlpha& e, const floa
 // SKIP (the plain raster, whose warps visit entries far from their pixels):
 // a round no pixel of which has q <= tau ends there.
 template <int TILE, bool SKIP, int R>
-__device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE, kBH>& sh, PixelState& st, int32_t base)
+__device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE>& sh, PixelState& st, int32_t base)
 {
     const int warp = threadIdx.x >> 5;
     if (__all_sync(0xffffffffu, st.live == 0)) return;
-    const int nk = warp_strip_list<TILE, kBH>(sh, cnt);
+    const int nk = warp_strip_list<TILE>(sh, cnt);
     const char* pa = reinterpret_cast<const char*>(sh.a);
     const char* pb = reinterpret_cast<const char*>(sh.b);
     const char* pc = reinterpret_cast<const char*>(sh.c);
@@ -214,7 +146,8 @@ __device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE, kBH>
 #pragma unroll
         for (int j = 0; j < R; ++j) {
             gb[j] = *reinterpret_cast<const float4*>(pb + k[j]);
-            entry_q(*reinterpret_cast<const float4*>(pa + k[j]), gb[j], st, q[j][0], q[j][1]);
+            entry_q(*reinterpret_cast<const float4*>(pa + k[j]), gb[j], st.x[0], st.x[1], st.y, q[j][0],
+                    q[j][1]);
         }
         if constexpr (SKIP) {
             bool any = false;
@@ -256,11 +189,11 @@ __device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE, kBH>
 
 // The counting twin: one pixel and one entry at a time, the same values.
 template <int TILE>
-__device__ __forceinline__ void composite_batch_count(int cnt, RasterShared<TILE, kBH>& sh, PixelState& st,
+__device__ __forceinline__ void composite_batch_count(int cnt, RasterShared<TILE>& sh, PixelState& st,
                                                       int32_t base)
 {
     const int warp = threadIdx.x >> 5;
-    const int nk = warp_strip_list<TILE, kBH>(sh, cnt);
+    const int nk = warp_strip_list<TILE>(sh, cnt);
     float T[2], C0[2], C1[2], C2[2];
     upk2(st.T, T[0], T[1]);
     upk2(st.C0, C0[0], C0[1]);
@@ -307,7 +240,7 @@ __device__ __forceinline__ void composite_batch_count(int cnt, RasterShared<TILE
 // runs and staged chunks to (raster_common.cuh).
 template <int TILE, bool COUNT, bool LAZY, int R>
 struct FwdSpan {
-    using SH = RasterShared<TILE, kBH>;
+    using SH = RasterShared<TILE>;
     static constexpr int kBatch = SH::BATCH;
     SH& sh;
     const float4* __restrict__ xy_ab;
@@ -324,7 +257,7 @@ struct FwdSpan {
             // checked: the caller has just counted the terminated pixels (block
             // barrier included) with nothing composited since
             if (!(checked && b0 == 0) && __syncthreads_count(done()) == SH::TB::NT) return b0;
-            const int cnt = stage_batch<TILE, kBH>(src, b0, n, sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty);
+            const int cnt = stage_batch<TILE>(src, b0, n, sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty);
             __syncthreads();
             composite_staged(cnt, base + b0);
         }
@@ -334,7 +267,7 @@ struct FwdSpan {
     __device__ __forceinline__ void stage_at(int slot, uint32_t g)
     {
         float4 A, B, C;
-        stage_record<TILE, kBH>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
+        stage_record<TILE>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
         sh.a[slot] = A;
         sh.b[slot] = B;
         sh.c[slot] = C;
@@ -359,14 +292,14 @@ struct FwdSpan {
 // One tile t by the whole block (the body of the raster kernels below).
 template <int TILE, bool COUNT, bool LAZY, int R>
 __device__ __forceinline__ void raster_tile(
-    int t, RasterShared<TILE, kBH>& sh, WalkShared<TILE, LAZY>& ws, const float4* __restrict__ xy_ab,
+    int t, RasterShared<TILE>& sh, WalkShared<TILE, LAZY>& ws, const float4* __restrict__ xy_ab,
     const float4* __restrict__ c_o_z, const float4* __restrict__ rgbv, uint64_t* words,
     const int32_t* __restrict__ off, const RasterArgs& a, int cullmode, float* __restrict__ out_rgb,
     float* __restrict__ out_alpha, int32_t* __restrict__ out_last, int32_t* __restrict__ out_ntests,
     unsigned long long* __restrict__ ops_total, float* __restrict__ out_T, int32_t* __restrict__ out_end,
     const PlanView& pl, int cap, int32_t* __restrict__ out_wend = nullptr)
 {
-    using TB = TileBlocks<TILE, kBH>;
+    using TB = TileBlocks<TILE>;
     const int tx = t % a.tiles_x, ty = t / a.tiles_x;
     const int lane = threadIdx.x & 31;
     // the lane's first pixel; the second is four to its right
@@ -428,16 +361,11 @@ __device__ __forceinline__ void raster_tile(
         walk_tile<TILE, LAZY, TB::NT>(words, off, t, K, kbegin, kend, cap, ws, span, out_end ? words : nullptr);
     if (out_end && threadIdx.x == 0) out_end[t] = end;
     if (out_wend) {
-        // per 8 x 4 block of pixels, the stream position past the entry that
-        // stopped its last pixel (the tile's end when one of its pixels never
-        // stopped): the backward has nothing to do for it at or beyond it.
-        // Lanes 0..15 hold the upper four rows of the warp's block.
-        int32_t m = !inside ? INT32_MIN : (st.live ? end : st.stop + 1);
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-        const int col = TB::x0() / 8, row = TB::y0() / 4 + (lane >> 4);
-        if ((lane & 15) == 0)
-            out_wend[(int64_t)t * (TILE * TILE / 32) + row * TB::COLS + col] = m == INT32_MIN ? 0 : min(m, end);
+        // per warp, the stream position past the entry that stopped its last
+        // pixel (the tile's end when one of its pixels never stopped): the
+        // backward has nothing to do for the warp at or beyond it
+        const int32_t m = __reduce_max_sync(0xffffffffu, !inside ? INT32_MIN : (st.live ? end : st.stop + 1));
+        if (lane == 0) out_wend[(int64_t)t * TB::NW + (threadIdx.x >> 5)] = m == INT32_MIN ? 0 : min(m, end);
     }
     bool unfinished = false;
     if (pl.flag && kend < K) {
@@ -539,7 +467,7 @@ __device__ __forceinline__ void raster_tile(
 // Threads of a tile's block and the blocks an SM holds: 16 x 16 tiles' seven
 // blocks of 128 threads fill the shared memory (31.8 KB each).
 template <int TILE>
-constexpr int raster_threads() { return TileBlocks<TILE, kBH>::NT; }
+constexpr int raster_threads() { return TileBlocks<TILE>::NT; }
 template <int TILE>
 constexpr int raster_min_blocks() { return TILE == 16 ? 7 : TILE == 8 ? 16 : 2; }
 // ... and with rounds of four
@@ -556,7 +484,7 @@ k_raster(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o_z, con
          int32_t* __restrict__ out_end, const PlanView pl, int cap, int32_t* __restrict__ out_wend)
 {
     grid_dependency_sync();
-    __shared__ RasterShared<TILE, kBH> sh;
+    __shared__ RasterShared<TILE> sh;
     __shared__ WalkShared<TILE, LAZY> ws;
     raster_tile<TILE, COUNT, LAZY, R>(blockIdx.x, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode, out_rgb, out_alpha,
                                    out_last, out_ntests, ops_total, out_T, out_end, pl, cap, out_wend);
@@ -574,7 +502,7 @@ k_raster_listed(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o
                 const int32_t* __restrict__ list, int cap)
 {
     grid_dependency_sync();
-    __shared__ RasterShared<TILE, kBH> sh;
+    __shared__ RasterShared<TILE> sh;
     __shared__ WalkShared<TILE, true> ws;
     PlanView pl;
     pl.bins = plan;
@@ -654,7 +582,7 @@ __global__ void __launch_bounds__(raster_threads<TILE>(), raster_min_blocks<TILE
 k_raster_views(const __grid_constant__ ViewRasterSet vs, const int32_t* __restrict__ order,
                int32_t* __restrict__ counter)
 {
-    __shared__ RasterShared<TILE, kBH> sh;
+    __shared__ RasterShared<TILE> sh;
     __shared__ WalkShared<TILE, LAZY> ws;
     __shared__ int32_t s_item;
     for (;;) {

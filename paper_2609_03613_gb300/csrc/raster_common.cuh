@@ -13,31 +13,98 @@
 
 namespace gs {
 
+// ------------------------------------------------------------------ packed float32 pairs
+__device__ __forceinline__ uint64_t pk2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void upk2(uint64_t v, float& lo, float& hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t same2(float v) { return pk2(v, v); }
+
+// exp(-q) of two q by spec_exp_core's steps (internal.cuh), bit for bit where
+// its value is used (0 <= q <= 87).  The reduced argument is carried negated
+// (s = -r), which mirrors every rounding: the odd Horner stages come out
+// negated and the last one does not.  2^n is applied to the normal result by
+// adding n to its exponent field: the low 9 bits of the shifter's bits are
+// zero, so bits(k) << 23 is n << 23.
+__device__ __forceinline__ void spec_exp_neg2(float q0, float q1, float& e0, float& e1)
+{
+    const uint64_t q = pk2(q0, q1);
+    const uint64_t k = fma2(q, same2(-1.44269504088896341f), same2(12582912.0f));
+    const uint64_t n = add2(k, same2(-12582912.0f));
+    uint64_t s = fma2(n, same2(0.693145751953125f), q);
+    s = fma2(n, same2(1.42860682030941723e-6f), s);
+    uint64_t p = fma2(same2(-1.0f / 5040.0f), s, same2(1.0f / 720.0f));
+    p = fma2(p, s, same2(-1.0f / 120.0f));
+    p = fma2(p, s, same2(1.0f / 24.0f));
+    p = fma2(p, s, same2(-1.0f / 6.0f));
+    p = fma2(p, s, same2(0.5f));
+    p = fma2(p, s, same2(-1.0f));
+    p = fma2(p, s, same2(1.0f));
+    float p0, p1, k0, k1;
+    upk2(p, p0, p1);
+    upk2(k, k0, k1);
+    e0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(k0) << 23));
+    e1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(k1) << 23));
+}
+
+// One staged entry at two pixels of a row (centres x0, x1; y): q of each.
+__device__ __forceinline__ void entry_q(const float4& ga, const float4& gb, float x0, float x1, float y, float& q0,
+                                        float& q1)
+{
+    const float dy = ga.y - y;
+    const uint64_t dx = pk2(ga.x - x0, ga.x - x1);
+    upk2(fma2(dx, fma2(same2(ga.z), dx, same2(ga.w * dy)), same2((gb.x * dy) * dy)), q0, q1);
+}
+
 struct RasterArgs {
     int width, height, tiles_x, n_tiles, stride;
     float bg0, bg1, bg2;
     int32_t gid_base = 0;  // stream words hold gid_base + gid (the last-id output subtracts it)
 };
 
-// A warp owns a block of 8 x BH pixels of the tile (BH = 4: a pixel a lane;
-// BH = 8: two).  Blocks are laid out TILE/8 wide and TILE/BH tall, warps
-// row-major over them; the block of the tile has one warp for each.
-template <int TILE, int BH>
+// A warp owns a block of 8 x 8 pixels of the tile, two a lane.  Blocks are laid
+// out TILE/8 wide and tall, warps row-major over them; the block of the tile
+// has one warp for each.
+template <int TILE>
 struct TileBlocks {
-    static constexpr int COLS = TILE / 8, ROWS = TILE / BH;
+    static constexpr int COLS = TILE / 8, ROWS = TILE / 8;
     static constexpr int NW = COLS * ROWS;    // warps of the tile
     static constexpr int NT = 32 * NW;        // threads of the tile
     __device__ static int x0() { return ((threadIdx.x >> 5) % COLS) * 8; }
-    __device__ static int y0() { return ((threadIdx.x >> 5) / COLS) * BH; }
+    __device__ static int y0() { return ((threadIdx.x >> 5) / COLS) * 8; }
 };
 
 // Entries staged per batch.
 template <int TILE>
 constexpr int raster_batch() { return TILE == 8 ? 128 : 256; }
 
-template <int TILE, int BH>
+template <int TILE>
 struct RasterShared {
-    using TB = TileBlocks<TILE, BH>;
+    using TB = TileBlocks<TILE>;
     static constexpr int BATCH = raster_batch<TILE>();
     float4 a[BATCH + 1];  // {mx, my, a/2, b}; the last slot of each array is a
     float4 b[BATCH + 1];  // {c/2, o, tau, gid bits}        zero record, which no
@@ -56,8 +123,8 @@ struct RasterShared {
 // The staged entries (of cnt) whose warp mask admits the calling warp, in
 // stage order, into sh.list[warp], followed by three references to the zero
 // record (a whole round of two or four); returns their count.  Whole warp.
-template <int TILE, int BH>
-__device__ __forceinline__ int warp_strip_list(RasterShared<TILE, BH>& sh, int cnt)
+template <int TILE>
+__device__ __forceinline__ int warp_strip_list(RasterShared<TILE>& sh, int cnt)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int nw = 0;
@@ -68,26 +135,26 @@ __device__ __forceinline__ int warp_strip_list(RasterShared<TILE, BH>& sh, int c
         if (mine) sh.list[warp][nw + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(16 * j);
         nw += __popc(bal);
     }
-    if (lane < 3) sh.list[warp][nw + lane] = (uint16_t)(16 * RasterShared<TILE, BH>::BATCH);
+    if (lane < 3) sh.list[warp][nw + lane] = (uint16_t)(16 * RasterShared<TILE>::BATCH);
     __syncwarp();
     return nw;
 }
 
 // Warp mask of an entry: bit w is set when the entry's alpha >= 1/255
 // ellipse (the tile cull's bound Q(d) <= tau / margin, d = mean - pixel
-// centre, widened as there) reaches a pixel centre of warp w's 8 x BH block of
-// the tile (origin x0, y0).  Per band of BH pixel rows the ellipse's
+// centre, widened as there) reaches a pixel centre of warp w's 8 x 8 block of
+// the tile (origin x0, y0).  Per band of eight pixel rows the ellipse's
 // x-extent over the band's centre rows (the row-span geometry of the bin
 // stage: band ends and the ellipse's leftmost / rightmost points) is widened
 // by 5e-3 relative + 0.05 px and tested against each block's centre columns,
 // so a warp never skips a pixel the entry can reach.  The geometry takes the
 // hardware's approximate division and square root (relative errors near
 // 2^-22, far inside the widening).
-template <int TILE, int BH>
+template <int TILE>
 __device__ __forceinline__ uint32_t strip_mask(float mx, float my, float ha, float hb, float hc, float tau,
                                                float margin, float x0, float y0)
 {
-    using WB = TileBlocks<TILE, BH>;
+    using WB = TileBlocks<TILE>;
     constexpr int NWT = WB::NW;
     const uint32_t all = NWT >= 32 ? 0xffffffffu : ((1u << NWT) - 1u);
     if (!(margin > 0.0f)) return all;
@@ -105,7 +172,7 @@ __device__ __forceinline__ uint32_t strip_mask(float mx, float my, float ha, flo
     uint32_t m = 0u;
 #pragma unroll
     for (int by = 0; by < WB::ROWS; ++by) {
-        float yl = my - (y0 + (float)(BH * by) + ((float)BH - 0.5f)), yh = my - (y0 + (float)(BH * by) + 0.5f);
+        float yl = my - (y0 + (float)(8 * by) + 7.5f), yh = my - (y0 + (float)(8 * by) + 0.5f);
         yl = yl - (0.05f + 5e-3f * fabsf(yl));
         yh = yh + (0.05f + 5e-3f * fabsf(yh));
         const float ya = fmaxf(yl, -dymax), yb = fminf(yh, dymax);
@@ -137,7 +204,7 @@ constexpr int kPlain = 4;      // neither: the plain raster
 // q = c_o_z[g] and colour c = rgbv[g]: {mx, my, a/2, b}, {c/2, o, tau, gid
 // bits} and the colour with the warp mask in .w (zero when the tile cull
 // drops the entry: no warp's list admits it).
-template <int TILE, int BH>
+template <int TILE>
 __device__ __forceinline__ void stage_record(uint32_t g, const float4& p, const float4& q, float4 c, int cullmode,
                                              int tx, int ty, float4& A, float4& B, float4& C)
 {
@@ -149,7 +216,7 @@ __device__ __forceinline__ void stage_record(uint32_t g, const float4& p, const 
     bool keep = true;
     if (cullmode & kCullTile)
         keep = !tile_culled(A.x, A.y, A.z, A.w, B.x, q.w, c.w, (float)(tx * TILE), (float)(ty * TILE), (float)TILE);
-    const uint32_t m = (cullmode & kCullWarp) ? strip_mask<TILE, BH>(A.x, A.y, A.z, A.w, B.x, q.w, c.w,
+    const uint32_t m = (cullmode & kCullWarp) ? strip_mask<TILE>(A.x, A.y, A.z, A.w, B.x, q.w, c.w,
                                                                      (float)(tx * TILE), (float)(ty * TILE))
                                               : 0xffffffffu;
     c.w = __uint_as_float(keep ? m : 0u);
@@ -161,13 +228,13 @@ __device__ __forceinline__ void stage_record(uint32_t g, const float4& p, const 
 // the colour with the warp mask in .w (zero for an entry the tile cull
 // drops).  Returns the number staged (block-uniform); the caller
 // synchronises the block before reading sh.
-template <int TILE, int BH>
+template <int TILE>
 __device__ __forceinline__ int stage_batch(const uint64_t* src, int32_t b0, int32_t n_entries,
-                                           RasterShared<TILE, BH>& sh, const float4* __restrict__ xy_ab,
+                                           RasterShared<TILE>& sh, const float4* __restrict__ xy_ab,
                                            const float4* __restrict__ c_o_z, const float4* __restrict__ rgbv,
                                            int cullmode, int tx, int ty)
 {
-    using SH = RasterShared<TILE, BH>;
+    using SH = RasterShared<TILE>;
     const int cnt = min(SH::BATCH, n_entries - b0);
     // entry i of the batch goes to slot i: the tile cull and the warp mask
     // leave a zero mask, which no warp's list admits (stream order is kept
@@ -175,7 +242,7 @@ __device__ __forceinline__ int stage_batch(const uint64_t* src, int32_t b0, int3
     auto put = [&](int i) {
         const uint32_t g = (uint32_t)(src[b0 + i] & 0xffffffffull);
         float4 A, B, C;
-        stage_record<TILE, BH>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
+        stage_record<TILE>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
         sh.a[i] = A;
         sh.b[i] = B;
         sh.c[i] = C;
