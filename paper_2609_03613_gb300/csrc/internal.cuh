@@ -575,6 +575,8 @@ int raster_bwd_prepare();
 int bin_offsets_prepare();
 // batch_bins.cu
 int group_offsets_prepare();
+// bins.cu
+int sort_listed_prepare();
 int raster_bwd(gs_ctx* ctx, const ProjView& pv, const gs_camera* cam, const uint64_t* words, const int32_t* offsets,
                int32_t stride, const float* bg, const int32_t* last, const float* final_T,
                const int32_t* tile_end, const float* dl_drgb, const float* dl_dalpha, const GradView& gv,

@@ -387,7 +387,9 @@ __device__ __forceinline__ int32_t walk_tile(const uint64_t* words, const int32_
                 continue;
             }
             // one long segment: sorted in shared memory by the block, or before
-            // the raster
+            // the raster (in depth buckets ranked batch by batch, as
+            // k_sort_listed does, measured no faster here: 164 against 162 us
+            // for 3M Gaussians seen from inside a cluster)
             const bool sorted = n > raster_sort_cap(TILE);
             if (!sorted) {
                 for (int i = threadIdx.x; i < n; i += NT) ws.sort[i] = __ldcs(wl + at + i);

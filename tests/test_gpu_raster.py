@@ -37,15 +37,21 @@ def test_ragged_sizes_and_round_widths(w, h, tile):
         assert_image(mode, sc, cam, tile, 64 if mode == "exact" else 1, ref)
 
 
+@pytest.mark.parametrize("depths", ["spread", "equal", "skewed"])
 @pytest.mark.parametrize("tile", [8, 16])
-@pytest.mark.parametrize("count", [127, 128, 129, 255, 256, 257, 511, 512, 513, 2047, 2048, 2049])
-def test_segments_at_batch_and_sort_limits(count, tile):
-    # one bin a tile holding `count` entries (all inside one tile, none
-    # terminating it): staged at rank, sorted by the block, or sorted before
-    # the raster
+@pytest.mark.parametrize("count", [128, 129, 256, 257, 512, 513, 2048, 2049, 8191, 8192, 8193])
+def test_segments_at_batch_and_sort_limits(count, tile, depths):
+    # one bin a tile holding `count` entries (all inside one tile, which stops
+    # after some two thousand of them): staged at
+    # rank, in depth buckets in the raster, or sorted before it.  Equal depths
+    # and depths crowded at one end fill a bucket past its limit.
     rng = np.random.default_rng(count)
     cam = scenes.tiny_camera()
     z = rng.uniform(-0.4, 0.4, count)
+    if depths == "equal":
+        z = np.where(rng.random(count) < 0.7, 0.1, z)
+    elif depths == "skewed":
+        z = 0.4 - 0.8 * rng.random(count) ** 40
     xy = (132.0 + rng.uniform(-1.0, 1.0, (count, 2)) - cam.cx) * (3.0 - z)[:, None] / cam.fx
     sc = scenes.Scene(np.column_stack([xy, z]).astype(np.float32), np.full((count, 3), 0.002, np.float32),
                       np.tile(np.array([1, 0, 0, 0], np.float32), (count, 1)),
