@@ -34,9 +34,6 @@ struct BatchState {
     cudaGraphExec_t gexec = nullptr;
     std::vector<unsigned char> gkey;
     int64_t glaunches = 0;
-    int32_t* d_counter = nullptr;  // schedule of the persistent multi-view raster (65 int32)
-    int32_t* d_order = nullptr;    // its work items, longest tiles first
-    size_t order_cap = 0;
     // the group of views binned together (batch_bins.cu)
     gs_ctx* group = nullptr;                  // its scratch, stream and offsets, error word
     GroupViews* gview = nullptr;              // its view table
@@ -56,8 +53,6 @@ void batch_destroy(gs_ctx* c)
         if (b->join[v]) cudaEventDestroy(b->join[v]);
     }
     if (b->fork) cudaEventDestroy(b->fork);
-    if (b->d_counter) cudaFree(b->d_counter);
-    if (b->d_order) cudaFree(b->d_order);
     if (b->group) gs_destroy(b->group);
     if (b->gview) group_views_free(b->gview);
     if (b->h_group_m) cudaFreeHost(b->h_group_m);
@@ -100,11 +95,9 @@ static BatchState* batch_state(gs_ctx* c)
     if (!c->batch) {
         BatchState* b = new BatchState();
         if (cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
-            cudaMalloc(&b->d_counter, 65 * sizeof(int32_t)) != cudaSuccess ||
             cudaMallocHost(&b->h_group_m, kMaxBatchViews * sizeof(int64_t)) != cudaSuccess ||
             !(b->gview = group_views_new())) {
             if (b->fork) cudaEventDestroy(b->fork);
-            if (b->d_counter) cudaFree(b->d_counter);
             if (b->h_group_m) cudaFreeHost(b->h_group_m);
             delete b;
             return nullptr;
@@ -202,16 +195,7 @@ static int batch_group(gs_ctx* c, const gs_scene* sc, const gs_camera* cams, int
 static int batch_buffers(gs_ctx* c, const gs_scene* sc, const gs_camera* cams, int nv, int32_t* const* last,
                          int32_t flags)
 {
-    {
-        BatchState* b = batch_state(c);
-        if (!b) return GS_ERR_NO_MEMORY;
-        size_t tiles = 0;
-        for (int v = 0; v < nv; ++v) tiles += (size_t)gs_num_tiles(cams[v].width, cams[v].height, 16);
-        void* p = b->d_order;
-        const int r = ensure(&p, &b->order_cap, tiles * sizeof(int32_t) + 256);
-        if (r != GS_OK) return r;
-        b->d_order = (int32_t*)p;
-    }
+    if (!batch_state(c)) return GS_ERR_NO_MEMORY;
     for (int v = 0; v < nv; ++v) {
         gs_ctx* vc;
         int r = view_ctx(c, v, &vc);
@@ -293,7 +277,8 @@ static int batch_impl(gs_ctx* c, const gs_scene* sc, const gs_camera* cams, int 
     // persistent raster launch over all its views' tiles
     if (b->ngroup > 0) {
         gc->capturing = c->capturing;
-        r = group_binning(gc, b->gview, flags, b->h_group_m, st);
+        TileOrder order;
+        r = group_binning(gc, b->gview, flags, b->h_group_m, &order, st);
         gc->capturing = 0;
         if (r != GS_OK) return r;
         RasterView rv[kMaxBatchViews];
@@ -315,7 +300,7 @@ static int batch_impl(gs_ctx* c, const gs_scene* sc, const gs_camera* cams, int 
             x.last = (last && last[v]) ? last[v] : reinterpret_cast<int32_t*>(b->views[v]->r_out);
             x.gid_base = (int32_t)(p * n);
         }
-        if ((r = raster_views(c, rv, k, b->d_counter, b->d_order, st)) != GS_OK) return r;
+        if ((r = raster_views(c, rv, k, order, gc->d_tail + kTailWork, st)) != GS_OK) return r;
     }
     for (int v = 0; v < nv; ++v)
         if (forked[v]) GS_CUDA_TRY(cudaStreamWaitEvent(st, b->join[v], 0));
@@ -410,14 +395,14 @@ extern "C" int gs_render_batch(gs_ctx* c, const gs_scene* sc, const gs_camera* c
     }
     if (b->group) {
         const gs_ctx* gc = b->group;
-        const void* gptr[] = {gc->r_proj, gc->r_stream, gc->r_off, gc->d_tiles, gc->d_goff, gc->d_scan, gc->d_tail};
+        const void* gptr[] = {gc->r_proj, gc->r_stream, gc->r_off, gc->d_tiles, gc->d_goff, gc->d_scan, gc->d_tail,
+                              gc->d_tiles_order};
         put(gptr, sizeof(gptr));
         put(&gc->r_m_cap, sizeof(gc->r_m_cap));
         put(b->group_pos, sizeof(b->group_pos));
     }
     put(&flags, sizeof(flags));
     put(&c->device, sizeof(c->device));
-    put(&b->d_order, sizeof(b->d_order));
     if (!(b->gexec && b->gkey == key)) {
         if (b->gexec) {
             cudaGraphExecDestroy(b->gexec);

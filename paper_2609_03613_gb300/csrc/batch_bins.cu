@@ -237,7 +237,7 @@ struct GroupRows {
         const int y = row - gv.row_base[v], tx = gv.tiles_x[v], K = gv.K[v];
         return OffsetRow{D + gv.d_base[v] + (int64_t)y * (tx + 1), (int64_t)gv.tiles_y[v] * (tx + 1), tx, K,
                          gv.seg_base[v] + (int64_t)y * tx * K, gv.seg_base[v] + (int64_t)y * tx,
-                         (int64_t)tx * gv.tiles_y[v]};
+                         (int64_t)tx * gv.tiles_y[v], gv.tile_base[v] + y * tx};
     }
 };
 
@@ -258,6 +258,21 @@ k_group_cursors(const int32_t* __restrict__ off, const __grid_constant__ GroupVi
         while (v + 1 < gv.nv && gv.seg_base[v + 1] <= q) ++v;
         const int64_t l = q - gv.seg_base[v], t = l / gv.K[v], b = l - t * gv.K[v];
         cur[gv.seg_base[v] + b * gv.tiles_x[v] * gv.tiles_y[v] + t] = off[q];
+    }
+}
+
+// The tile order (OffsetsExtra), where no offsets pass wrote it.
+__global__ void __launch_bounds__(256)
+k_group_order(const int32_t* __restrict__ off, const __grid_constant__ GroupViews gv, int32_t* __restrict__ count,
+              int32_t* __restrict__ order)
+{
+    const int n = gv.tile_base[gv.nv];
+    int v = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        while (v + 1 < gv.nv && gv.tile_base[v + 1] <= i) ++v;
+        const int64_t q = gv.seg_base[v] + (int64_t)(i - gv.tile_base[v]) * gv.K[v];
+        const int b = 31 - __clz(off[q + gv.K[v]] - off[q] + 1);
+        order[(int64_t)b * n + atomicAdd(count + b, 1)] = i;
     }
 }
 
@@ -382,11 +397,14 @@ int group_reserve(gs_ctx* gc, const GroupViews* gvp, int64_t m_cap)
     gc->d_tiles = (int32_t*)tp;
     if ((r = goff_reserve(gc, N)) != GS_OK) return r;
     if ((r = scan_reserve(gc, N > NS ? N : NS)) != GS_OK) return r;
-    // ... and one flag word a tile row (the offsets' pass)
+    // ... and one flag word a tile row (the offsets' pass), its lists
+    if ((r = bins_reserve(gc, 1, NS)) != GS_OK) return r;
+    if ((r = tile_order_reserve(gc, gv.tile_base[gv.nv])) != GS_OK) return r;
     return ensure(&gc->d_scan, &gc->scan_bytes, ((size_t)gv.row_base[gv.nv] + 2) * sizeof(uint64_t));
 }
 
-int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m_views, cudaStream_t st)
+int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m_views, TileOrder* order,
+                  cudaStream_t st)
 {
     const GroupViews& gv = *gvp;
     const int64_t N = gv.n * gv.nv, NS = gv.seg_base[gv.nv];
@@ -441,15 +459,24 @@ int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m
     const unsigned g_sm = (unsigned)gc->num_sms * 8;
     const int n_rows = gv.row_base[gv.nv];
     gc->launches += 1;
-    if (osm <= kOffMaxSmem) {
+    GS_CUDA_TRY(cudaMemsetAsync(gc->d_tail, 0, kTailHead * 4, st));
+    const bool one_pass = osm <= kOffMaxSmem;
+    const int32_t min_len = raster_sort_cap(16) + 1;
+    if (one_pass) {
         // one pass over every view's tile rows, cursors included (prefixes, a
         // transposition, a scan, the over-capacity pass and a copy before:
         // 57 us of kernels for 16 views of 1M Gaussians; the scatter with its
         // cursors in segment order and four entries in flight 947 us)
         uint64_t* flags;
         if ((r = scan_flags(gc, n_rows, &flags, st)) != GS_OK) return r;
+        OffsetsExtra ex;
+        ex.long_list = gc->d_tail + kTailLong;
+        ex.min_len = min_len;
+        ex.count = gc->d_tail;
+        ex.order = gc->d_tiles_order;
+        ex.stride = gv.tile_base[gv.nv];
         GS_CUDA_TRY(launch_k(gc, k_bin_offsets<GroupRows>, (unsigned)n_rows, kOffThreads, osm, st, GroupRows{s.D, gv},
-                             n_rows, gc->r_m, gc->r_m_cap, flags, gc->d_scan_done, gc->r_off, s.cur, gc->d_err));
+                             n_rows, gc->r_m, gc->r_m_cap, flags, gc->d_scan_done, gc->r_off, s.cur, gc->d_err, ex));
         gc->launches += 1;
     } else {
         // a view's tile rows too wide for one block's shared memory
@@ -459,8 +486,12 @@ int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m
         if ((r = scan_impl(gc, LoadI32{s.cur}, NS, gc->r_off, nullptr, st)) != GS_OK) return r;
         k_zero_if_over<<<g_sm, 256, 0, st>>>(gc->r_m, gc->r_m_cap, gc->r_off, NS + 1, gc->d_err);
         k_group_cursors<<<g_sm, 256, 0, st>>>(gc->r_off, gv, s.cur);
-        gc->launches += 4;
+        k_group_order<<<g_sm, 256, 0, st>>>(gc->r_off, gv, gc->d_tail, gc->d_tiles_order);
+        gc->launches += 5;
     }
+    order->count = gc->d_tail;
+    order->lists = gc->d_tiles_order;
+    order->stride = gv.tile_base[gv.nv];
     // the scatter: every entry a slot in its view's (tile, bin) segment
     if (N > 0)
         k_group_scatter<<<g_sm * 2, 256, 0, st>>>(s.rs_g, s.rs_ya, s.rs_w, s.rs_z, roff, gv, gc->r_m, gc->r_m_cap,
@@ -468,7 +499,7 @@ int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m
     gc->launches += 1;
     GS_CUDA_TRY(cudaGetLastError());
     // segments longer than the raster sorts in shared memory
-    return sort_long_segments(gc, NS, gc->r_off, gc->r_stream, raster_sort_cap(16) + 1, st);
+    return sort_long_segments(gc, NS, gc->r_off, gc->r_stream, min_len, one_pass, st);
 }
 
 }  // namespace gs

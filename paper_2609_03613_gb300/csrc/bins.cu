@@ -245,7 +245,7 @@ int bins_reserve(gs_ctx* ctx, int64_t m_cap, int64_t nseg)
     if ((r = ensure(&p, &ctx->sel_cap, align256((size_t)nseg) + (size_t)(nseg + 1) * 8 + 256)) != GS_OK) return r;
     ctx->d_sel = (uint8_t*)p;
     p = ctx->d_tail;
-    if ((r = ensure(&p, &ctx->tail_cap, (size_t)(tail_capacity(nseg) + 1) * 4)) != GS_OK) return r;
+    if ((r = ensure(&p, &ctx->tail_cap, (size_t)(tail_capacity(nseg) + kTailHead) * 4)) != GS_OK) return r;
     ctx->d_tail = (int32_t*)p;
     return GS_OK;
 }
@@ -468,17 +468,15 @@ k_repair_tail(const int32_t* __restrict__ off, const int32_t* __restrict__ tail,
 }
 
 // EXACT with the repair in the raster: only segments of at least min_len
-// entries are sorted here.  A flat pass over the offsets lists them (one
-// thread per segment; most frames have none), then one block per listed
-// segment sorts it -- in shared memory when it fits, else in place.
+// entries are sorted here, one block a listed segment -- in shared memory when
+// it fits, else in place.  The list comes from the offsets' pass, or, where
+// there was none, from a flat pass over the offsets (one thread per segment).
 __global__ void k_list_long(const int32_t* __restrict__ off, int64_t nseg, int min_len, int32_t* __restrict__ list,
-                            int32_t cap, int* err, const ScatterPass sp, int K, const int32_t* __restrict__ flagged)
+                            int32_t cap, int* err)
 {
     grid_dependency_sync();
-    if (sp.pass == 2 && flagged[0] == 0) return;  // no tile to complete
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nseg; q += (int64_t)gridDim.x * blockDim.x) {
         if (off[q + 1] - off[q] < min_len) continue;
-        if (!sp.keep(q / K, (int)(q % K))) continue;
         const int slot = atomicAdd(&list[0], 1);
         if (slot < cap) list[1 + slot] = (int32_t)q;
         else raise_error(err, GS_ERR_CAPACITY);
@@ -502,14 +500,16 @@ constexpr int kSortBlocks = 3;  // an SM (70 KB of shared memory each)
 
 __global__ void __launch_bounds__(kSortThreads, kSortBlocks)
 k_sort_listed(const int32_t* __restrict__ off, const int32_t* __restrict__ list, int32_t cap,
-              uint64_t* __restrict__ words)
+              uint64_t* __restrict__ words, const ScatterPass sp, int K, const int32_t* __restrict__ flagged)
 {
     grid_dependency_sync();
+    if (sp.pass == 2 && flagged[0] == 0) return;  // no tile to complete
     extern __shared__ __align__(16) unsigned char sort_dyn[];
     SortShared& s = *reinterpret_cast<SortShared*>(sort_dyn);
     const int nl = min(list[0], cap);
     for (int k = blockIdx.x; k < nl; k += gridDim.x) {
         const int32_t q = list[1 + k];
+        if (!sp.keep(q / K, q % K)) continue;  // block-uniform
         const int l = off[q + 1] - off[q];
         uint64_t* seg = words + off[q];
         if (l <= kSortCap) {
@@ -549,21 +549,32 @@ __global__ void k_fill_selected(const int32_t* __restrict__ off, int64_t nseg, c
     }
 }
 
-int sort_long_segments(gs_ctx* ctx, int64_t nseg, const int32_t* offsets, uint64_t* words, int32_t min_len,
-                       cudaStream_t st)
+static int launch_long(gs_ctx* ctx, int64_t nseg, const int32_t* offsets, uint64_t* words, int32_t min_len, bool listed,
+                       const ScatterPass& sp, int K, cudaStream_t st)
 {
     if (nseg <= 0) return GS_OK;
-    int r;
     const int32_t tail_cap = tail_capacity(nseg);
-    if ((r = bins_reserve(ctx, 1, nseg)) != GS_OK) return r;
-    GS_CUDA_TRY(cudaMemsetAsync(ctx->d_tail, 0, 4, st));
-    const int64_t want = (nseg + 255) / 256, grid = (int64_t)ctx->num_sms * 8;
-    GS_CUDA_TRY(launch_k(ctx, k_list_long, (unsigned)(want < grid ? want : grid), 256, 0, st, offsets, nseg, min_len, ctx->d_tail, tail_cap,
-                                                                        ctx->d_err, ScatterPass(), 1, nullptr));
-    GS_CUDA_TRY(launch_k(ctx, k_sort_listed, (unsigned)ctx->num_sms * kSortBlocks, kSortThreads, sizeof(SortShared), st, offsets, ctx->d_tail, tail_cap, words));
-    ctx->launches += 2;
+    int32_t* list = ctx->d_tail + kTailLong;
+    if (!listed) {
+        GS_CUDA_TRY(cudaMemsetAsync(list, 0, 4, st));
+        const int64_t want = (nseg + 255) / 256, grid = (int64_t)ctx->num_sms * 8;
+        GS_CUDA_TRY(launch_k(ctx, k_list_long, (unsigned)(want < grid ? want : grid), 256, 0, st, offsets, nseg, min_len,
+                             list, tail_cap, ctx->d_err));
+        ctx->launches += 1;
+    }
+    GS_CUDA_TRY(launch_k(ctx, k_sort_listed, (unsigned)ctx->num_sms * kSortBlocks, kSortThreads, sizeof(SortShared), st,
+                         offsets, list, tail_cap, words, sp, K, sp.pass ? ctx->d_plist : nullptr));
+    ctx->launches += 1;
     GS_CUDA_TRY(cudaGetLastError());
     return GS_OK;
+}
+
+int sort_long_segments(gs_ctx* ctx, int64_t nseg, const int32_t* offsets, uint64_t* words, int32_t min_len, bool listed,
+                       cudaStream_t st)
+{
+    int r;
+    if (nseg > 0 && (r = bins_reserve(ctx, 1, nseg)) != GS_OK) return r;
+    return launch_long(ctx, nseg, offsets, words, min_len, listed, ScatterPass(), 1, st);
 }
 
 int repair(gs_ctx* ctx, int32_t n_tiles, const int64_t* m_dev, uint64_t* words, const int32_t* offsets,
@@ -573,7 +584,7 @@ int repair(gs_ctx* ctx, int32_t n_tiles, const int64_t* m_dev, uint64_t* words, 
 }
 
 int repair_min(gs_ctx* ctx, int32_t n_tiles, const int64_t* m_dev, uint64_t* words, const int32_t* offsets,
-               uint8_t* selected_out, int32_t min_len, cudaStream_t st, int pass)
+               uint8_t* selected_out, int32_t min_len, cudaStream_t st, int pass, bool listed)
 {
     const gs_config& c = ctx->cfg;
     const int64_t nseg = (int64_t)n_tiles * c.K;
@@ -600,29 +611,21 @@ int repair_min(gs_ctx* ctx, int32_t n_tiles, const int64_t* m_dev, uint64_t* wor
     }
     const int32_t tail_cap = tail_capacity(nseg);
     if ((r = bins_reserve(ctx, 1, nseg)) != GS_OK) return r;
-    if (!(ctx->zeroed_tail == ctx->d_tail && ctx->zeroed_tail_bytes == ctx->tail_cap))
-        GS_CUDA_TRY(cudaMemsetAsync(ctx->d_tail, 0, 4, st));
-    ctx->zeroed_tail = nullptr;  // zeroed by the frame's first kernel once, for this call
     if (c.mode == GS_MODE_BINNED_EXACT && min_len > kRpWarpCap) {
-        if (nseg > 0) {
-            const int64_t want = (nseg + 255) / 256;
-            const unsigned g = (unsigned)(want < (int64_t)grid ? want : (int64_t)grid);
-            ScatterPass sp;
-            if (pass) {
-                sp.plan = ctx->d_plan;
-                sp.T = n_tiles;
-                sp.pass = pass;
-            }
-            GS_CUDA_TRY(launch_k(ctx, k_list_long, g, 256, 0, st, offsets, nseg, min_len, ctx->d_tail, tail_cap, ctx->d_err, sp, c.K,
-                                           pass ? ctx->d_plist : nullptr));
-            GS_CUDA_TRY(launch_k(ctx, k_sort_listed, (unsigned)ctx->num_sms * kSortBlocks, kSortThreads, sizeof(SortShared), st, offsets, ctx->d_tail, tail_cap, words));
-            ctx->launches += 2;
+        ScatterPass sp;
+        if (pass) {
+            sp.plan = ctx->d_plan;
+            sp.T = n_tiles;
+            sp.pass = pass;
         }
-    } else if (n_tiles > 0)
-        k_repair_tiles<<<(unsigned)n_tiles, kRpThreads, 0, st>>>(offsets, c.K, sel, words, ctx->d_tail, tail_cap,
-                                                                 ctx->d_err, min_len);
-    if (!(c.mode == GS_MODE_BINNED_EXACT && min_len > kRpWarpCap)) {
-        k_repair_tail<<<(unsigned)ctx->num_sms, 1024, 0, st>>>(offsets, ctx->d_tail, tail_cap, words);
+        if ((r = launch_long(ctx, nseg, offsets, words, min_len, listed, sp, c.K, st)) != GS_OK) return r;
+    } else {
+        int32_t* list = ctx->d_tail + kTailLong;
+        GS_CUDA_TRY(cudaMemsetAsync(list, 0, 4, st));
+        if (n_tiles > 0)
+            k_repair_tiles<<<(unsigned)n_tiles, kRpThreads, 0, st>>>(offsets, c.K, sel, words, list, tail_cap,
+                                                                     ctx->d_err, min_len);
+        k_repair_tail<<<(unsigned)ctx->num_sms, 1024, 0, st>>>(offsets, list, tail_cap, words);
         ctx->launches += (n_tiles > 0 ? 2 : 1);
     }
     GS_CUDA_TRY(cudaGetLastError());

@@ -130,7 +130,6 @@ extern "C" int gs_create(gs_ctx** out, const gs_config* cfg)
     if (cudaMalloc(&c->d_err, sizeof(int)) != cudaSuccess) { delete c; return GS_ERR_NO_MEMORY; }
     cudaMemset(c->d_err, 0, sizeof(int));
     if (cudaMalloc(&c->d_bp, sizeof(BinParams)) != cudaSuccess) { gs_destroy(c); return GS_ERR_NO_MEMORY; }
-    if (cudaMalloc(&c->d_tile_counter, 64 * sizeof(int32_t)) != cudaSuccess) { gs_destroy(c); return GS_ERR_NO_MEMORY; }
     if (cudaMalloc(&c->r_m, 2 * sizeof(int64_t)) != cudaSuccess) { gs_destroy(c); return GS_ERR_NO_MEMORY; }
     if (cudaMalloc(&c->d_ops, sizeof(int64_t)) != cudaSuccess) { gs_destroy(c); return GS_ERR_NO_MEMORY; }
     if (cudaMalloc(&c->d_scan_done, sizeof(unsigned int)) != cudaSuccess) { gs_destroy(c); return GS_ERR_NO_MEMORY; }
@@ -166,7 +165,7 @@ extern "C" int gs_destroy(gs_ctx* c)
     }
     void* ptrs[] = {c->d_err, c->d_scan, c->d_goff, c->d_keys[0], c->d_keys[1], c->d_vals[0],
                     c->d_vals[1], c->d_hist, c->d_count, c->d_bin, c->d_bp, c->d_sel, c->d_tail,
-                    c->d_tiles_order, c->d_tile_counter, c->r_proj, c->r_isect, c->r_stream,
+                    c->d_tiles_order, c->r_proj, c->r_isect, c->r_stream,
                     c->r_off, c->r_m, c->r_scene, c->r_out, c->d_ops, c->d_tiles, c->d_samples,
                     c->r_T, c->r_tend, c->r_wend, c->d_planner, c->d_feat, c->d_plan, c->d_plist,
                     c->d_order_ws, c->d_scan_done};
@@ -402,12 +401,14 @@ extern "C" int gs_sort_or_bin(gs_ctx* ctx, const void* projected, const float* s
         GS_CUDA_TRY(cudaMemcpyAsync(zrange_out, ctx->d_bp, 2 * sizeof(float), cudaMemcpyDeviceToDevice, st));
     if (ctx->cfg.mode == GS_MODE_BINNED_EXACT) {
         stage_begin(ctx, GS_STAGE_BIN, st);
-        r = exact_bins(ctx, pv, n, cam, false, m_cap, m_dev, stream_words, offsets, st);
+        const int32_t min_len = ctx->cfg.repair_in_raster ? raster_sort_cap(ctx->cfg.tile_size) + 1 : 2;
+        bool listed;
+        r = exact_bins(ctx, pv, n, cam, false, m_cap, m_dev, stream_words, offsets, st,
+                       ctx->cfg.repair_in_raster ? min_len : 0, &listed);
         stage_end(ctx, GS_STAGE_BIN, st);
         if (r != GS_OK) return r;
         stage_begin(ctx, GS_STAGE_REPAIR, st);
-        r = repair_min(ctx, T, m_dev, stream_words, offsets, nullptr,
-                       ctx->cfg.repair_in_raster ? raster_sort_cap(ctx->cfg.tile_size) + 1 : 2, st);
+        r = repair_min(ctx, T, m_dev, stream_words, offsets, nullptr, min_len, st, 0, listed);
         stage_end(ctx, GS_STAGE_REPAIR, st);
         return r;
     }
@@ -623,12 +624,15 @@ int gs::render_binning(gs_ctx* c, int64_t n, const float* scales, const gs_camer
             if ((r = planner_buffers(c, T)) != GS_OK) return r;
         }
         stage_begin(c, GS_STAGE_BIN, st);
-        r = exact_bins(c, pv, n, cam, true, c->r_m_cap, c->r_m, c->r_stream, c->r_off, st, rows, planned);
+        const int32_t min_len = c->cfg.repair_in_raster ? raster_sort_cap(c->cfg.tile_size) + 1 : 2;
+        bool listed;
+        r = exact_bins(c, pv, n, cam, true, c->r_m_cap, c->r_m, c->r_stream, c->r_off, st,
+                       c->cfg.repair_in_raster ? min_len : 0, &listed, rows, planned);
+        c->long_listed = listed;
         stage_end(c, GS_STAGE_BIN, st);
         if (r != GS_OK) return r;
         stage_begin(c, GS_STAGE_REPAIR, st);
-        r = repair_min(c, T, c->r_m, c->r_stream, c->r_off, nullptr,
-                       c->cfg.repair_in_raster ? raster_sort_cap(c->cfg.tile_size) + 1 : 2, st, planned ? 1 : 0);
+        r = repair_min(c, T, c->r_m, c->r_stream, c->r_off, nullptr, min_len, st, planned ? 1 : 0, listed);
         stage_end(c, GS_STAGE_REPAIR, st);
     } else {
         r = emit_only(c, pv, n, cam, isect_view(c->r_isect, c->r_m_cap), c->r_m_cap, c->r_m, st);
@@ -664,7 +668,8 @@ int gs::render_after_project(gs_ctx* c, int64_t n, const float* scales, const gs
     // resumes pixels whose stops it does not know: tile ends only)
     int32_t* wend = save && !planned ? c->r_wend : nullptr;
     r = raster_fwd(c, pv, cam, c->r_stream, c->r_off, stride, bg, d_rgb, d_alpha, d_last, nullptr,
-                   st, save ? c->r_T : nullptr, save ? c->r_tend : nullptr, pl, wend);
+                   st, save ? c->r_T : nullptr, save ? c->r_tend : nullptr, pl, wend,
+                   c->cfg.mode == GS_MODE_BINNED_EXACT && c->tile_ordered ? frame_tile_order(c, T) : TileOrder());
     stage_end(c, GS_STAGE_RASTER, st);
     if (r != GS_OK) return r;
     if (planned) {
@@ -672,7 +677,8 @@ int gs::render_after_project(gs_ctx* c, int64_t n, const float* scales, const gs
         // segments sorted, the tiles composited on from where they stopped
         stage_begin(c, GS_STAGE_COMPLETE, st);
         r = exact_scatter_rest(c, n, cam, c->r_m_cap, c->r_m, c->r_stream, c->r_off, st);
-        if (r == GS_OK) r = repair_min(c, T, c->r_m, c->r_stream, c->r_off, nullptr, raster_sort_cap(c->cfg.tile_size) + 1, st, 2);
+        if (r == GS_OK) r = repair_min(c, T, c->r_m, c->r_stream, c->r_off, nullptr, raster_sort_cap(c->cfg.tile_size) + 1, st, 2,
+                                       c->long_listed != 0);
         if (r == GS_OK)
             r = raster_listed(c, pv, cam, c->r_stream, c->r_off, stride, bg, d_rgb, d_alpha, d_last, c->d_plan,
                               c->d_plist, st, save ? c->r_T : nullptr, save ? c->r_tend : nullptr);
@@ -903,7 +909,7 @@ extern "C" int gs_render(gs_ctx* c, const gs_scene* sc, const gs_camera* cam, co
         int timing, device, flags;
         // the internal scratch the captured kernels address (a grown buffer
         // is a new allocation: the graph is captured again)
-        const void* scratch[14];
+        const void* scratch[15];
         size_t scratch_bytes[10];
     } key;
     if (flags & GS_RENDER_SAVE) {
@@ -935,7 +941,7 @@ extern "C" int gs_render(gs_ctx* c, const gs_scene* sc, const gs_camera* cam, co
     key.saved_wend = c->r_wend;
     const void* scratch[] = {c->d_scan, c->d_goff, c->d_keys[0], c->d_keys[1], c->d_vals[0], c->d_vals[1],
                              c->d_hist, c->d_count, c->d_bin, c->d_sel, c->d_tail, c->d_tiles, c->d_samples,
-                             c->d_plan};
+                             c->d_plan, c->d_tiles_order};
     const size_t scratch_bytes[] = {c->scan_bytes, c->goff_cap, c->sort_cap, c->hist_cap, c->count_cap,
                                     c->bin_cap, c->sel_cap, c->tail_cap, c->tiles_cap, c->samples_cap};
     static_assert(sizeof(scratch) == sizeof(key.scratch) && sizeof(scratch_bytes) == sizeof(key.scratch_bytes),

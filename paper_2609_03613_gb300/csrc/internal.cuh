@@ -229,8 +229,8 @@ struct gs_ctx {
     // (scan_arena_bytes): a grown buffer is a new one.
     int64_t scan_arena = 0, scan_used = 0;
     size_t scan_arena_bytes = 0;
-    // the same for the EXACT bin stage's difference counts and the repair's
-    // long-segment counter: the zeroed pointer and its buffer's size then
+    // the same for the EXACT bin stage's difference counts and the counters of
+    // d_tail: the zeroed pointer and its buffer's size then
     int32_t* zeroed_D = nullptr;
     size_t zeroed_D_bytes = 0;
     int32_t* zeroed_tail = nullptr;
@@ -257,14 +257,13 @@ struct gs_ctx {
     gs::BinParams* d_bp = nullptr;
     uint8_t* d_sel = nullptr;    // per-segment repair selection
     size_t sel_cap = 0;
-    int32_t* d_tail = nullptr;   // segments too long for a shared-memory sort
+    int32_t* d_tail = nullptr;   // kTailHead counters, then the segments too long for a shared-memory sort
     size_t tail_cap = 0;
     int32_t* d_tiles = nullptr;   // tile-count difference grid, tile offsets, cursors
     size_t tiles_cap = 0;
     uint32_t* d_samples = nullptr; // depth-range samples (their keys as float bits)
     size_t samples_cap = 0;
-    int32_t* d_tiles_order = nullptr;  // persistent raster tile order
-    int32_t* d_tile_counter = nullptr;
+    int32_t* d_tiles_order = nullptr;  // the raster's tiles by span length (gs::TileOrder)
     size_t order_cap = 0;
     // whole-frame buffers (gs_render)
     void* r_proj = nullptr; size_t r_proj_cap = 0;
@@ -314,6 +313,8 @@ struct gs_ctx {
     float* d_feat = nullptr; size_t feat_cap = 0;
     uint8_t* d_plan = nullptr; size_t plan_cap_bytes = 0;  // [T] first-pass bins, [T] completion flags, [T] row flags
     int32_t* d_plist = nullptr; size_t plist_cap = 0;      // [1 + T]: count, then the flagged tiles
+    // what the last whole frame's offsets pass wrote: its long segments, its tile order
+    int long_listed = 0, tile_ordered = 0;
     int32_t* exact_roff = nullptr;  // row-record offsets of the last planned frame's bin construction
     // batched multi-view rendering (gs_render_batch)
     gs::BatchState* batch = nullptr;
@@ -395,6 +396,30 @@ inline bool frame_planned(const gs_ctx* c)
     return c->cfg.planner && c->cfg.mode == GS_MODE_BINNED_EXACT && c->cfg.repair_in_raster && c->cfg.tile_cull;
 }
 
+// The tiles of a frame (or of a batch's views) from the longest spans to the
+// shortest, so that the raster's last blocks are the short ones: 32 lists by
+// floor(log2(span + 1)), list b at lists + b stride with count[b] tiles.
+// Filled by the offsets' pass; which tile of a list comes first is open.
+constexpr int kTileLists = 32;
+struct TileOrder {
+    const int32_t* count = nullptr;
+    const int32_t* lists = nullptr;
+    int64_t stride = 0;
+};
+// The counters at the head of gs_ctx::d_tail: TileOrder's counts, the batched
+// raster's work counter, the number of long segments (the list follows it).
+constexpr int kTailWork = kTileLists, kTailLong = kTileLists + 1, kTailHead = kTileLists + 2;
+// What the offsets' pass also writes: the segments of at least min_len
+// entries (long_list = {count, segments...}; min_len 0: none) and the tile
+// order (order null: none).
+struct OffsetsExtra {
+    int32_t* long_list = nullptr;
+    int32_t min_len = 0;
+    int32_t* count = nullptr;
+    int32_t* order = nullptr;
+    int64_t stride = 0;
+};
+
 int ensure(void** p, size_t* cap, size_t bytes);
 int check_config(const gs_config* cfg);
 
@@ -441,13 +466,16 @@ int launch_depth_range_into(const gs_config& c, const ProjView& pv, const float*
 // counts and the expansion, which needs ctx->d_goff -- computed here unless
 // goff_ready).  Segments are left unsorted.
 // rows_ready: count_rows_scan has also written the row-record offsets.
+// long_min: segments of at least that many entries are listed on the way where
+// the path's offsets come from one pass (*long_listed), which on a whole frame
+// also orders its tiles for the raster (frame_tile_order).
 // With planned (the tile cull on): after the counts, the bin planner sets
 // each tile's first-pass bins (plan_frame) and only entries of those bins are
 // scattered; exact_scatter_rest then places the other entries of the tiles
 // the first raster pass flagged.
 int exact_bins(gs_ctx* ctx, const ProjView& pv, int64_t n, const gs_camera* cam, bool goff_ready, int64_t m_cap,
-               const int64_t* m_dev, uint64_t* words, int32_t* offsets, cudaStream_t st, bool rows_ready = false,
-               bool planned = false);
+               const int64_t* m_dev, uint64_t* words, int32_t* offsets, cudaStream_t st, int32_t long_min,
+               bool* long_listed, bool rows_ready = false, bool planned = false);
 int exact_scatter_rest(gs_ctx* ctx, int64_t n, const gs_camera* cam, int64_t m_cap, const int64_t* m_dev,
                        uint64_t* words, const int32_t* offsets, cudaStream_t st);
 // the regions of a tile-cull EXACT frame that its projection zeroes (tiles.cu)
@@ -462,11 +490,18 @@ int64_t group_scan_items(gs_ctx* ctx, int32_t tiles_y, int K);
 // frame's first pass (bins below ctx->d_plan) or of its completing pass (the
 // other bins of flagged tiles); 0: every segment
 int repair_min(gs_ctx* ctx, int32_t n_tiles, const int64_t* m_dev, uint64_t* stream_words, const int32_t* offsets,
-               uint8_t* selected_out, int32_t min_len, cudaStream_t st, int pass = 0);
+               uint8_t* selected_out, int32_t min_len, cudaStream_t st, int pass = 0, bool listed = false);
+// the frame's tile order, when its tiles outnumber what the raster holds at
+// once and the offsets' pass wrote it (else empty)
+TileOrder frame_tile_order(const gs_ctx* ctx, int64_t T);
+int tile_order_reserve(gs_ctx* ctx, int64_t T);
+// whether all T tiles of that size are resident at once in the raster
+bool raster_resident(const gs_ctx* ctx, int tile, int64_t T);
 // sort every segment of a flat segment array [nseg] longer than min_len - 1
-// entries (the segments the raster cannot sort in shared memory)
+// entries (the segments the raster cannot sort in shared memory); listed: the
+// offsets' pass has listed them
 int sort_long_segments(gs_ctx* ctx, int64_t nseg, const int32_t* offsets, uint64_t* words, int32_t min_len,
-                       cudaStream_t st);
+                       bool listed, cudaStream_t st);
 // segments longer than this are sorted before the raster when the raster
 // sorts the segments it reaches (8 x 8 tiles: a smaller buffer, so that more
 // of their one-warp blocks fit an SM)
@@ -540,7 +575,8 @@ int depth_range_goff(gs_ctx* ctx, const ProjView& pv, const float* scales, int64
 int raster_fwd(gs_ctx* ctx, const ProjView& pv, const gs_camera* cam, uint64_t* stream_words,
                const int32_t* offsets, int32_t stride, const float* bg, float* rgb, float* alpha,
                int32_t* last, int32_t* ntests, cudaStream_t st, float* final_T = nullptr,
-               int32_t* tile_end = nullptr, const PlanView& plan = PlanView(), int32_t* warp_end = nullptr);
+               int32_t* tile_end = nullptr, const PlanView& plan = PlanView(), int32_t* warp_end = nullptr,
+               const TileOrder& order = TileOrder());
 // the completing pass of a planned frame: every tile of list (device {count,
 // tiles...}) composited on from the bin where its first pass stopped (plan
 // [T]), from the pixel state that pass left in rgb / alpha / last (EXACT,
@@ -565,9 +601,10 @@ struct RasterView {
     int32_t* last;
     int32_t gid_base;  // stream words hold gid_base + the view's gid (a batch group's shared records)
 };
-// all views' tiles in one persistent launch, longest tiles first
-// (sched: 65 device int32; order: one int32 per tile of all views)
-int raster_views(gs_ctx* ctx, const RasterView* views, int nv, int32_t* sched, int32_t* order, cudaStream_t st);
+// all views' tiles in one persistent launch, longest tiles first (order: the
+// tiles of all views, numbered view by view; work: a zeroed device counter)
+int raster_views(gs_ctx* ctx, const RasterView* views, int nv, const TileOrder& order, int32_t* work,
+                 cudaStream_t st);
 
 // raster_bwd.cu
 int raster_bwd_prepare();
@@ -619,7 +656,10 @@ int group_reserve(gs_ctx* gc, const GroupViews* gv, int64_t m_cap);
 // intersect, depth range, bins and the long-segment sort of every view of the
 // group (stream and offsets in gc->r_stream, gc->r_off); per-view entry
 // counts copied to the pinned host array h_m_views [nv]
-int group_binning(gs_ctx* gc, const GroupViews* gv, int32_t flags, int64_t* h_m_views, cudaStream_t st);
+// (the tile order and the zeroed work counter of raster_views in gc->d_tail and
+// gc->d_tiles_order)
+int group_binning(gs_ctx* gc, const GroupViews* gv, int32_t flags, int64_t* h_m_views, TileOrder* order,
+                  cudaStream_t st);
 
 // batch.cu: per-context batch state (sub-contexts, streams, graph)
 struct BatchState;

@@ -14,7 +14,10 @@ namespace gs {
 // by decoupled look-back over the rows' published totals (bounded waits),
 // and writes offsets and, when given, the scatter cursors.  Over capacity
 // (or past INT32_MAX) every offset is written 0 and GS_ERR_CAPACITY raised,
-// so nothing downstream reads out of bounds.  Replaces a per-layer prefix,
+// so nothing downstream reads out of bounds.  On the way it lists the long
+// segments and orders the tiles by span (OffsetsExtra): a pass over all the
+// offsets and its launch less each (5 us at 1080p; the batch's three ordering
+// kernels took 43 us).  Replaces a per-layer prefix,
 // a transposition, a device-wide scan and the over-capacity pass.
 constexpr int kOffThreads = 1024;
 constexpr size_t kOffMaxSmem = 160 * 1024;
@@ -28,13 +31,14 @@ struct OffsetRow {
     int64_t layer;
     int tiles_x, K;
     int64_t seg, cur, cur_bin;
+    int32_t tile;  // its first tile
 };
 
 // Rows: OffsetRow of row y (0 <= y < n_rows, in segment order).
 template <class Rows>
 __global__ void __launch_bounds__(kOffThreads)
 k_bin_offsets(const __grid_constant__ Rows rows, int n_rows, const int64_t* __restrict__ m_dev, int64_t m_cap,
-              uint64_t* flags, unsigned int* ticket, int32_t* __restrict__ off, int32_t* __restrict__ cur, int* err)
+              uint64_t* flags, unsigned int* ticket, int32_t* __restrict__ off, int32_t* __restrict__ cur, int* err, const OffsetsExtra ex)
 {
     grid_dependency_sync();
     extern __shared__ int32_t s_c[];  // [tiles_x][K + 1]: counts, then exclusive offsets in the row
@@ -129,7 +133,18 @@ k_bin_offsets(const __grid_constant__ Rows rows, int n_rows, const int64_t* __re
         const int x = j / K, b = j - x * K;
         const int32_t v = over ? 0 : (int32_t)(pre + s_c[x * KP + b]);
         off[rw.seg + j] = v;
+        if (ex.min_len > 0 && !over) {
+            const int32_t end = b + 1 < K ? s_c[x * KP + b + 1] : (x + 1 < tiles_x ? s_c[(x + 1) * KP] : (int32_t)total);
+            if (end - s_c[x * KP + b] >= ex.min_len)
+                ex.long_list[1 + atomicAdd(ex.long_list, 1)] = (int32_t)(rw.seg + j);
+        }
     }
+    if (ex.order)
+        for (int x = threadIdx.x; x < tiles_x; x += kOffThreads) {
+            const int32_t n = over ? 0 : (x + 1 < tiles_x ? s_c[(x + 1) * KP] : (int32_t)total) - s_c[x * KP];
+            const int q = 31 - __clz(n + 1);
+            ex.order[q * ex.stride + atomicAdd(ex.count + q, 1)] = rw.tile + x;
+        }
     if (cur) {  // bin by bin, tiles inside
         for (int j = threadIdx.x; j < items; j += kOffThreads) {
             const int b = j / tiles_x, x = j - b * tiles_x;

@@ -464,6 +464,24 @@ __device__ __forceinline__ void raster_tile(
     }
 }
 
+// The k-th tile of the order (warp-uniform k; -1: there is none).  Whole warp.
+__device__ __forceinline__ int ordered_tile(const TileOrder& o, int32_t k)
+{
+    const int q = kTileLists - 1 - (int)(threadIdx.x & 31);  // longest first
+    const int32_t c = o.count[q];
+    int32_t incl = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int32_t u = __shfl_up_sync(0xffffffffu, incl, d);
+        if ((int)(threadIdx.x & 31) >= d) incl += u;
+    }
+    const unsigned past = __ballot_sync(0xffffffffu, incl > k);
+    if (past == 0u) return -1;
+    const int l = __ffs(past) - 1;
+    const int32_t at = k - __shfl_sync(0xffffffffu, incl - c, l);
+    return o.lists[(kTileLists - 1 - l) * o.stride + at];
+}
+
 // Threads of a tile's block and the blocks an SM holds: 16 x 16 tiles' seven
 // blocks of 128 threads fill the shared memory (31.8 KB each).
 template <int TILE>
@@ -481,12 +499,14 @@ k_raster(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o_z, con
          uint64_t* words, const int32_t* __restrict__ off, RasterArgs a, int cullmode,
          float* __restrict__ out_rgb, float* __restrict__ out_alpha, int32_t* __restrict__ out_last,
          int32_t* __restrict__ out_ntests, unsigned long long* __restrict__ ops_total, float* __restrict__ out_T,
-         int32_t* __restrict__ out_end, const PlanView pl, int cap, int32_t* __restrict__ out_wend)
+         int32_t* __restrict__ out_end, const PlanView pl, int cap, int32_t* __restrict__ out_wend, const TileOrder ord)
 {
     grid_dependency_sync();
     __shared__ RasterShared<TILE> sh;
     __shared__ WalkShared<TILE, LAZY> ws;
-    raster_tile<TILE, COUNT, LAZY, R>(blockIdx.x, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode, out_rgb, out_alpha,
+    const int t = ord.lists ? ordered_tile(ord, (int32_t)blockIdx.x) : (int)blockIdx.x;
+    if (t < 0) return;
+    raster_tile<TILE, COUNT, LAZY, R>(t, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode, out_rgb, out_alpha,
                                    out_last, out_ntests, ops_total, out_T, out_end, pl, cap, out_wend);
 }
 
@@ -517,7 +537,7 @@ k_raster_listed(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o
 }
 
 // Several views in one persistent launch: blocks take (view, tile) work items
-// from a counter, in view order, until all views' tiles are composited.
+// from a counter, longest tiles first, until all views' tiles are composited.
 struct ViewRasterSet {
     struct View {
         const float4* xy_ab;
@@ -543,57 +563,24 @@ __device__ __forceinline__ int view_of(const ViewRasterSet& vs, int32_t item)
     return v;
 }
 
-// Longest tiles first: work items bucketed by floor(log2(span + 1)), buckets
-// handed out from the longest (so the last items of the persistent launch are
-// the short ones).  sched: [0..32) bucket counts, [32..64) cursors.
-__global__ void k_view_buckets(const __grid_constant__ ViewRasterSet vs, int32_t* __restrict__ sched)
-{
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < vs.total; i += gridDim.x * blockDim.x) {
-        const ViewRasterSet::View& V = vs.v[view_of(vs, i)];
-        const int64_t t = i - V.item0;
-        const int32_t len = V.off[(t + 1) * V.a.stride] - V.off[t * V.a.stride];
-        atomicAdd(&sched[31 - __clz(len + 1)], 1);
-    }
-}
-
-__global__ void k_view_bucket_starts(int32_t* __restrict__ sched)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int32_t run = 0;
-    for (int b = 31; b >= 0; --b) {
-        sched[32 + b] = run;
-        run += sched[b];
-    }
-}
-
-__global__ void k_view_order(const __grid_constant__ ViewRasterSet vs, int32_t* __restrict__ sched,
-                             int32_t* __restrict__ order)
-{
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < vs.total; i += gridDim.x * blockDim.x) {
-        const ViewRasterSet::View& V = vs.v[view_of(vs, i)];
-        const int64_t t = i - V.item0;
-        const int32_t len = V.off[(t + 1) * V.a.stride] - V.off[t * V.a.stride];
-        order[atomicAdd(&sched[32 + 31 - __clz(len + 1)], 1)] = i;
-    }
-}
-
 template <int TILE, bool LAZY>
 __global__ void __launch_bounds__(raster_threads<TILE>(), raster_min_blocks<TILE>())
-k_raster_views(const __grid_constant__ ViewRasterSet vs, const int32_t* __restrict__ order,
-               int32_t* __restrict__ counter)
+k_raster_views(const __grid_constant__ ViewRasterSet vs, const TileOrder order, int32_t* __restrict__ counter)
 {
     __shared__ RasterShared<TILE> sh;
     __shared__ WalkShared<TILE, LAZY> ws;
     __shared__ int32_t s_item;
     for (;;) {
-        if (threadIdx.x == 0) {
-            const int32_t k = atomicAdd(counter, 1);
-            s_item = k < vs.total ? order[k] : vs.total;
+        if (threadIdx.x < 32) {
+            int32_t k = 0;
+            if (threadIdx.x == 0) k = atomicAdd(counter, 1);
+            const int t = ordered_tile(order, __shfl_sync(0xffffffffu, k, 0));
+            if (threadIdx.x == 0) s_item = t;
         }
         __syncthreads();  // also: every thread is done with the previous tile's shared memory
         const int32_t item = s_item;
         __syncthreads();
-        if (item >= vs.total) break;
+        if (item < 0) break;
         const ViewRasterSet::View& V = vs.v[view_of(vs, item)];
         raster_tile<TILE, false, LAZY, 2>(item - V.item0, sh, ws, V.xy_ab, V.c_o_z, V.rgbv, V.words, V.off, V.a,
                                               V.cullmode, V.rgb, V.alpha, V.last, nullptr, nullptr, nullptr, nullptr,
@@ -602,10 +589,22 @@ k_raster_views(const __grid_constant__ ViewRasterSet vs, const int32_t* __restri
 }
 
 template <int TILE>
+static bool resident(const gs_ctx* ctx, int64_t T)
+{
+    return T <= (int64_t)ctx->num_sms * raster_wide_blocks<TILE>();
+}
+
+bool raster_resident(const gs_ctx* ctx, int tile, int64_t T)
+{
+    return tile == 8 ? resident<8>(ctx, T) : tile == 32 ? resident<32>(ctx, T) : resident<16>(ctx, T);
+}
+
+template <int TILE>
 static cudaError_t launch_tile(const gs_ctx* ctx, bool count, bool lazy, unsigned grid, cudaStream_t st,
                                const ProjView& pv, uint64_t* words, const int32_t* off, const RasterArgs& a, int cull,
                                float* rgb, float* alpha, int32_t* last, int32_t* ntests, unsigned long long* ops,
-                               float* final_T, int32_t* tile_end, const PlanView& pl, int cap, int32_t* warp_end)
+                               float* final_T, int32_t* tile_end, const PlanView& pl, int cap, int32_t* warp_end,
+                               const TileOrder& order)
 {
     // Rounds of four when all the frame's tiles are resident at once (each
     // SM's few warps wait for their own results, and a wide round has twice as
@@ -614,19 +613,19 @@ static cudaError_t launch_tile(const gs_ctx* ctx, bool count, bool lazy, unsigne
     // an SM instead of four (8160 tiles: 229 us against 244; 3600 tiles, global:
     // 276 against 331).  8 x 8 tiles have one warp a block, as many blocks
     // either way, and always go by four (2646 tiles: 63.4 us against 69.5).
-    const bool wide = TILE == 8 || grid <= (unsigned)(ctx->num_sms * raster_wide_blocks<TILE>());
+    const bool wide = TILE == 8 || raster_resident(ctx, TILE, grid);
     constexpr int RN = TILE == 8 ? 4 : 2;
     const auto kern = count  ? (lazy ? k_raster<TILE, true, true, RN> : k_raster<TILE, true, false, RN>)
                       : wide ? (lazy ? k_raster<TILE, false, true, 4> : k_raster<TILE, false, false, 4>)
                              : (lazy ? k_raster<TILE, false, true, RN> : k_raster<TILE, false, false, RN>);
     return launch_k(ctx, kern, grid, raster_threads<TILE>(), 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, off, a, cull,
-                    rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end);
+                    rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end, order);
 }
 
 int raster_fwd(gs_ctx* ctx, const ProjView& pv, const gs_camera* cam, uint64_t* words,
                const int32_t* offsets, int32_t stride, const float* bg, float* rgb, float* alpha,
                int32_t* last, int32_t* ntests, cudaStream_t st, float* final_T, int32_t* tile_end,
-               const PlanView& pl, int32_t* warp_end)
+               const PlanView& pl, int32_t* warp_end, const TileOrder& order)
 {
     const int tile = ctx->cfg.tile_size;
     RasterArgs a;
@@ -653,9 +652,9 @@ int raster_fwd(gs_ctx* ctx, const ProjView& pv, const gs_camera* cam, uint64_t* 
     if (count) GS_CUDA_TRY(cudaMemsetAsync(ops, 0, sizeof(unsigned long long), st));
     cudaError_t e;
     switch (tile) {
-        case 8: e = launch_tile<8>(ctx, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end); break;
-        case 32: e = launch_tile<32>(ctx, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end); break;
-        default: e = launch_tile<16>(ctx, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end); break;
+        case 8: e = launch_tile<8>(ctx, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end, order); break;
+        case 32: e = launch_tile<32>(ctx, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end, order); break;
+        default: e = launch_tile<16>(ctx, count, lazy, grid, st, pv, words, offsets, a, cull_here, rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end, order); break;
     }
     GS_CUDA_TRY(e);
     ctx->launches += 1;
@@ -691,7 +690,7 @@ int raster_listed(gs_ctx* ctx, const ProjView& pv, const gs_camera* cam, uint64_
     return GS_OK;
 }
 
-int raster_views(gs_ctx* ctx, const RasterView* views, int nv, int32_t* sched, int32_t* order, cudaStream_t st)
+int raster_views(gs_ctx* ctx, const RasterView* views, int nv, const TileOrder& order, int32_t* work, cudaStream_t st)
 {
     if (nv < 1 || nv > kMaxBatchViews) return GS_ERR_INVALID_ARG;
     ViewRasterSet vs;
@@ -726,16 +725,10 @@ int raster_views(gs_ctx* ctx, const RasterView* views, int nv, int32_t* sched, i
     vs.nviews = nv;
     vs.total = total;
     if (total == 0) return GS_OK;
-    // sched: [0..32) bucket counts, [32..64) bucket cursors, [64] work counter
-    GS_CUDA_TRY(cudaMemsetAsync(sched, 0, 65 * sizeof(int32_t), st));
-    const unsigned gi = (unsigned)((total + 255) / 256 < ctx->num_sms * 4 ? (total + 255) / 256 : ctx->num_sms * 4);
-    k_view_buckets<<<gi, 256, 0, st>>>(vs, sched);
-    k_view_bucket_starts<<<1, 32, 0, st>>>(sched);
-    k_view_order<<<gi, 256, 0, st>>>(vs, sched, order);
-    const int resident = ctx->num_sms * raster_min_blocks<16>();
-    const unsigned grid = (unsigned)(resident < total ? resident : total);
-    k_raster_views<16, true><<<grid, raster_threads<16>(), 0, st>>>(vs, order, sched + 64);
-    ctx->launches += 4;
+    const int held = ctx->num_sms * raster_min_blocks<16>();
+    const unsigned grid = (unsigned)(held < total ? held : total);
+    k_raster_views<16, true><<<grid, raster_threads<16>(), 0, st>>>(vs, order, work);
+    ctx->launches += 1;
     GS_CUDA_TRY(cudaGetLastError());
     return GS_OK;
 }

@@ -451,7 +451,7 @@ struct FrameRows {
     __device__ __forceinline__ OffsetRow operator()(int y) const
     {
         return OffsetRow{D + (int64_t)y * (tiles_x + 1), layer, tiles_x, K, (int64_t)y * tiles_x * K,
-                         (int64_t)y * tiles_x, (int64_t)tiles_x * tiles_y};
+                         (int64_t)y * tiles_x, (int64_t)tiles_x * tiles_y, y * tiles_x};
     }
 };
 
@@ -602,8 +602,7 @@ static int exact_scatter(gs_ctx* ctx, const ExactScratch& v, int64_t n, int32_t 
 // The regions a frame of the tile-cull EXACT path needs zeroed, so that no
 // memset sits between its kernels: the frame's scan-flag arena (the row-count
 // scan, the offsets scan and, on deep frames, the grouped scatter's count
-// scan), the bin stage's difference counts, the repair's long-segment
-// counter.  The projection (*fz) clears the row-count scan's flags, the
+// scan), the bin stage's difference counts, the counters of d_tail.  The projection (*fz) clears the row-count scan's flags, the
 // depth-range sampling (ctx->late_*) the rest.  Reserves the scratch they
 // live in.
 int exact_frame_zero(gs_ctx* ctx, int64_t n, const gs_camera* cam, int64_t m_cap, FrameZero* fz)
@@ -614,6 +613,7 @@ int exact_frame_zero(gs_ctx* ctx, int64_t n, const gs_camera* cam, int64_t m_cap
     int r;
     if ((r = exact_bins_reserve(ctx, n, m_cap, tiles_x, tiles_y, K)) != GS_OK) return r;
     if ((r = bins_reserve(ctx, 1, nseg)) != GS_OK) return r;
+    if (!ctx->capturing && !raster_resident(ctx, tile, T) && (r = tile_order_reserve(ctx, T)) != GS_OK) return r;
     ExactScratch v;
     exact_scratch(ctx, n, m_cap, tiles_x, tiles_y, K, &v);
     auto blocks = [](int64_t items) { return items > 0 ? (items + kScanTile - 1) / kScanTile : 1; };
@@ -632,7 +632,7 @@ int exact_frame_zero(gs_ctx* ctx, int64_t n, const gs_camera* cam, int64_t m_cap
     ctx->late_p[1] = static_cast<int32_t*>(ctx->d_scan) + 2 * w2;
     ctx->late_n[1] = 2 * (words - w2);
     ctx->late_p[2] = ctx->d_tail;
-    ctx->late_n[2] = 1;
+    ctx->late_n[2] = kTailHead;
     ctx->scan_arena = words;
     ctx->scan_used = 0;
     ctx->scan_arena_bytes = ctx->scan_bytes;
@@ -668,10 +668,31 @@ int exact_scatter_rest(gs_ctx* ctx, int64_t n, const gs_camera* cam, int64_t m_c
     return exact_scatter(ctx, v, n, tiles_x, tiles_y, K, m_cap, m_dev, words, offsets, sp, st);
 }
 
-int exact_bins(gs_ctx* ctx, const ProjView& pv, int64_t n, const gs_camera* cam, bool goff_ready, int64_t m_cap,
-               const int64_t* m_dev, uint64_t* words, int32_t* offsets, cudaStream_t st, bool rows_ready,
-               bool planned)
+// The frame's long segments and tile order go to d_tail and d_tiles_order.
+TileOrder frame_tile_order(const gs_ctx* ctx, int64_t T)
 {
+    TileOrder o;
+    if (raster_resident(ctx, ctx->cfg.tile_size, T) || ctx->order_cap < (size_t)T * kTileLists * 4) return o;
+    o.count = ctx->d_tail;
+    o.lists = ctx->d_tiles_order;
+    o.stride = T;
+    return o;
+}
+
+int tile_order_reserve(gs_ctx* ctx, int64_t T)
+{
+    void* p = ctx->d_tiles_order;
+    const int r = ensure(&p, &ctx->order_cap, (size_t)T * kTileLists * 4);
+    ctx->d_tiles_order = (int32_t*)p;
+    return r;
+}
+
+int exact_bins(gs_ctx* ctx, const ProjView& pv, int64_t n, const gs_camera* cam, bool goff_ready, int64_t m_cap,
+               const int64_t* m_dev, uint64_t* words, int32_t* offsets, cudaStream_t st, int32_t long_min,
+               bool* long_listed, bool rows_ready, bool planned)
+{
+    *long_listed = false;
+    ctx->tile_ordered = 0;
     const int tile = ctx->cfg.tile_size, K = ctx->cfg.K;
     const int32_t tiles_x = (cam->width + tile - 1) / tile, tiles_y = (cam->height + tile - 1) / tile;
     const int64_t T = (int64_t)tiles_x * tiles_y, nseg = T * K;
@@ -708,9 +729,30 @@ int exact_bins(gs_ctx* ctx, const ProjView& pv, int64_t n, const gs_camera* cam,
             // one pass: counts, tile-major scan, look-back over tile rows
             uint64_t* flags;
             if ((r = scan_flags(ctx, tiles_y, &flags, st)) != GS_OK) return r;
+            if ((r = bins_reserve(ctx, 1, nseg)) != GS_OK) return r;
+            if (!(ctx->zeroed_tail == ctx->d_tail && ctx->zeroed_tail_bytes == ctx->tail_cap))
+                GS_CUDA_TRY(cudaMemsetAsync(ctx->d_tail, 0, kTailHead * 4, st));
+            ctx->zeroed_tail = nullptr;  // zeroed by the frame's first kernel once, for this call
+            OffsetsExtra ex;
+            ex.long_list = ctx->d_tail + kTailLong;
+            ex.min_len = long_min;
+            *long_listed = true;
+            const TileOrder to = frame_tile_order(ctx, T);
+            // A whole frame: the raster follows.  Not a deep one, whose tiles are
+            // all long and stop early, so that their lengths do not tell their
+            // work and taking neighbours apart only costs L2 hits (3M Gaussians
+            // seen from inside a cluster: raster 162 us in image order, 166
+            // longest first; 1M at 1080p 229 and 219, 437k at 1237x823 133 and
+            // 121).
+            ctx->tile_ordered = rows_ready && to.lists && !grouped_path(m_cap, tiles_x, tiles_y, K);
+            if (ctx->tile_ordered) {
+                ex.count = ctx->d_tail;
+                ex.order = ctx->d_tiles_order;
+                ex.stride = T;
+            }
             GS_CUDA_TRY(launch_k(ctx, k_bin_offsets<FrameRows>, (unsigned)tiles_y, kOffThreads, osm, st,
                                  FrameRows{v.D, tiles_x, tiles_y, K, rlayer}, (int)tiles_y, m_dev, m_cap, flags,
-                                 ctx->d_scan_done, offsets, want_cur ? v.cur : nullptr, ctx->d_err));
+                                 ctx->d_scan_done, offsets, want_cur ? v.cur : nullptr, ctx->d_err, ex));
             ctx->launches += 1;
         } else {
             // rows too wide for one block's shared memory: per-layer prefix,
