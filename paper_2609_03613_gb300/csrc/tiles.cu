@@ -198,6 +198,59 @@ k_layer_rows_prefix(int32_t* __restrict__ D, int tiles_x, int tiles_y, int64_t l
     }
 }
 
+// What a planned frame's pass can tell of a record from its tile row, bin and
+// span alone, by the block, so that most records it drops are dropped on their
+// first word: a first pass the bins below the row's largest plan, a completing
+// pass the bins from the row's smallest plan of a flagged tile on, and there
+// the spans that meet a flagged tile (one bit a tile, for frames of up to
+// kMaskWords * 32 tiles).
+constexpr int kMaxRows = 4096;  // row records hold 12 bits of tile row
+constexpr int kMaskWords = 4096;
+constexpr int kNoRow = 256;     // above every bin
+
+// s_row[y] of every tile row; with mask, the flagged tiles (flagged = {count,
+// tiles...}, a completing pass's).  Ends with a block barrier.
+__device__ __forceinline__ void plan_rows(const ScatterPass& sp, int tiles_x, int tiles_y,
+                                          const int32_t* __restrict__ flagged, int32_t* s_row, uint32_t* mask)
+{
+    const int words = (tiles_x + 31) / 32;
+    for (int y = threadIdx.x; y < tiles_y; y += blockDim.x) s_row[y] = sp.pass == 1 ? 0 : kNoRow;
+    if (mask)
+        for (int q = threadIdx.x; q < tiles_y * words; q += blockDim.x) mask[q] = 0u;
+    __syncthreads();
+    if (sp.pass == 1) {
+#pragma unroll 8
+        for (int t = threadIdx.x; t < tiles_x * tiles_y; t += blockDim.x)
+            atomicMax(&s_row[t / tiles_x], (int)__ldg(sp.plan + t));
+    } else {
+        for (int i = threadIdx.x; i < flagged[0]; i += blockDim.x) {
+            const int t = flagged[1 + i], y = t / tiles_x, x = t - y * tiles_x;
+            atomicMin(&s_row[y], (int)__ldg(sp.plan + t));
+            if (mask) atomicOr(&mask[y * words + (x >> 5)], 1u << (x & 31));
+        }
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ bool plan_row_live(const ScatterPass& sp, const int32_t* s_row, uint32_t ya)
+{
+    const int b = (int)(ya >> 24), r = s_row[ya & 0xfffu];
+    return sp.pass == 1 ? b < r : b >= r;
+}
+
+// whether tiles [x0, x0 + w) of row y (1 <= w) meet the mask
+__device__ __forceinline__ bool mask_meets(const uint32_t* mask, int words, int y, int x0, int w)
+{
+    const int x1 = x0 + w - 1, q0 = x0 >> 5, q1 = x1 >> 5;
+    for (int q = q0; q <= q1; ++q) {
+        uint32_t m = mask[y * words + q];
+        if (q == q0) m &= 0xffffffffu << (x0 & 31);
+        if (q == q1) m &= 0xffffffffu >> (31 - (x1 & 31));
+        if (m) return true;
+    }
+    return false;
+}
+
 // The tile a pass keeps of a record (ScatterPass::keep), from the lane that
 // holds it in the warp's shared copy of the row words.
 struct KeepPlanned {
@@ -216,39 +269,66 @@ struct KeepPlanned {
 template <bool PLANNED>
 __global__ void __launch_bounds__(256)
 k_bin_scatter_rows(const uint32_t* __restrict__ rs_g, const uint32_t* __restrict__ rs_ya, const uint32_t* __restrict__ rs_w,
-                   const uint32_t* __restrict__ rs_z, const int32_t* __restrict__ roff, int64_t n, int tiles_x,
+                   const uint32_t* __restrict__ rs_z, const int32_t* __restrict__ roff, int64_t n, int tiles_x, int tiles_y,
                    const int64_t* __restrict__ m_dev, int64_t m_cap, const Cursors cur,
                    uint64_t* __restrict__ words, const ScatterPass sp, const int32_t* __restrict__ flagged)
 {
     grid_dependency_sync();
     __shared__ ScatterShared s_sc[8];
     __shared__ uint32_t s_ya[PLANNED ? 8 : 1][32];
+    __shared__ int32_t s_row[PLANNED ? kMaxRows : 1];
+    __shared__ uint32_t s_mask[PLANNED ? kMaskWords : 1];
     if (*m_dev > m_cap) return;
     if (PLANNED && sp.pass == 2 && flagged[0] == 0) return;  // no tile to complete
+    const int mwords = (tiles_x + 31) / 32;
+    const bool masked = PLANNED && sp.pass == 2 && tiles_y * mwords <= kMaskWords;
+    if constexpr (PLANNED) plan_rows(sp, tiles_x, tiles_y, flagged, s_row, masked ? s_mask : nullptr);
     const int64_t R = roff[n];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nchunks = (R + 31) / 32;
-    const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; c < nchunks; c += wstride) {
-        uint32_t w = 0, g = 0, ya = 0, z = 0;
-        const int64_t k = c * 32 + lane;
-        if (k < R) {  // read once: streamed past L2
-            ya = __ldcs(rs_ya + k);
-            if (!PLANNED || sp.row_live((int)(ya & 0xfffu))) {
+    const int64_t w0 = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp, wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
+    // records read once: streamed past L2
+    auto first_slot = [&](uint32_t ya) {
+        return (uint32_t)(((int64_t)(ya & 0xfffu) * tiles_x + ((ya >> 12) & 0xfffu)) * cur.tile +
+                          (int64_t)(ya >> 24) * cur.bin);
+    };
+    if constexpr (PLANNED) {
+        // most chunks hold nothing the pass takes: the next row words are on
+        // their way while one is looked at
+        uint32_t next = w0 * 32 + lane < R ? __ldcs(rs_ya + w0 * 32 + lane) : 0xffffffffu;
+        for (int64_t c = w0; c < nchunks; c += wstride) {
+            const int64_t k = c * 32 + lane, kn = (c + wstride) * 32 + lane;
+            uint32_t w = 0, g = 0, ya = next, z = 0;
+            next = kn < R ? __ldcs(rs_ya + kn) : 0xffffffffu;
+            const bool live = k < R && plan_row_live(sp, s_row, ya);
+            if (!__any_sync(0xffffffffu, live)) continue;
+            if (live) {
+                w = __ldcs(rs_w + k);
+                if (w != 0u && masked &&
+                    !mask_meets(s_mask, mwords, (int)(ya & 0xfffu), (int)((ya >> 12) & 0xfffu), (int)w))
+                    w = 0;
+                sp.trim(ya, w, tiles_x);
+                if (w != 0u) {
+                    g = __ldcs(rs_g + k);
+                    z = __ldcs(rs_z + k);
+                }
+            }
+            if (!__any_sync(0xffffffffu, w != 0u)) continue;
+            s_ya[warp][lane] = ya;  // read after the warp barriers of the scatter
+            scatter_row_records(w, g, z, first_slot(ya), (uint32_t)cur.tile, cur.p, words, s_sc[warp],
+                                KeepPlanned{sp, s_ya[warp], tiles_x});
+        }
+    } else {
+        for (int64_t c = w0; c < nchunks; c += wstride) {
+            uint32_t w = 0, g = 0, ya = 0, z = 0;
+            const int64_t k = c * 32 + lane;
+            if (k < R) {
+                ya = __ldcs(rs_ya + k);
                 w = __ldcs(rs_w + k);
                 g = __ldcs(rs_g + k);
                 z = __ldcs(rs_z + k);
-                if (PLANNED) sp.trim(ya, w, tiles_x);
             }
-        }
-        const uint32_t slot = (uint32_t)(((int64_t)(ya & 0xfffu) * tiles_x + ((ya >> 12) & 0xfffu)) * cur.tile +
-                                         (int64_t)(ya >> 24) * cur.bin);
-        if constexpr (PLANNED) {
-            s_ya[warp][lane] = ya;  // read after the warp barriers of the scatter
-            scatter_row_records(w, g, z, slot, (uint32_t)cur.tile, cur.p, words, s_sc[warp],
-                                KeepPlanned{sp, s_ya[warp], tiles_x});
-        } else {
-            scatter_row_records(w, g, z, slot, (uint32_t)cur.tile, cur.p, words, s_sc[warp], KeepAll());
+            scatter_row_records(w, g, z, first_slot(ya), (uint32_t)cur.tile, cur.p, words, s_sc[warp], KeepAll());
         }
     }
 }
@@ -292,7 +372,21 @@ __device__ __forceinline__ void record_slice(int64_t R, int C, int c, int64_t* r
 // key of a row record: (tile row, bin)
 __device__ __forceinline__ int group_key(uint32_t ya, int K) { return (int)(ya & 0xfffu) * K + (int)(ya >> 24); }
 
+// The record word and width at k, the width 0 when the pass drops it.
+template <bool PLANNED>
+__device__ __forceinline__ uint32_t group_record(const uint32_t* __restrict__ rs_ya, const uint32_t* __restrict__ rs_w,
+                                                 int64_t k, const ScatterPass& sp, const int32_t* s_row, int tiles_x,
+                                                 uint32_t& ya)
+{
+    ya = rs_ya[k];
+    if (PLANNED && !plan_row_live(sp, s_row, ya)) return 0u;
+    uint32_t w = rs_w[k];
+    if (PLANNED) sp.trim(ya, w, tiles_x);
+    return w;
+}
+
 // pass 1: H[key * C + c] = non-empty records of slice c with that key
+template <bool PLANNED>
 __global__ void __launch_bounds__(kGroupThreads)
 k_group_count(const uint32_t* __restrict__ rs_ya, const uint32_t* __restrict__ rs_w, const int32_t* __restrict__ roff,
               int64_t n, int K, int nkeys, const int64_t* __restrict__ m_dev, int64_t m_cap, int32_t* __restrict__ H,
@@ -300,16 +394,17 @@ k_group_count(const uint32_t* __restrict__ rs_ya, const uint32_t* __restrict__ r
 {
     grid_dependency_sync();
     extern __shared__ int32_t s_h[];
+    __shared__ int32_t s_row[PLANNED ? kMaxRows : 1];
     const int C = gridDim.x, c = blockIdx.x;
     for (int i = threadIdx.x; i < nkeys; i += blockDim.x) s_h[i] = 0;
+    if (PLANNED) plan_rows(sp, tiles_x, nkeys / K, nullptr, s_row, nullptr);
     __syncthreads();
     if (*m_dev <= m_cap) {
         int64_t r0, r1;
         record_slice(roff[n], C, c, &r0, &r1);
         for (int64_t k = r0 + threadIdx.x; k < r1; k += blockDim.x) {
-            uint32_t w = rs_w[k], ya = rs_ya[k];
-            sp.trim(ya, w, tiles_x);
-            if (w != 0u) atomicAdd(&s_h[group_key(ya, K)], 1);
+            uint32_t ya;
+            if (group_record<PLANNED>(rs_ya, rs_w, k, sp, s_row, tiles_x, ya) != 0u) atomicAdd(&s_h[group_key(ya, K)], 1);
         }
     }
     __syncthreads();
@@ -319,6 +414,7 @@ k_group_count(const uint32_t* __restrict__ rs_ya, const uint32_t* __restrict__ r
 // pass 2: list[Hs[key * C + c] + rank] = the record {gid, row word, width,
 // depth bits} (any order within a key), so the scatter reads its group
 // contiguously
+template <bool PLANNED>
 __global__ void __launch_bounds__(kGroupThreads)
 k_group_write(const uint32_t* __restrict__ rs_g, const uint32_t* __restrict__ rs_ya,
               const uint32_t* __restrict__ rs_w, const uint32_t* __restrict__ rs_z, const int32_t* __restrict__ roff,
@@ -327,15 +423,17 @@ k_group_write(const uint32_t* __restrict__ rs_g, const uint32_t* __restrict__ rs
 {
     grid_dependency_sync();
     extern __shared__ int32_t s_h[];  // [nkeys] next slot, from the slice's base
+    __shared__ int32_t s_row[PLANNED ? kMaxRows : 1];
     const int C = gridDim.x, c = blockIdx.x;
     if (*m_dev > m_cap) return;
     for (int i = threadIdx.x; i < nkeys; i += blockDim.x) s_h[i] = Hs[(int64_t)i * C + c];
+    if (PLANNED) plan_rows(sp, tiles_x, nkeys / K, nullptr, s_row, nullptr);
     __syncthreads();
     int64_t r0, r1;
     record_slice(roff[n], C, c, &r0, &r1);
     for (int64_t k = r0 + threadIdx.x; k < r1; k += blockDim.x) {
-        uint32_t w = rs_w[k], ya = rs_ya[k];
-        sp.trim(ya, w, tiles_x);
+        uint32_t ya;
+        const uint32_t w = group_record<PLANNED>(rs_ya, rs_w, k, sp, s_row, tiles_x, ya);
         if (w == 0u) continue;
         list[atomicAdd(&s_h[group_key(ya, K)], 1)] = make_uint4(rs_g[k], ya, w, rs_z[k]);
     }
@@ -572,12 +670,12 @@ static int exact_scatter(gs_ctx* ctx, const ExactScratch& v, int64_t n, int32_t 
         // (a planned first pass groups only the records it keeps)
         const int C = group_slices(ctx->num_sms);
         const size_t hsm = (size_t)nkeys * 4;
-        GS_CUDA_TRY(launch_k(ctx, k_group_count, (unsigned)C, kGroupThreads, hsm, st, v.rs_ya, v.rs_w, v.roff, n, K, nkeys, m_dev, m_cap,
+        GS_CUDA_TRY(launch_k(ctx, sp.pass ? k_group_count<true> : k_group_count<false>, (unsigned)C, kGroupThreads, hsm, st, v.rs_ya, v.rs_w, v.roff, n, K, nkeys, m_dev, m_cap,
                                                                 v.H, sp, tiles_x));
         ctx->launches += 1;
         int r;
         if ((r = scan_impl(ctx, LoadI32{v.H}, (int64_t)nkeys * C, v.Hs, nullptr, st)) != GS_OK) return r;
-        GS_CUDA_TRY(launch_k(ctx, k_group_write, (unsigned)C, kGroupThreads, hsm, st, v.rs_g, v.rs_ya, v.rs_w, v.rs_z, v.roff, n, K, nkeys,
+        GS_CUDA_TRY(launch_k(ctx, sp.pass ? k_group_write<true> : k_group_write<false>, (unsigned)C, kGroupThreads, hsm, st, v.rs_g, v.rs_ya, v.rs_w, v.rs_z, v.roff, n, K, nkeys,
                                                                 m_dev, m_cap, v.Hs, v.list, sp, tiles_x));
         GS_CUDA_TRY(launch_k(ctx, k_scatter_groups, (unsigned)nkeys, kScatterGroupThreads, (size_t)tiles_x * 4, st, 
             v.list, v.Hs, C, offsets, tiles_x, K, m_dev, m_cap, words, sp, flagged));
@@ -591,8 +689,8 @@ static int exact_scatter(gs_ctx* ctx, const ExactScratch& v, int64_t n, int32_t 
             GS_CUDA_TRY(launch_k(ctx, k_flagged_cursors, (unsigned)ctx->num_sms * 2, 256, 0, st, flagged, offsets, K, cur));
             ctx->launches += 1;
         }
-        GS_CUDA_TRY(launch_k(ctx, sp.pass ? k_bin_scatter_rows<true> : k_bin_scatter_rows<false>, g_sm * 2, 256, 0, st, v.rs_g, v.rs_ya, v.rs_w, v.rs_z, v.roff, n, tiles_x, m_dev,
-                                                     m_cap, cur, words, sp, flagged));
+        GS_CUDA_TRY(launch_k(ctx, sp.pass ? k_bin_scatter_rows<true> : k_bin_scatter_rows<false>, sp.pass ? g_sm : g_sm * 2, 256, 0, st, v.rs_g, v.rs_ya, v.rs_w, v.rs_z, v.roff, n, tiles_x, tiles_y,
+                                                     m_dev, m_cap, cur, words, sp, flagged));
         ctx->launches += 1;
     }
     GS_CUDA_TRY(cudaGetLastError());
@@ -650,6 +748,9 @@ int bin_offsets_prepare()
 {
     GS_CUDA_TRY(cudaFuncSetAttribute(k_bin_offsets<FrameRows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kOffMaxSmem));
+    // the planned grouping's keys and row table together pass 48 KB
+    GS_CUDA_TRY(cudaFuncSetAttribute(k_group_count<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxGroupKeys * 4));
+    GS_CUDA_TRY(cudaFuncSetAttribute(k_group_write<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxGroupKeys * 4));
     return group_offsets_prepare();
 }
 
