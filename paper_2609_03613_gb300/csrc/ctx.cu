@@ -168,7 +168,7 @@ extern "C" int gs_destroy(gs_ctx* c)
                     c->d_tiles_order, c->r_proj, c->r_isect, c->r_stream,
                     c->r_off, c->r_m, c->r_scene, c->r_out, c->d_ops, c->d_tiles, c->d_samples,
                     c->r_T, c->r_tend, c->r_wend, c->d_planner, c->d_feat, c->d_plan, c->d_plist,
-                    c->d_order_ws, c->d_scan_done};
+                    c->d_order_ws, c->d_scan_done, c->d_gsort};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (c->h_m) cudaFreeHost(c->h_m);
@@ -600,7 +600,10 @@ int gs::render_binning(gs_ctx* c, int64_t n, const float* scales, const gs_camer
     stage_begin(c, GS_STAGE_INTERSECT, st);
     // EXACT with the tile cull: the row-record offsets in the same pass
     const bool rows = c->cfg.mode == GS_MODE_BINNED_EXACT && c->cfg.tile_cull;
-    r = rows ? count_rows_scan(c, pv, n, c->r_m, st) : count_scan(c, pv, n, c->r_m, st);
+    const bool global = c->cfg.mode == GS_MODE_GLOBAL_SORT;
+    r = global ? frame_sort_gaussians(c, pv, n, c->r_m_cap, T, c->r_m, st)
+        : rows ? count_rows_scan(c, pv, n, c->r_m, st)
+               : count_scan(c, pv, n, c->r_m, st);
     if (r != GS_OK) return r;
     if (!(flags & GS_RENDER_NO_SYNC)) {
         // size the entry buffers: read M once, grow if needed
@@ -634,6 +637,12 @@ int gs::render_binning(gs_ctx* c, int64_t n, const float* scales, const gs_camer
         stage_begin(c, GS_STAGE_REPAIR, st);
         r = repair_min(c, T, c->r_m, c->r_stream, c->r_off, nullptr, min_len, st, planned ? 1 : 0, listed);
         stage_end(c, GS_STAGE_REPAIR, st);
+    } else if (global) {
+        stage_end(c, GS_STAGE_INTERSECT, st);
+        stage_begin(c, GS_STAGE_SORT, st);
+        r = frame_sort_entries(c, pv, n, c->r_m_cap, (W + c->cfg.tile_size - 1) / c->cfg.tile_size, T, c->r_m,
+                               c->r_stream, c->r_off, st);
+        stage_end(c, GS_STAGE_SORT, st);
     } else {
         r = emit_only(c, pv, n, cam, isect_view(c->r_isect, c->r_m_cap), c->r_m_cap, c->r_m, st);
         stage_end(c, GS_STAGE_INTERSECT, st);
@@ -909,7 +918,7 @@ extern "C" int gs_render(gs_ctx* c, const gs_scene* sc, const gs_camera* cam, co
         int timing, device, flags;
         // the internal scratch the captured kernels address (a grown buffer
         // is a new allocation: the graph is captured again)
-        const void* scratch[15];
+        const void* scratch[16];
         size_t scratch_bytes[10];
     } key;
     if (flags & GS_RENDER_SAVE) {
@@ -941,7 +950,7 @@ extern "C" int gs_render(gs_ctx* c, const gs_scene* sc, const gs_camera* cam, co
     key.saved_wend = c->r_wend;
     const void* scratch[] = {c->d_scan, c->d_goff, c->d_keys[0], c->d_keys[1], c->d_vals[0], c->d_vals[1],
                              c->d_hist, c->d_count, c->d_bin, c->d_sel, c->d_tail, c->d_tiles, c->d_samples,
-                             c->d_plan, c->d_tiles_order};
+                             c->d_plan, c->d_tiles_order, c->d_gsort};
     const size_t scratch_bytes[] = {c->scan_bytes, c->goff_cap, c->sort_cap, c->hist_cap, c->count_cap,
                                     c->bin_cap, c->sel_cap, c->tail_cap, c->tiles_cap, c->samples_cap};
     static_assert(sizeof(scratch) == sizeof(key.scratch) && sizeof(scratch_bytes) == sizeof(key.scratch_bytes),

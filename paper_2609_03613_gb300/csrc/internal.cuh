@@ -249,6 +249,9 @@ struct gs_ctx {
     size_t sort_cap = 0;
     uint32_t* d_hist = nullptr;
     size_t hist_cap = 0;
+    // a global-sort frame's Gaussians in depth order (frame_sort.cu)
+    void* d_gsort = nullptr;
+    size_t gsort_cap = 0;
     // binning
     int32_t* d_count = nullptr;  // T*K counters
     size_t count_cap = 0;
@@ -447,6 +450,16 @@ int emit_only(gs_ctx* ctx, const ProjView& pv, int64_t n, const gs_camera* cam, 
 // sort.cu
 int global_sort(gs_ctx* ctx, const IsectView& is, int64_t m_cap, const int64_t* m_dev,
                 int32_t n_tiles, uint64_t* stream_words, int32_t* offsets, cudaStream_t st);
+
+int sort_reserve(gs_ctx* ctx, int64_t m_cap);
+
+// frame_sort.cu: the stream of a whole global-sort frame from the projected
+// Gaussians, in two steps (M is known after the first)
+int frame_sort_reserve(gs_ctx* ctx, int64_t n, int64_t m_cap, int32_t n_tiles);
+int frame_sort_gaussians(gs_ctx* ctx, const ProjView& pv, int64_t n, int64_t m_cap, int32_t n_tiles, int64_t* m_dev,
+                         cudaStream_t st);
+int frame_sort_entries(gs_ctx* ctx, const ProjView& pv, int64_t n, int64_t m_cap, int32_t tiles_x, int32_t n_tiles,
+                       const int64_t* m_dev, uint64_t* words, int32_t* offsets, cudaStream_t st);
 
 // bins.cu
 int depth_range(gs_ctx* ctx, const ProjView& pv, const float* scales, const IsectView& is,

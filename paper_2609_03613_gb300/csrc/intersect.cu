@@ -124,7 +124,6 @@ int launch_emit(gs_ctx* ctx, const ProjView& pv, int64_t n, const gs_camera* cam
 }  // namespace gs
 
 namespace gs {
-int sort_reserve(gs_ctx* ctx, int64_t m_cap);
 int bins_reserve(gs_ctx* ctx, int64_t m_cap, int64_t nseg);
 
 int exact_bins_reserve(gs_ctx* ctx, int64_t n, int64_t m_cap, int32_t tiles_x, int32_t tiles_y, int K);
@@ -149,7 +148,7 @@ int reserve_internal(gs_ctx* ctx, int64_t n, int64_t m_cap, int32_t width, int32
     if ((r = ensure(&ctx->d_scan, &ctx->scan_bytes, (size_t)words * sizeof(uint64_t))) != GS_OK) return r;
     if ((r = goff_reserve(ctx, n)) != GS_OK) return r;
     if ((r = samples_reserve(ctx)) != GS_OK) return r;
-    if (ctx->cfg.mode == GS_MODE_GLOBAL_SORT) return sort_reserve(ctx, m_cap);
+    if (ctx->cfg.mode == GS_MODE_GLOBAL_SORT) return frame_sort_reserve(ctx, n, m_cap, tiles_x * tiles_y);
     if ((r = bins_reserve(ctx, m_cap, (int64_t)tiles_x * tiles_y * ctx->cfg.K)) != GS_OK) return r;
     if (ctx->cfg.mode == GS_MODE_BINNED_EXACT)
         return exact_bins_reserve(ctx, n, m_cap, tiles_x, tiles_y, ctx->cfg.K);
