@@ -1,6 +1,6 @@
 // raster.cu -- K6 / K16: front-to-back compositing over each tile's span of
 // the tile-major stream (Sec. 3.4; supplement "Binned raster traversal after
-// repair").  One CTA per tile, two pixels a thread, the span consumed in
+// repair").  One CTA per tile, one or two pixels a thread, the span consumed in
 // batches staged through shared memory, and a block-wide vote ends the tile
 // once every pixel has terminated.
 //
@@ -26,67 +26,126 @@
 
 namespace gs {
 
-// A lane's two pixels of its warp's 8 x 8 block: (x, y) and (x + 4, y).  They
-// share dy and the entry's shared-memory reads, and what is done to both runs
-// on packed float32 pairs (each half rounded as the scalar operation).
+// A lane's P pixels.  Two: (x, y) and (x + 4, y) of the warp's 8 x 8 block;
+// they share dy and the entry's shared-memory reads, and what is done to both
+// runs on packed float32 pairs (each half rounded as the scalar operation).
+// One: a pixel of the warp's 8 x 4 block, scalar.
+template <int P>
+struct Lane;
+template <>
+struct Lane<2> {
+    using V = uint64_t;  // pixel 0 in the low half
+    static __device__ __forceinline__ V same(float v) { return same2(v); }
+    static __device__ __forceinline__ V put(const float (&v)[2]) { return pk2(v[0], v[1]); }
+    static __device__ __forceinline__ void get(V v, float (&o)[2]) { upk2(v, o[0], o[1]); }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return fma2(a, b, c); }
+    static __device__ __forceinline__ V mul(V a, V b) { return mul2(a, b); }
+    static __device__ __forceinline__ void exp_neg(const float (&q)[2], float (&e)[2])
+    {
+        spec_exp_neg2(q[0], q[1], e[0], e[1]);
+    }
+    static __device__ __forceinline__ float least(const float (&v)[2]) { return fminf(v[0], v[1]); }
+    // the lane's pixel h in its warp's block
+    static __device__ __forceinline__ int x(int lane, int h) { return (lane & 3) + 4 * h; }
+    static __device__ __forceinline__ int y(int lane) { return lane >> 2; }
+};
+template <>
+struct Lane<1> {
+    using V = float;
+    static __device__ __forceinline__ V same(float v) { return v; }
+    static __device__ __forceinline__ V put(const float (&v)[1]) { return v[0]; }
+    static __device__ __forceinline__ void get(V v, float (&o)[1]) { o[0] = v; }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return fmaf(a, b, c); }
+    static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
+    static __device__ __forceinline__ void exp_neg(const float (&q)[1], float (&e)[1]) { e[0] = spec_exp_core(-q[0]); }
+    static __device__ __forceinline__ float least(const float (&v)[1]) { return v[0]; }
+    static __device__ __forceinline__ int x(int lane, int) { return lane & 7; }
+    static __device__ __forceinline__ int y(int lane) { return lane >> 3; }
+};
 
-// Per-thread compositing state: two pixels.  A pixel that has stopped (or lies
-// outside the image) has a NaN centre, so that no entry passes it again.
+// Per-thread compositing state.  A pixel that has stopped (or lies outside the
+// image) has a NaN centre, so that no entry passes it again.
+template <int P>
 struct PixelState {
-    float x[2], y;  // pixel centres
-    uint64_t T, C0, C1, C2;  // packed, pixel 0 in the low half
-    int32_t last[2], ntests[2];
+    using V = typename Lane<P>::V;
+    float x[P], y;  // pixel centres
+    V T, C0, C1, C2;
+    int32_t last[P], ntests[P];
     int32_t stop;   // stream position of the entry that stopped a pixel last
     int live;       // bit h: pixel h is still compositing
     unsigned long long ops;
 };
 
+// q of one staged entry at the lane's pixels.
+template <int P>
+__device__ __forceinline__ void entry_dist(const float4& ga, const float4& gb, const PixelState<P>& st, float (&q)[P])
+{
+    if constexpr (P == 2) {
+        entry_q(ga, gb, st.x[0], st.x[1], st.y, q[0], q[1]);
+    } else {
+        const float dx = ga.x - st.x[0], dy = ga.y - st.y;
+        q[0] = fmaf(dx, fmaf(ga.z, dx, ga.w * dy), (gb.x * dy) * dy);
+    }
+}
+
 // alpha of one entry where the pixel takes it (pass), else 0.  0 <= q <= tau
 // as one unsigned compare of the float bits (negative q and NaN compare above
 // any positive tau).
+template <int P>
 struct EntryAlpha {
-    float a0, a1;
-    bool pass0, pass1;
+    float a[P];
+    bool pass[P];
 };
-__device__ __forceinline__ EntryAlpha entry_alpha(float q0, float q1, const float4& gb)
+template <int P>
+__device__ __forceinline__ EntryAlpha<P> entry_alpha(const float (&q)[P], const float4& gb)
 {
-    float e0, e1;
-    spec_exp_neg2(q0, q1, e0, e1);
-    upk2(mul2(same2(gb.y), pk2(e0, e1)), e0, e1);
-    const float f0 = fminf(0.99f, e0), f1 = fminf(0.99f, e1);
+    using L = Lane<P>;
+    float e[P];
+    L::exp_neg(q, e);
+    L::get(L::mul(L::same(gb.y), L::put(e)), e);
     const uint32_t tau = __float_as_uint(gb.z);
-    EntryAlpha r;
-    r.pass0 = __float_as_uint(q0) <= tau && f0 >= 1.0f / 255.0f;
-    r.pass1 = __float_as_uint(q1) <= tau && f1 >= 1.0f / 255.0f;
-    r.a0 = r.pass0 ? f0 : 0.0f;
-    r.a1 = r.pass1 ? f1 : 0.0f;
+    EntryAlpha<P> r;
+#pragma unroll
+    for (int h = 0; h < P; ++h) {
+        const float f = fminf(0.99f, e[h]);
+        r.pass[h] = __float_as_uint(q[h]) <= tau && f >= 1.0f / 255.0f;
+        r.a[h] = r.pass[h] ? f : 0.0f;
+    }
     return r;
 }
 
-// C = fma(colour, w, C) at both pixels.
-__device__ __forceinline__ void add_colour(const float4& c, uint64_t w, PixelState& st)
+// C = fma(colour, w, C) at the lane's pixels.
+template <int P>
+__device__ __forceinline__ void add_colour(const float4& c, typename Lane<P>::V w, PixelState<P>& st)
 {
-    st.C0 = fma2(same2(c.x), w, st.C0);
-    st.C1 = fma2(same2(c.y), w, st.C1);
-    st.C2 = fma2(same2(c.z), w, st.C2);
+    using L = Lane<P>;
+    st.C0 = L::fma(L::same(c.x), w, st.C0);
+    st.C1 = L::fma(L::same(c.y), w, st.C1);
+    st.C2 = L::fma(L::same(c.z), w, st.C2);
 }
 
-// T (1 - alpha) at both pixels, 1 - alpha rounded once.
-__device__ __forceinline__ uint64_t transmit(uint64_t T, uint64_t a)
+// T (1 - alpha) at the lane's pixels, 1 - alpha rounded once.
+template <int P>
+__device__ __forceinline__ typename Lane<P>::V transmit(typename Lane<P>::V T, typename Lane<P>::V a)
 {
-    return mul2(T, fma2(a, same2(-1.0f), same2(1.0f)));
+    using L = Lane<P>;
+    return L::mul(T, L::fma(a, L::same(-1.0f), L::same(1.0f)));
 }
 
 // One entry (id g, stream position pos) with its stops: a pixel whose
 // transmittance would fall below 1e-4 stops before it is applied.
-__device__ __forceinline__ void apply_with_stops(const EntryAlpha& e, const float4& c, int32_t g, int32_t pos,
-                                                 PixelState& st)
+template <int P>
+__device__ __forceinline__ void apply_with_stops(const EntryAlpha<P>& e, const float4& c, int32_t g, int32_t pos,
+                                                 PixelState<P>& st)
 {
-    float T[2], t[2], a[2] = {e.a0, e.a1};
-    upk2(st.T, T[0], T[1]);
-    upk2(transmit(st.T, pk2(a[0], a[1])), t[0], t[1]);
+    using L = Lane<P>;
+    float T[P], t[P], a[P];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < P; ++h) a[h] = e.a[h];
+    L::get(st.T, T);
+    L::get(transmit<P>(st.T, L::put(a)), t);
+#pragma unroll
+    for (int h = 0; h < P; ++h) {
         if (((st.live >> h) & 1) && t[h] < 1e-4f) {
             st.live &= ~(1 << h);
             st.x[h] = __uint_as_float(0x7fc00000u);
@@ -98,8 +157,8 @@ __device__ __forceinline__ void apply_with_stops(const EntryAlpha& e, const floa
         }
         if (a[h] > 0.0f) st.last[h] = g;
     }
-    add_colour(c, mul2(pk2(a[0], a[1]), st.T), st);
-    st.T = pk2(t[0], t[1]);
+    add_colour<P>(c, L::mul(L::put(a), st.T), st);
+    st.T = L::put(t);
 }
 
 // Composite the cnt staged entries of a batch into the calling thread's
@@ -124,12 +183,13 @@ __device__ __forceinline__ void apply_with_stops(const EntryAlpha& e, const floa
 //
 // SKIP (the plain raster, whose warps visit entries far from their pixels):
 // a round no pixel of which has q <= tau ends there.
-template <int TILE, bool SKIP, int R>
-__device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE>& sh, PixelState& st, int32_t base)
+template <int TILE, int P, bool SKIP, int R>
+__device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE, P>& sh, PixelState<P>& st, int32_t base)
 {
+    using L = Lane<P>;
     const int warp = threadIdx.x >> 5;
     if (__all_sync(0xffffffffu, st.live == 0)) return;
-    const int nk = warp_strip_list<TILE>(sh, cnt);
+    const int nk = warp_strip_list(sh, cnt);
     const char* pa = reinterpret_cast<const char*>(sh.a);
     const char* pb = reinterpret_cast<const char*>(sh.b);
     const char* pc = reinterpret_cast<const char*>(sh.c);
@@ -142,45 +202,45 @@ __device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE>& sh,
             k[j + 1] = pair >> 16;
         }
         float4 gb[R];
-        float q[R][2];
+        float q[R][P];
 #pragma unroll
         for (int j = 0; j < R; ++j) {
             gb[j] = *reinterpret_cast<const float4*>(pb + k[j]);
-            entry_q(*reinterpret_cast<const float4*>(pa + k[j]), gb[j], st.x[0], st.x[1], st.y, q[j][0],
-                    q[j][1]);
+            entry_dist<P>(*reinterpret_cast<const float4*>(pa + k[j]), gb[j], st, q[j]);
         }
         if constexpr (SKIP) {
             bool any = false;
 #pragma unroll
             for (int j = 0; j < R; ++j)
-                any |= min(__float_as_uint(q[j][0]), __float_as_uint(q[j][1])) <= __float_as_uint(gb[j].z);
+#pragma unroll
+                for (int h = 0; h < P; ++h) any |= __float_as_uint(q[j][h]) <= __float_as_uint(gb[j].z);
             if (!__any_sync(0xffffffffu, any)) continue;
         }
-        EntryAlpha e[R];
-        uint64_t A[R], T[R + 1];
+        EntryAlpha<P> e[R];
+        typename L::V A[R], T[R + 1];
         T[0] = st.T;
 #pragma unroll
-        for (int j = 0; j < R; ++j) e[j] = entry_alpha(q[j][0], q[j][1], gb[j]);
+        for (int j = 0; j < R; ++j) e[j] = entry_alpha<P>(q[j], gb[j]);
 #pragma unroll
         for (int j = 0; j < R; ++j) {
-            A[j] = pk2(e[j].a0, e[j].a1);
-            T[j + 1] = transmit(T[j], A[j]);
+            A[j] = L::put(e[j].a);
+            T[j + 1] = transmit<P>(T[j], A[j]);
         }
-        float t0, t1;
-        upk2(T[R], t0, t1);
-        if (__any_sync(0xffffffffu, fminf(t0, t1) < 1e-4f)) {
+        float t[P];
+        L::get(T[R], t);
+        if (__any_sync(0xffffffffu, L::least(t) < 1e-4f)) {
 #pragma unroll
             for (int j = 0; j < R; ++j)
-                apply_with_stops(e[j], *reinterpret_cast<const float4*>(pc + k[j]), __float_as_int(gb[j].w),
-                                 base + (int32_t)(k[j] >> 4), st);
+                apply_with_stops<P>(e[j], *reinterpret_cast<const float4*>(pc + k[j]), __float_as_int(gb[j].w),
+                                    base + (int32_t)(k[j] >> 4), st);
             if (__all_sync(0xffffffffu, st.live == 0)) break;
         } else {
 #pragma unroll
             for (int j = 0; j < R; ++j) {
-                add_colour(*reinterpret_cast<const float4*>(pc + k[j]), mul2(A[j], T[j]), st);
+                add_colour<P>(*reinterpret_cast<const float4*>(pc + k[j]), L::mul(A[j], T[j]), st);
                 const int32_t g = __float_as_int(gb[j].w);
-                st.last[0] = e[j].pass0 ? g : st.last[0];
-                st.last[1] = e[j].pass1 ? g : st.last[1];
+#pragma unroll
+                for (int h = 0; h < P; ++h) st.last[h] = e[j].pass[h] ? g : st.last[h];
             }
             st.T = T[R];
         }
@@ -189,11 +249,11 @@ __device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE>& sh,
 
 // The counting twin: one pixel and one entry at a time, the same values.
 template <int TILE>
-__device__ __forceinline__ void composite_batch_count(int cnt, RasterShared<TILE>& sh, PixelState& st,
+__device__ __forceinline__ void composite_batch_count(int cnt, RasterShared<TILE, 2>& sh, PixelState<2>& st,
                                                       int32_t base)
 {
     const int warp = threadIdx.x >> 5;
-    const int nk = warp_strip_list<TILE>(sh, cnt);
+    const int nk = warp_strip_list(sh, cnt);
     float T[2], C0[2], C1[2], C2[2];
     upk2(st.T, T[0], T[1]);
     upk2(st.C0, C0[0], C0[1]);
@@ -238,16 +298,16 @@ __device__ __forceinline__ void composite_batch_count(int cnt, RasterShared<TILE
 
 // A run of entries composited into the tile's pixels: what the walk hands its
 // runs and staged chunks to (raster_common.cuh).
-template <int TILE, bool COUNT, bool LAZY, int R>
+template <int TILE, int P, bool COUNT, bool LAZY, int R>
 struct FwdSpan {
-    using SH = RasterShared<TILE>;
+    using SH = RasterShared<TILE, P>;
     static constexpr int kBatch = SH::BATCH;
     SH& sh;
     const float4* __restrict__ xy_ab;
     const float4* __restrict__ c_o_z;
     const float4* __restrict__ rgbv;
     int cullmode, tx, ty;
-    PixelState& st;
+    PixelState<P>& st;
     // n entries from src (global or shared memory) in batches: -1 after the
     // last, or the offset of the first batch left once every pixel of the
     // tile has terminated
@@ -257,17 +317,19 @@ struct FwdSpan {
             // checked: the caller has just counted the terminated pixels (block
             // barrier included) with nothing composited since
             if (!(checked && b0 == 0) && __syncthreads_count(done()) == SH::TB::NT) return b0;
-            const int cnt = stage_batch<TILE>(src, b0, n, sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty);
+            const int cnt = stage_batch(src, b0, n, sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty);
             __syncthreads();
             composite_staged(cnt, base + b0);
         }
         return -1;
     }
     __device__ __forceinline__ bool done() const { return st.live == 0; }
+    // shared memory free between the batches (the staging arrays')
+    __device__ __forceinline__ uint32_t* scratch() const { return reinterpret_cast<uint32_t*>(sh.a); }
     __device__ __forceinline__ void stage_at(int slot, uint32_t g)
     {
         float4 A, B, C;
-        stage_record<TILE>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
+        stage_record<TILE, P>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
         sh.a[slot] = A;
         sh.b[slot] = B;
         sh.c[slot] = C;
@@ -278,8 +340,8 @@ struct FwdSpan {
             composite_batch_count<TILE>(cnt, sh, st, base);
         } else {
             if constexpr (!LAZY)
-                if (cullmode & kPlain) return composite_batch<TILE, true, R>(cnt, sh, st, base);
-            composite_batch<TILE, false, R>(cnt, sh, st, base);
+                if (cullmode & kPlain) return composite_batch<TILE, P, true, R>(cnt, sh, st, base);
+            composite_batch<TILE, P, false, R>(cnt, sh, st, base);
         }
     }
 };
@@ -290,32 +352,35 @@ struct FwdSpan {
 // composited (longer ones were sorted eagerly), so segments after every
 // pixel's termination are never sorted.
 // One tile t by the whole block (the body of the raster kernels below).
-template <int TILE, bool COUNT, bool LAZY, int R>
+template <int TILE, int P, bool COUNT, bool LAZY, int R>
 __device__ __forceinline__ void raster_tile(
-    int t, RasterShared<TILE>& sh, WalkShared<TILE, LAZY>& ws, const float4* __restrict__ xy_ab,
+    int t, RasterShared<TILE, P>& sh, WalkShared<TILE, LAZY>& ws, const float4* __restrict__ xy_ab,
     const float4* __restrict__ c_o_z, const float4* __restrict__ rgbv, uint64_t* words,
     const int32_t* __restrict__ off, const RasterArgs& a, int cullmode, float* __restrict__ out_rgb,
     float* __restrict__ out_alpha, int32_t* __restrict__ out_last, int32_t* __restrict__ out_ntests,
     unsigned long long* __restrict__ ops_total, float* __restrict__ out_T, int32_t* __restrict__ out_end,
     const PlanView& pl, int cap, int32_t* __restrict__ out_wend = nullptr)
 {
-    using TB = TileBlocks<TILE>;
+    using TB = TileBlocks<TILE, P>;
+    using L = Lane<P>;
     const int tx = t % a.tiles_x, ty = t / a.tiles_x;
     const int lane = threadIdx.x & 31;
-    // the lane's first pixel; the second is four to its right
-    const int px = tx * TILE + TB::x0() + (lane & 3), py = ty * TILE + TB::y0() + (lane >> 2);
-    const int inside = py < a.height ? (px < a.width ? 1 : 0) | (px + 4 < a.width ? 2 : 0) : 0;
+    const int px0 = tx * TILE + TB::x0(), py0 = ty * TILE + TB::y0();  // the warp's block
+    const int py = py0 + L::y(lane);
+    int inside = 0;
+#pragma unroll
+    for (int h = 0; h < P; ++h) inside |= (py < a.height && px0 + L::x(lane, h) < a.width ? 1 : 0) << h;
 
     // float32 operations of the compositing definition each pixel executes
     // (COUNT builds): 8 per visit (offsets, q, sign test), 17 more when exp is
     // evaluated (exp, o*e, clamp, threshold), 3 when alpha passes (1-alpha,
     // T*, stop test), 4 when applied (alpha*T and three colour fmas)
-    PixelState st;
+    PixelState<P> st;
     st.y = (float)py + 0.5f;
-    st.T = same2(1.0f);
-    st.C0 = st.C1 = st.C2 = 0ull;
+    st.T = L::same(1.0f);
+    st.C0 = st.C1 = st.C2 = L::same(0.0f);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < P; ++h) {
         st.last[h] = -1;
         st.ntests[h] = 0;
     }
@@ -331,11 +396,13 @@ __device__ __forceinline__ void raster_tile(
         else kend = B;
     }
     if (pl.resume) {
-        float T[2] = {1.0f, 1.0f}, C[3][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+        float T[P], C[3][P];
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int h = 0; h < P; ++h) {
+            T[h] = 1.0f;
+            C[0][h] = C[1][h] = C[2][h] = 0.0f;
             if ((inside >> h) & 1) {
-                const int64_t p = (int64_t)py * a.width + px + 4 * h;
+                const int64_t p = (int64_t)py * a.width + px0 + L::x(lane, h);
                 // the first pass's state: C in rgb, T in alpha (negative once the
                 // pixel stopped), last
                 const float Ts = out_alpha[p];
@@ -346,26 +413,39 @@ __device__ __forceinline__ void raster_tile(
                 C[2][h] = out_rgb[3 * p + 2];
                 st.last[h] = out_last[p];
             }
-        st.T = pk2(T[0], T[1]);
-        st.C0 = pk2(C[0][0], C[0][1]);
-        st.C1 = pk2(C[1][0], C[1][1]);
-        st.C2 = pk2(C[2][0], C[2][1]);
+        }
+        st.T = L::put(T);
+        st.C0 = L::put(C[0]);
+        st.C1 = L::put(C[1]);
+        st.C2 = L::put(C[2]);
     }
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-        st.x[h] = (st.live >> h) & 1 ? (float)(px + 4 * h) + 0.5f : __uint_as_float(0x7fc00000u);
+    for (int h = 0; h < P; ++h)
+        st.x[h] = (st.live >> h) & 1 ? (float)(px0 + L::x(lane, h)) + 0.5f : __uint_as_float(0x7fc00000u);
     sh.init_pad();
-    FwdSpan<TILE, COUNT, LAZY, R> span{sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty, st};
+    FwdSpan<TILE, P, COUNT, LAZY, R> span{sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty, st};
     // saving for the backward: the sorted chunks go back into the stream
     const int32_t end =
         walk_tile<TILE, LAZY, TB::NT>(words, off, t, K, kbegin, kend, cap, ws, span, out_end ? words : nullptr);
     if (out_end && threadIdx.x == 0) out_end[t] = end;
     if (out_wend) {
-        // per warp, the stream position past the entry that stopped its last
-        // pixel (the tile's end when one of its pixels never stopped): the
-        // backward has nothing to do for the warp at or beyond it
-        const int32_t m = __reduce_max_sync(0xffffffffu, !inside ? INT32_MIN : (st.live ? end : st.stop + 1));
-        if (lane == 0) out_wend[(int64_t)t * TB::NW + (threadIdx.x >> 5)] = m == INT32_MIN ? 0 : min(m, end);
+        // per 8 x 8 block (a warp of the backward), the stream position past the
+        // entry that stopped its last pixel (the tile's end when one of its
+        // pixels never stopped): the backward has nothing to do for the block
+        // at or beyond it
+        const int32_t m = __reduce_max_sync(0xffffffffu, !inside ? 0 : (st.live ? end : min(st.stop + 1, end)));
+        constexpr int NB = TileBlocks<TILE, 2>::NW;
+        const int blk = TB::y0() / 8 * TB::COLS + TB::x0() / 8;
+        if constexpr (P == 2) {
+            if (lane == 0) out_wend[(int64_t)t * NB + blk] = m;
+        } else {
+            __shared__ int32_t s_wend[NB];
+            if (threadIdx.x < NB) s_wend[threadIdx.x] = 0;
+            __syncthreads();
+            if (lane == 0) atomicMax(&s_wend[blk], m);
+            __syncthreads();
+            if (threadIdx.x < NB) out_wend[(int64_t)t * NB + threadIdx.x] = s_wend[threadIdx.x];
+        }
     }
     bool unfinished = false;
     if (pl.flag && kend < K) {
@@ -403,37 +483,39 @@ __device__ __forceinline__ void raster_tile(
             pl.needed[t] = need;
         }
     }
-    float T[2], C0[2], C1[2], C2[2];
-    upk2(st.T, T[0], T[1]);
-    upk2(st.C0, C0[0], C0[1]);
-    upk2(st.C1, C1[0], C1[1]);
-    upk2(st.C2, C2[0], C2[1]);
+    float T[P], C0[P], C1[P], C2[P];
+    L::get(st.T, T);
+    L::get(st.C0, C0);
+    L::get(st.C1, C1);
+    L::get(st.C2, C2);
     if (unfinished) {  // the transmittance signed by termination
-        T[0] = st.live & 1 ? T[0] : -T[0];
-        T[1] = st.live & 2 ? T[1] : -T[1];
-    }
-    // The lanes of two neighbouring rows exchange one pixel each, so that
-    // eight lanes hold eight neighbouring pixels of one row (96 bytes of rgb)
-    // in each of the two store rounds: a lane of an even row then holds its
-    // pixel x of that row and of the next, one of an odd row its pixel x + 4
-    // of the row before and of its own.
-    const bool odd = (lane & 4) != 0;
-    auto pair_rows = [&](auto& v) {
-        const auto mine = odd ? v[0] : v[1];
-        const auto other = __shfl_xor_sync(0xffffffffu, mine, 4);
-        if (odd) v[0] = other;
-        else v[1] = other;
-    };
-    pair_rows(T);
-    pair_rows(C0);
-    pair_rows(C1);
-    pair_rows(C2);
-    pair_rows(st.last);
-    if (COUNT) pair_rows(st.ntests);
-    const int ox = tx * TILE + TB::x0() + (lane & 3) + (odd ? 4 : 0);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int oy = ty * TILE + TB::y0() + ((lane >> 2) & ~1) + h;
+        for (int h = 0; h < P; ++h) T[h] = (st.live >> h) & 1 ? T[h] : -T[h];
+    }
+    const bool odd = (lane & 4) != 0;
+    if constexpr (P == 2) {
+        // The lanes of two neighbouring rows exchange one pixel each, so that
+        // eight lanes hold eight neighbouring pixels of one row (96 bytes of
+        // rgb) in each of the two store rounds: a lane of an even row then
+        // holds its pixel x of that row and of the next, one of an odd row its
+        // pixel x + 4 of the row before and of its own.
+        auto pair_rows = [&](auto& v) {
+            const auto mine = odd ? v[0] : v[1];
+            const auto other = __shfl_xor_sync(0xffffffffu, mine, 4);
+            if (odd) v[0] = other;
+            else v[1] = other;
+        };
+        pair_rows(T);
+        pair_rows(C0);
+        pair_rows(C1);
+        pair_rows(C2);
+        pair_rows(st.last);
+        if (COUNT) pair_rows(st.ntests);
+    }
+    const int ox = px0 + (P == 2 ? (lane & 3) + (odd ? 4 : 0) : L::x(lane, 0));
+#pragma unroll
+    for (int h = 0; h < P; ++h) {
+        const int oy = P == 2 ? py0 + ((lane >> 2) & ~1) + h : py;
         if (ox >= a.width || oy >= a.height) continue;
         const int64_t p = (int64_t)oy * a.width + ox;
         if (unfinished) {
@@ -483,18 +565,20 @@ __device__ __forceinline__ int ordered_tile(const TileOrder& o, int32_t k)
 }
 
 // Threads of a tile's block and the blocks an SM holds: 16 x 16 tiles' seven
-// blocks of 128 threads fill the shared memory (31.8 KB each).
-template <int TILE>
-constexpr int raster_threads() { return TileBlocks<TILE>::NT; }
-template <int TILE>
-constexpr int raster_min_blocks() { return TILE == 16 ? 7 : TILE == 8 ? 16 : 2; }
-// ... and with rounds of four
-template <int TILE>
-constexpr int raster_wide_blocks() { return TILE == 16 ? 4 : TILE == 8 ? 16 : 1; }
+// blocks of 128 threads fill the shared memory (32.9 KB each).
+template <int TILE, int P = 2>
+constexpr int raster_threads() { return TileBlocks<TILE, P>::NT; }
+template <int TILE, int P = 2>
+constexpr int raster_min_blocks()
+{
+    return P == 2 ? (TILE == 16 ? 7 : TILE == 8 ? 16 : 2) : (TILE == 16 ? 3 : 12);
+}
+// Entries a round of composite_batch: four where a warp's registers allow it.
+template <int TILE, int P = 2>
+constexpr int raster_round() { return P == 1 || TILE == 8 ? 4 : 2; }
 
-template <int TILE, bool COUNT, bool LAZY, int R>
-__global__ void __launch_bounds__(raster_threads<TILE>(),
-                                  COUNT ? 1 : R == 4 ? raster_wide_blocks<TILE>() : raster_min_blocks<TILE>())
+template <int TILE, int P, bool COUNT, bool LAZY>
+__global__ void __launch_bounds__(raster_threads<TILE, P>(), COUNT ? 1 : raster_min_blocks<TILE, P>())
 k_raster(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o_z, const float4* __restrict__ rgbv,
          uint64_t* words, const int32_t* __restrict__ off, RasterArgs a, int cullmode,
          float* __restrict__ out_rgb, float* __restrict__ out_alpha, int32_t* __restrict__ out_last,
@@ -502,12 +586,13 @@ k_raster(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o_z, con
          int32_t* __restrict__ out_end, const PlanView pl, int cap, int32_t* __restrict__ out_wend, const TileOrder ord)
 {
     grid_dependency_sync();
-    __shared__ RasterShared<TILE> sh;
+    __shared__ RasterShared<TILE, P> sh;
     __shared__ WalkShared<TILE, LAZY> ws;
     const int t = ord.lists ? ordered_tile(ord, (int32_t)blockIdx.x) : (int)blockIdx.x;
     if (t < 0) return;
-    raster_tile<TILE, COUNT, LAZY, R>(t, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode, out_rgb, out_alpha,
-                                   out_last, out_ntests, ops_total, out_T, out_end, pl, cap, out_wend);
+    raster_tile<TILE, P, COUNT, LAZY, raster_round<TILE, P>()>(t, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode,
+                                                               out_rgb, out_alpha, out_last, out_ntests, ops_total,
+                                                               out_T, out_end, pl, cap, out_wend);
 }
 
 // The completing pass of a planned frame: persistent blocks take the listed
@@ -522,7 +607,7 @@ k_raster_listed(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o
                 const int32_t* __restrict__ list, int cap)
 {
     grid_dependency_sync();
-    __shared__ RasterShared<TILE> sh;
+    __shared__ RasterShared<TILE, 2> sh;
     __shared__ WalkShared<TILE, true> ws;
     PlanView pl;
     pl.bins = plan;
@@ -530,7 +615,7 @@ k_raster_listed(const float4* __restrict__ xy_ab, const float4* __restrict__ c_o
     const int32_t nl = list[0];
     for (int32_t k = blockIdx.x; k < nl; k += gridDim.x) {
         const int t = list[1 + k];
-        raster_tile<TILE, false, true, TILE == 8 ? 4 : 2>(t, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode, out_rgb,
+        raster_tile<TILE, 2, false, true, raster_round<TILE>()>(t, sh, ws, xy_ab, c_o_z, rgbv, words, off, a, cullmode, out_rgb,
                                               out_alpha, out_last, nullptr, nullptr, out_T, out_end, pl, cap);
         __syncthreads();  // the next tile reuses the shared memory
     }
@@ -567,7 +652,7 @@ template <int TILE, bool LAZY>
 __global__ void __launch_bounds__(raster_threads<TILE>(), raster_min_blocks<TILE>())
 k_raster_views(const __grid_constant__ ViewRasterSet vs, const TileOrder order, int32_t* __restrict__ counter)
 {
-    __shared__ RasterShared<TILE> sh;
+    __shared__ RasterShared<TILE, 2> sh;
     __shared__ WalkShared<TILE, LAZY> ws;
     __shared__ int32_t s_item;
     for (;;) {
@@ -582,21 +667,38 @@ k_raster_views(const __grid_constant__ ViewRasterSet vs, const TileOrder order, 
         __syncthreads();
         if (item < 0) break;
         const ViewRasterSet::View& V = vs.v[view_of(vs, item)];
-        raster_tile<TILE, false, LAZY, 2>(item - V.item0, sh, ws, V.xy_ab, V.c_o_z, V.rgbv, V.words, V.off, V.a,
+        raster_tile<TILE, 2, false, LAZY, raster_round<TILE>()>(item - V.item0, sh, ws, V.xy_ab, V.c_o_z, V.rgbv, V.words, V.off, V.a,
                                               V.cullmode, V.rgb, V.alpha, V.last, nullptr, nullptr, nullptr, nullptr,
                                               PlanView(), V.cap);
     }
 }
 
-template <int TILE>
-static bool resident(const gs_ctx* ctx, int64_t T)
+// Whether a frame of T tiles goes by one pixel a lane.  A frame of few tiles
+// lasts as long as its deepest tile, whose warps wait for their own results:
+// twice the warps of one pixel a lane, each with rounds of four and the
+// registers of twelve (8 x 8) or three (16 x 16) blocks an SM, take it down
+// faster.  Past some tiles an SM the frame is bound by issue, where two pixels
+// a lane need fewer instructions.  Measured, two pixels a lane / one, us:
+// 16 x 16 tiles, Gaussians in clusters, 336 tiles 291 / 182, 475 tiles 168 /
+// 102, 1200 tiles 65 / 47, 2040 tiles 90 / 88; spread evenly, 475 tiles 49 /
+// 41, 1200 tiles 61 / 63, 1900 tiles 93 / 98; seen from inside, 1900 tiles 72 /
+// 86.  The plain raster, whose warps visit every entry of a tile: 300 tiles
+// 180 / 135, 475 tiles 158 / 145 and, even, 76 / 80, 1200 tiles 147 / 156 and
+// 102 / 135.  8 x 8 tiles: 840 tiles 178 / 115, 2646 tiles 63 / 47, 8160 tiles
+// 94 / 88 (even, 7500 tiles 102 / 100; plain, 4800 tiles 96 / 95).  32 x 32
+// tiles' 32 warps have to share one block's registers: 80 tiles 233 / 223,
+// plain 489 / 561, 300 tiles 80 / 94.
+static bool one_pixel(const gs_ctx* ctx, int tile, bool plain, int64_t T)
 {
-    return T <= (int64_t)ctx->num_sms * raster_wide_blocks<TILE>();
+    const int64_t per_sm = tile == 8 ? 48 : tile == 16 ? (plain ? 3 : 10) : 0;
+    return T <= per_sm * ctx->num_sms;
 }
 
+// Whether a frame's tiles are all resident at once (their order is then of no use).
 bool raster_resident(const gs_ctx* ctx, int tile, int64_t T)
 {
-    return tile == 8 ? resident<8>(ctx, T) : tile == 32 ? resident<32>(ctx, T) : resident<16>(ctx, T);
+    return T <= (int64_t)ctx->num_sms *
+                    (tile == 8 ? raster_min_blocks<8, 1>() : tile == 16 ? raster_min_blocks<16, 1>() : raster_min_blocks<32>());
 }
 
 template <int TILE>
@@ -606,19 +708,12 @@ static cudaError_t launch_tile(const gs_ctx* ctx, bool count, bool lazy, unsigne
                                float* final_T, int32_t* tile_end, const PlanView& pl, int cap, int32_t* warp_end,
                                const TileOrder& order)
 {
-    // Rounds of four when all the frame's tiles are resident at once (each
-    // SM's few warps wait for their own results, and a wide round has twice as
-    // many of them in flight): 256 tiles of 16 x 16, 20.4 us against 22.4;
-    // past that rounds of two, whose smaller register share holds seven blocks
-    // an SM instead of four (8160 tiles: 229 us against 244; 3600 tiles, global:
-    // 276 against 331).  8 x 8 tiles have one warp a block, as many blocks
-    // either way, and always go by four (2646 tiles: 63.4 us against 69.5).
-    const bool wide = TILE == 8 || raster_resident(ctx, TILE, grid);
-    constexpr int RN = TILE == 8 ? 4 : 2;
-    const auto kern = count  ? (lazy ? k_raster<TILE, true, true, RN> : k_raster<TILE, true, false, RN>)
-                      : wide ? (lazy ? k_raster<TILE, false, true, 4> : k_raster<TILE, false, false, 4>)
-                             : (lazy ? k_raster<TILE, false, true, RN> : k_raster<TILE, false, false, RN>);
-    return launch_k(ctx, kern, grid, raster_threads<TILE>(), 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, off, a, cull,
+    constexpr int ONE = TILE == 32 ? 2 : 1;
+    const bool one = !count && one_pixel(ctx, TILE, (cull & kPlain) != 0, grid);
+    const auto kern = count ? (lazy ? k_raster<TILE, 2, true, true> : k_raster<TILE, 2, true, false>)
+                      : one ? (lazy ? k_raster<TILE, ONE, false, true> : k_raster<TILE, ONE, false, false>)
+                            : (lazy ? k_raster<TILE, 2, false, true> : k_raster<TILE, 2, false, false>);
+    return launch_k(ctx, kern, grid, one ? raster_threads<TILE, ONE>() : raster_threads<TILE>(), 0, st, pv.xy_ab, pv.c_o_z, pv.rgb, words, off, a, cull,
                     rgb, alpha, last, ntests, ops, final_T, tile_end, pl, cap, warp_end, order);
 }
 

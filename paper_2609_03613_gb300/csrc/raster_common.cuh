@@ -86,25 +86,26 @@ struct RasterArgs {
     int32_t gid_base = 0;  // stream words hold gid_base + gid (the last-id output subtracts it)
 };
 
-// A warp owns a block of 8 x 8 pixels of the tile, two a lane.  Blocks are laid
-// out TILE/8 wide and tall, warps row-major over them; the block of the tile
-// has one warp for each.
-template <int TILE>
+// A warp owns a block of 8 x 4P pixels of the tile, P a lane.  Blocks are laid
+// out TILE/8 wide and TILE/4P tall, warps row-major over them; the block of
+// the tile has one warp for each.
+template <int TILE, int P = 2>
 struct TileBlocks {
-    static constexpr int COLS = TILE / 8, ROWS = TILE / 8;
-    static constexpr int NW = COLS * ROWS;    // warps of the tile
-    static constexpr int NT = 32 * NW;        // threads of the tile
+    static constexpr int BH = 4 * P;                     // rows of a block
+    static constexpr int COLS = TILE / 8, ROWS = TILE / BH;
+    static constexpr int NW = COLS * ROWS;               // warps of the tile
+    static constexpr int NT = 32 * NW;                   // threads of the tile
     __device__ static int x0() { return ((threadIdx.x >> 5) % COLS) * 8; }
-    __device__ static int y0() { return ((threadIdx.x >> 5) / COLS) * 8; }
+    __device__ static int y0() { return ((threadIdx.x >> 5) / COLS) * BH; }
 };
 
 // Entries staged per batch.
 template <int TILE>
 constexpr int raster_batch() { return TILE == 8 ? 128 : 256; }
 
-template <int TILE>
+template <int TILE, int P = 2>
 struct RasterShared {
-    using TB = TileBlocks<TILE>;
+    using TB = TileBlocks<TILE, P>;
     static constexpr int BATCH = raster_batch<TILE>();
     float4 a[BATCH + 1];  // {mx, my, a/2, b}; the last slot of each array is a
     float4 b[BATCH + 1];  // {c/2, o, tau, gid bits}        zero record, which no
@@ -123,8 +124,8 @@ struct RasterShared {
 // The staged entries (of cnt) whose warp mask admits the calling warp, in
 // stage order, into sh.list[warp], followed by three references to the zero
 // record (a whole round of two or four); returns their count.  Whole warp.
-template <int TILE>
-__device__ __forceinline__ int warp_strip_list(RasterShared<TILE>& sh, int cnt)
+template <int TILE, int P>
+__device__ __forceinline__ int warp_strip_list(RasterShared<TILE, P>& sh, int cnt)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int nw = 0;
@@ -135,26 +136,26 @@ __device__ __forceinline__ int warp_strip_list(RasterShared<TILE>& sh, int cnt)
         if (mine) sh.list[warp][nw + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(16 * j);
         nw += __popc(bal);
     }
-    if (lane < 3) sh.list[warp][nw + lane] = (uint16_t)(16 * RasterShared<TILE>::BATCH);
+    if (lane < 3) sh.list[warp][nw + lane] = (uint16_t)(16 * RasterShared<TILE, P>::BATCH);
     __syncwarp();
     return nw;
 }
 
 // Warp mask of an entry: bit w is set when the entry's alpha >= 1/255
 // ellipse (the tile cull's bound Q(d) <= tau / margin, d = mean - pixel
-// centre, widened as there) reaches a pixel centre of warp w's 8 x 8 block of
-// the tile (origin x0, y0).  Per band of eight pixel rows the ellipse's
+// centre, widened as there) reaches a pixel centre of warp w's block of the
+// tile (origin x0, y0).  Per band of a block's pixel rows the ellipse's
 // x-extent over the band's centre rows (the row-span geometry of the bin
 // stage: band ends and the ellipse's leftmost / rightmost points) is widened
 // by 5e-3 relative + 0.05 px and tested against each block's centre columns,
 // so a warp never skips a pixel the entry can reach.  The geometry takes the
 // hardware's approximate division and square root (relative errors near
 // 2^-22, far inside the widening).
-template <int TILE>
+template <int TILE, int P>
 __device__ __forceinline__ uint32_t strip_mask(float mx, float my, float ha, float hb, float hc, float tau,
                                                float margin, float x0, float y0)
 {
-    using WB = TileBlocks<TILE>;
+    using WB = TileBlocks<TILE, P>;
     constexpr int NWT = WB::NW;
     const uint32_t all = NWT >= 32 ? 0xffffffffu : ((1u << NWT) - 1u);
     if (!(margin > 0.0f)) return all;
@@ -172,7 +173,7 @@ __device__ __forceinline__ uint32_t strip_mask(float mx, float my, float ha, flo
     uint32_t m = 0u;
 #pragma unroll
     for (int by = 0; by < WB::ROWS; ++by) {
-        float yl = my - (y0 + (float)(8 * by) + 7.5f), yh = my - (y0 + (float)(8 * by) + 0.5f);
+        float yl = my - (y0 + (float)(WB::BH * (by + 1)) - 0.5f), yh = my - (y0 + (float)(WB::BH * by) + 0.5f);
         yl = yl - (0.05f + 5e-3f * fabsf(yl));
         yh = yh + (0.05f + 5e-3f * fabsf(yh));
         const float ya = fmaxf(yl, -dymax), yb = fminf(yh, dymax);
@@ -204,7 +205,7 @@ constexpr int kPlain = 4;      // neither: the plain raster
 // q = c_o_z[g] and colour c = rgbv[g]: {mx, my, a/2, b}, {c/2, o, tau, gid
 // bits} and the colour with the warp mask in .w (zero when the tile cull
 // drops the entry: no warp's list admits it).
-template <int TILE>
+template <int TILE, int P>
 __device__ __forceinline__ void stage_record(uint32_t g, const float4& p, const float4& q, float4 c, int cullmode,
                                              int tx, int ty, float4& A, float4& B, float4& C)
 {
@@ -216,8 +217,8 @@ __device__ __forceinline__ void stage_record(uint32_t g, const float4& p, const 
     bool keep = true;
     if (cullmode & kCullTile)
         keep = !tile_culled(A.x, A.y, A.z, A.w, B.x, q.w, c.w, (float)(tx * TILE), (float)(ty * TILE), (float)TILE);
-    const uint32_t m = (cullmode & kCullWarp) ? strip_mask<TILE>(A.x, A.y, A.z, A.w, B.x, q.w, c.w,
-                                                                     (float)(tx * TILE), (float)(ty * TILE))
+    const uint32_t m = (cullmode & kCullWarp) ? strip_mask<TILE, P>(A.x, A.y, A.z, A.w, B.x, q.w, c.w,
+                                                                        (float)(tx * TILE), (float)(ty * TILE))
                                               : 0xffffffffu;
     c.w = __uint_as_float(keep ? m : 0u);
     C = c;
@@ -228,13 +229,13 @@ __device__ __forceinline__ void stage_record(uint32_t g, const float4& p, const 
 // the colour with the warp mask in .w (zero for an entry the tile cull
 // drops).  Returns the number staged (block-uniform); the caller
 // synchronises the block before reading sh.
-template <int TILE>
+template <int TILE, int P>
 __device__ __forceinline__ int stage_batch(const uint64_t* src, int32_t b0, int32_t n_entries,
-                                           RasterShared<TILE>& sh, const float4* __restrict__ xy_ab,
+                                           RasterShared<TILE, P>& sh, const float4* __restrict__ xy_ab,
                                            const float4* __restrict__ c_o_z, const float4* __restrict__ rgbv,
                                            int cullmode, int tx, int ty)
 {
-    using SH = RasterShared<TILE>;
+    using SH = RasterShared<TILE, P>;
     const int cnt = min(SH::BATCH, n_entries - b0);
     // entry i of the batch goes to slot i: the tile cull and the warp mask
     // leave a zero mask, which no warp's list admits (stream order is kept
@@ -242,7 +243,7 @@ __device__ __forceinline__ int stage_batch(const uint64_t* src, int32_t b0, int3
     auto put = [&](int i) {
         const uint32_t g = (uint32_t)(src[b0 + i] & 0xffffffffull);
         float4 A, B, C;
-        stage_record<TILE>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
+        stage_record<TILE, P>(g, __ldg(xy_ab + g), __ldg(c_o_z + g), __ldg(rgbv + g), cullmode, tx, ty, A, B, C);
         sh.a[i] = A;
         sh.b[i] = B;
         sh.c[i] = C;
@@ -258,8 +259,10 @@ __device__ __forceinline__ int stage_batch(const uint64_t* src, int32_t b0, int3
 // Shared memory of the tile walk.
 template <int TILE, bool LAZY>
 struct WalkShared {
+    static constexpr int LOG = TILE == 8 ? 7 : 8;  // buckets of a long segment
     uint64_t sort[LAZY ? raster_sort_cap(TILE) : 1];
     int32_t off[LAZY ? GS_MAX_K + 1 : 1];
+    uint16_t boff[LAZY ? (1 << LOG) + 1 : 1];
 };
 
 // The sorted position of word `key`, entry i of the chunk held in ws.sort
@@ -293,8 +296,8 @@ __device__ __forceinline__ int chunk_rank(const WS& ws, int i, uint64_t key, int
 // consecutive segments of at most `cap` entries (and at most one batch), whose
 // words are loaded into shared memory, ranked within their segments and
 // staged straight at their sorted slots; a single longer segment of up to
-// raster_sort_cap(TILE) entries is sorted there by the block and handed over
-// as a run, one beyond that was sorted before the raster and is handed over
+// raster_sort_cap(TILE) entries is put in bucket order there and staged batch
+// by batch, one beyond that was sorted before the raster and is handed over
 // in place.  The chunks are the tile's repair bins.  ws.off holds all K + 1
 // bin offsets of the tile on return (LAZY).
 // Returns the stream index at which the walk ended: the end of the walked
@@ -386,20 +389,41 @@ __device__ __forceinline__ int32_t walk_tile(const uint64_t* words, const int32_
                 span.composite_staged(n, at);  // termination just counted above
                 continue;
             }
-            // one long segment: sorted in shared memory by the block, or before
-            // the raster (in depth buckets ranked batch by batch, as
-            // k_sort_listed does, measured no faster here: 164 against 162 us
-            // for 3M Gaussians seen from inside a cluster)
-            const bool sorted = n > raster_sort_cap(TILE);
-            if (!sorted) {
-                for (int i = threadIdx.x; i < n; i += NT) ws.sort[i] = __ldcs(wl + at + i);
-                __syncthreads();
-                bitonic_mem(ws.sort, n, threadIdx.x, NT, SyncBlock{});
-                if (writeback)
-                    for (int i = threadIdx.x; i < n; i += NT) writeback[at + i] = ws.sort[i];
+            if (n > raster_sort_cap(TILE)) {  // sorted before the raster
+                const int32_t r = span(words + at, n, true, at);
+                if (r >= 0) return at + r;
+                find();
+                continue;
             }
-            const int32_t r = span(sorted ? words + at : ws.sort, n, true, at);  // termination just counted above
-            if (r >= 0) return at + r;
+            // one long segment, into shared memory in order of depth buckets
+            // (or sorted by the network): its batches are then staged one by
+            // one, each thread ranking the words of the buckets a batch meets,
+            // so that batches past the tile's termination are never ranked
+            // (119 x 657 pixels of a few deep tiles: raster 303 -> 252 us with
+            // four warps a tile; 3M Gaussians seen from inside 162 -> 164)
+            using WS = WalkShared<TILE, LAZY>;
+            BucketMap map;
+            const bool ranked = block_buckets<NT, WS::LOG>(words + at, n, ws.sort, span.scratch(),
+                                                           span.scratch() + (1 << WS::LOG), ws.boff, map);
+            if (!ranked) bitonic_mem(ws.sort, n, threadIdx.x, NT, SyncBlock{});
+            if (writeback)
+                for (int i = threadIdx.x; i < n; i += NT) {
+                    const uint64_t w = ws.sort[i];
+                    writeback[at + (ranked ? bucket_rank(ws.sort, ws.boff, map, w) : i)] = w;
+                }
+            for (int b0 = 0; b0 < n; b0 += Span::kBatch) {
+                if (b0 > 0 && __syncthreads_count(span.done()) == NT) return at + b0;
+                const int b1 = min(b0 + Span::kBatch, n);
+                const int i0 = ranked ? ws.boff[map.of(ws.sort[b0])] : b0;
+                const int i1 = ranked ? ws.boff[map.of(ws.sort[b1 - 1]) + 1] : b1;
+                for (int i = i0 + (int)threadIdx.x; i < i1; i += NT) {
+                    const uint64_t w = ws.sort[i];
+                    const int r = ranked ? bucket_rank(ws.sort, ws.boff, map, w) : i;
+                    if (r >= b0 && r < b1) span.stage_at(r - b0, (uint32_t)w);
+                }
+                __syncthreads();
+                span.composite_staged(b1 - b0, at + b0);
+            }
             find();
         }
         return ws.off[kend];

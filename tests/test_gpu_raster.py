@@ -28,13 +28,39 @@ def assert_image(mode, sc, cam, tile, K, ref, **cfg):
 
 
 @pytest.mark.parametrize("tile", [8, 16, 32])
-@pytest.mark.parametrize("w,h", [(1, 1), (4, 7), (5, 8), (9, 17), (36, 33), (512, 304), (513, 304)])
-def test_ragged_sizes_and_round_widths(w, h, tile):
+@pytest.mark.parametrize("w,h", [(1, 1), (4, 7), (5, 8), (9, 17), (36, 33), (384, 304), (385, 304),
+                                 (608, 768), (609, 768)])
+def test_ragged_sizes_and_pixels_a_lane(w, h, tile):
     sc = scenes.mixture_scene(3000, 91)
     cam = scenes.hd_camera(width=w, height=h, f=max(w, h) * 0.6)
     ref = O.render(sc, cam, tile, bg=(0.1, 0.2, 0.3))[3]
     for mode in ("exact", "global"):
         assert_image(mode, sc, cam, tile, 64 if mode == "exact" else 1, ref)
+
+
+@pytest.mark.parametrize("w,h", [(640, 608), (641, 608)])
+def test_both_sides_of_the_rule(w, h):
+    # 1520 tiles go by one pixel a lane, 1558 by two: the image, and the ends
+    # of the 8 x 8 blocks that the backward starts from (it skips what lies
+    # beyond, so a frame's gradients equal those of the stages, which walk on
+    # to the tile's end, up to the order of their float32 atomics)
+    sc = scenes.mixture_scene(60_000, 92)
+    cam = scenes.hd_camera(width=w, height=h, f=400.0)
+    ref = O.render(sc, cam, 16, bg=(0.1, 0.2, 0.3))[3]
+    assert_image("exact", sc, cam, 16, 64, ref)
+    dC, dA = (torch.from_numpy(x).cuda() for x in scenes.incoming_grads(h, w, seed=3))
+    ds = G.DeviceScene.from_numpy(sc)
+    ctx = G.Context("exact")
+    ctx.render(ds, cam, flags=G.RENDER_SAVE)
+    got = G.grad_fields(ctx.render_bwd(dC, dA), sc.n)
+    proj = ctx.project(ds, cam)
+    isect, m_cap, m_dev, _ = ctx.tile_intersect(proj, sc.n, cam)
+    words, offsets, _ = ctx.sort_or_bin(proj, ds.scales, sc.n, cam, isect, m_cap, m_dev)
+    saved = ctx.rasterize_fwd(proj, sc.n, cam, words, offsets, save=True)[3]
+    want = G.grad_fields(ctx.rasterize_bwd(proj, sc.n, cam, words, offsets, saved, dC, dA), sc.n)
+    assert ctx.error() == 0
+    for k in got:
+        np.testing.assert_allclose(got[k].cpu(), want[k].cpu(), rtol=1e-5, atol=1e-6 * float(want[k].abs().max()))
 
 
 @pytest.mark.parametrize("depths", ["spread", "equal", "skewed"])
