@@ -66,8 +66,8 @@ __global__ void k_group_counts(const int32_t* __restrict__ goff, int64_t n, int 
 // goff[G] - base <= j < goff[G + 1] - base, found by binary search over the
 // view's items (one thread per sample, grid.y = the view).
 __global__ void __launch_bounds__(256)
-k_group_sample_gids(const int32_t* __restrict__ goff, const GroupViews gv, const ViewCount* __restrict__ vc, int S,
-                    uint32_t* __restrict__ out)
+k_group_sample_keys(const int32_t* __restrict__ goff, const float4* __restrict__ c_o_z, const GroupViews gv,
+                    const ViewCount* __restrict__ vc, int S, uint32_t* __restrict__ out)
 {
     const int v = blockIdx.y;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -81,7 +81,7 @@ k_group_sample_gids(const int32_t* __restrict__ goff, const GroupViews gv, const
         if (goff[mid] <= j) lo = mid;
         else hi = mid - 1;
     }
-    out[(int64_t)v * S + i] = (uint32_t)lo;
+    out[(int64_t)v * S + i] = __float_as_uint(c_o_z[lo].z);
 }
 
 // One block per view: Alg. 2 over the view's samples, its bin parameters.
@@ -93,7 +93,7 @@ k_group_depth_range(const float4* __restrict__ c_o_z, const GroupViews gv, const
     a.near_plane = gv.near_plane[v];
     a.far_plane = gv.far_plane[v];
     a.K = gv.K[v];
-    depth_range_block(c_o_z, nullptr, GidFromSamples{samples + (int64_t)v * a.S}, vc[v].M, a, bp + v);
+    depth_range_block(c_o_z, nullptr, KeyFromSamples{samples + (int64_t)v * a.S}, vc[v].M, a, bp + v);
 }
 
 // The row spans of k_row_spans (tiles.cu) for the group's items: each lane's
@@ -426,18 +426,8 @@ int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m
     k_group_counts<<<1, 32, 0, st>>>(gc->d_goff, gv.n, gv.nv, S, s.vc, s.m_views);
     if (h_m_views)
         GS_CUDA_TRY(cudaMemcpyAsync(h_m_views, s.m_views, (size_t)gv.nv * 8, cudaMemcpyDeviceToHost, st));
-    if (N > 0) k_group_sample_gids<<<dim3((unsigned)((S + 255) / 256), (unsigned)gv.nv), 256, 0, st>>>(gc->d_goff, gv, s.vc, S, s.samples);
-    DrArgs a;
-    a.S = S;
-    a.near_shift = 0;  // EXACT mode
-    a.near_alpha = gc->cfg.near_alpha;
-    a.near_gamma = gc->cfg.near_gamma;
-    a.p_lo = gc->cfg.p_lo;
-    a.p_hi = gc->cfg.p_hi;
-    a.pad = gc->cfg.pad;
-    a.eps = gc->cfg.eps;
-    a.near_plane = a.far_plane = 0.0f;
-    a.K = 0;  // set per view
+    if (N > 0) k_group_sample_keys<<<dim3((unsigned)((S + 255) / 256), (unsigned)gv.nv), 256, 0, st>>>(gc->d_goff, pv.c_o_z, gv, s.vc, S, s.samples);
+    const DrArgs a = dr_args(gc->cfg, 0, 0.0f, 0.0f, 0);  // EXACT mode; planes and K are set per view
     k_group_depth_range<<<(unsigned)gv.nv, kDrThreads, 0, st>>>(pv.c_o_z, gv, s.vc, s.samples, a, s.bp);
     gc->launches += N > 0 ? 3 : 2;
     // row spans and per-row difference counts, then the offsets

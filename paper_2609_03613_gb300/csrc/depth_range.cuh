@@ -11,14 +11,36 @@ namespace gs {
 constexpr int kDrThreads = 1024;
 constexpr int kDrMaxS = 8192;
 
+constexpr int kDrBits = 11;            // bits of a radix pass
+constexpr int kDrBins = 1 << kDrBits;  // 64 a warp of the block
+
 struct DrArgs {
     float near_plane, far_plane;
     int S;
     int near_shift;
     float near_alpha, near_gamma;
-    float p_lo, p_hi, pad, eps;
+    float pad, eps;
+    double lo, hi;  // the percentiles as fractions of 1
     int K;
 };
+
+// Of a context's settings; near_shift only where the mode shifts the keys.
+inline DrArgs dr_args(const gs_config& c, int near_shift, float near_plane, float far_plane, int K)
+{
+    DrArgs a;
+    a.near_plane = near_plane;
+    a.far_plane = far_plane;
+    a.S = c.sample_count;
+    a.near_shift = near_shift;
+    a.near_alpha = c.near_alpha;
+    a.near_gamma = c.near_gamma;
+    a.pad = c.pad;
+    a.eps = c.eps;
+    a.lo = (double)c.p_lo / 100.0;
+    a.hi = (double)c.p_hi / 100.0;
+    a.K = K;
+    return a;
+}
 
 __device__ __forceinline__ float zkey_of(float z, const float* __restrict__ scales, uint32_t g, float a, float gm)
 {
@@ -28,56 +50,49 @@ __device__ __forceinline__ float zkey_of(float z, const float* __restrict__ scal
     return z - fminf(a * smax, gm * z);
 }
 
-__device__ __forceinline__ int64_t rank_of(float p, int64_t n)
+__device__ __forceinline__ int rank_of(double p, int n)
 {
-    int64_t k = (int64_t)ceil((double)p / 100.0 * (double)n);
-    if (k < 1) k = 1;
-    if (k > n) k = n;
-    return k;
+    const double k = ceil(p * (double)n);
+    return k < 1.0 ? 1 : k > (double)n ? n : (int)k;
 }
 
 // Bin parameters from [zmin, zmax]: z'min = max(zmin, eps),
 // z'max = max(zmax, z'min + 1e-6), lmin/lmax their logs, and K-1 log-spaced
-// split depths exp(lmin + (lmax - lmin) k/K), kept non-decreasing.
+// split depths exp(lmin + (lmax - lmin) k/K), kept non-decreasing (a running
+// maximum).  By the block's first warp.
 __device__ __forceinline__ void write_bin_params(BinParams* bp, float zmin, float zmax, int K, float eps, int nsamples)
 {
-    __shared__ float s_l[2];
-    if (threadIdx.x == 0) {
-        const float zmn = fmaxf(zmin, eps);
-        const float zmx = fmaxf(zmax, zmn + 1e-6f);
-        s_l[0] = spec_log(zmn);
-        s_l[1] = spec_log(zmx);
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    const float zmn = fmaxf(zmin, eps);
+    const float zmx = fmaxf(zmax, zmn + 1e-6f);
+    const float l = spec_log(lane == 0 ? zmn : zmx);
+    const float lmin = __shfl_sync(0xffffffffu, l, 0), lmax = __shfl_sync(0xffffffffu, l, 1);
+    if (lane == 0) {
         bp->zmin = zmin;
         bp->zmax = zmax;
-        bp->lmin = s_l[0];
-        bp->lmax = s_l[1];
+        bp->lmin = lmin;
+        bp->lmax = lmax;
         bp->K = K;
         bp->nsamples = nsamples;
     }
-    __syncthreads();
-    __shared__ float s_split[GS_MAX_K];
-    const float lmin = s_l[0], lmax = s_l[1];
-    for (int k = 1 + threadIdx.x; k < K; k += blockDim.x) {
-        const float t = (float)k / (float)K;
-        s_split[k - 1] = spec_exp(lmin + (lmax - lmin) * t);
+    float carry = -INFINITY;
+    for (int k0 = 1; k0 < K; k0 += 32) {
+        const float t = (float)(k0 + lane) / (float)K;
+        float s = spec_exp(lmin + (lmax - lmin) * t);
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const float u = __shfl_up_sync(0xffffffffu, s, d);
+            if (lane >= d && s < u) s = u;
+        }
+        if (s < carry) s = carry;
+        carry = __shfl_sync(0xffffffffu, s, 31);
+        if (k0 + lane < K) bp->splits[k0 + lane - 1] = s;
     }
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int k = 1; k < K - 1; ++k)
-            if (s_split[k] < s_split[k - 1]) s_split[k] = s_split[k - 1];
-    __syncthreads();
-    for (int k = threadIdx.x; k < K - 1; k += blockDim.x) bp->splits[k] = s_split[k];
 }
 
-// ... or from a per-sample gid array (the batched views' sampling).
-struct GidFromSamples {
-    static constexpr bool kKeys = false;
-    const uint32_t* gid;  // indexed by sample number
-    __device__ uint32_t operator()(int64_t i, int64_t) const { return gid[i]; }
-};
-
-// ... or the samples' keys themselves (depth, or the near-shifted key, as
-// float bits), gathered by the wide sampling kernel.
+// The samples' keys themselves (depth, or the near-shifted key, as float
+// bits), gathered by a wide sampling kernel.
 struct KeyFromSamples {
     static constexpr bool kKeys = true;
     const uint32_t* key;  // indexed by sample number
@@ -93,62 +108,55 @@ __device__ __forceinline__ float sample_key(const float4* __restrict__ c_o_z, co
     return z;
 }
 
-// Rank search of one radix pass, by one warp: the digit d whose cumulative
-// count first reaches k (k >= 1), and k minus the counts below d, written by
-// the one lane that returns true.  Lane l holds digits 8l .. 8l+7.
-__device__ __forceinline__ bool warp_digit_select(const uint32_t* __restrict__ h, int64_t k, uint32_t* dsel,
-                                                  int64_t* krem)
+// The bin of h[0..64 * 32) whose cumulative count first reaches k (k >= 1),
+// by one warp: lane l's group is the 64 bins from 64 l on, group its count.
+// k is left less the counts before the bin.
+__device__ __forceinline__ uint32_t warp_bin_select(const uint32_t* __restrict__ h, uint32_t group, int& k)
 {
     const int lane = threadIdx.x & 31;
-    uint32_t c[8], sum = 0;
+    auto scan = [&](uint32_t v) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        c[j] = h[8 * lane + j];
-        sum += c[j];
-    }
-    uint32_t incl = sum;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t u = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += u;
-    }
-    const unsigned hit = __ballot_sync(0xffffffffu, (int64_t)incl >= k);
-    const int L = hit ? __ffs(hit) - 1 : 31;
-    const uint32_t before = __shfl_sync(0xffffffffu, incl - sum, L);
-    if (lane == L) {
-        int64_t kk = k - (int64_t)before;
-        uint32_t d = 8u * L + 7u;
-        for (int j = 0; j < 8; ++j) {
-            if ((int64_t)c[j] >= kk) {
-                d = 8u * L + j;
-                break;
-            }
-            kk -= c[j];
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, v, d);
+            if (lane >= d) v += u;
         }
-        *dsel = d;
-        *krem = kk;
-    }
-    return lane == L;
+        return v;
+    };
+    const uint32_t gi = scan(group);
+    const int L = __ffs(__ballot_sync(0xffffffffu, (int)gi >= k)) - 1;
+    k -= (int)__shfl_sync(0xffffffffu, gi - group, L);
+    const uint2 c = *reinterpret_cast<const uint2*>(h + 64 * L + 2 * lane);
+    const uint32_t bi = scan(c.x + c.y);
+    const int l = __ffs(__ballot_sync(0xffffffffu, (int)bi >= k)) - 1;
+    k -= (int)__shfl_sync(0xffffffffu, bi - c.x - c.y, l);
+    const int cx = (int)__shfl_sync(0xffffffffu, c.x, l);
+    const uint32_t bin = 64u * L + 2u * l + (k > cx ? 1u : 0u);
+    if (k > cx) k -= cx;
+    return bin;
 }
 
 // Alg. 2 by one block of kDrThreads threads over the first S' = min(S, M)
 // samples gid_of(i, floor(i M / S')) of M entries: the positive depths (or
 // near-shifted keys) clamped to [max(near, eps), far], their exact p_lo / p_hi
-// order statistics by radix select, padded by pad of the span; the bin
+// order statistics by radix select on the float bits (positive floats: bit
+// order = value order) above the least, padded by pad of the span; the bin
 // parameters of [zmin, zmax] are written to bp.
+//
+// One block and a chain of barriers: what it costs is latency, so each thread
+// keeps its samples in registers, a pass takes 11 bits (two or three passes),
+// the first counts once for both ranks, and every warp sums its 64 bins for
+// the two that select.  (Samples compacted in shared memory, passes of 8 bits,
+// splits kept monotone by one thread: 13.7 us a frame, now 7.5.)
 template <class GidOf>
 __device__ __forceinline__ void depth_range_block(const float4* __restrict__ c_o_z, const float* __restrict__ scales,
                                                   GidOf gid_of, int64_t M, const DrArgs& a, BinParams* bp)
 {
-    __shared__ uint32_t s_v[kDrMaxS];
-    __shared__ int s_n;
-    __shared__ uint32_t s_h[2][256];
+    static_assert(kDrBins == 64 * (kDrThreads / 32), "64 bins a warp");
+    __shared__ __align__(8) uint32_t s_h[2][kDrBins];
+    __shared__ uint32_t s_red[3][kDrThreads / 32];
     __shared__ uint32_t s_pref[2];
-    __shared__ int64_t s_k[2];
-    __shared__ int s_low;
-    if (threadIdx.x == 0) s_n = 0;
-    __syncthreads();
-    const int64_t ns = M < (int64_t)a.S ? M : (int64_t)a.S;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ns = (int)(M < (int64_t)a.S ? M : (int64_t)a.S);
     const float lo_clamp = fmaxf(a.near_plane, a.eps);
     // every sample's key: read (the sampling kernel gathered them), or its
     // gid then its depth (and scale) gathered at once, so the dependent loads
@@ -158,102 +166,101 @@ __device__ __forceinline__ void depth_range_block(const float4* __restrict__ c_o
     if constexpr (GidOf::kKeys) {
 #pragma unroll
         for (int r = 0; r < kPer; ++r) {
-            const int64_t i = (int64_t)r * kDrThreads + threadIdx.x;
+            const int i = r * kDrThreads + (int)threadIdx.x;
             zk[r] = i < ns ? __uint_as_float(gid_of(i, 0)) : 0.0f;
         }
     } else {
+        // floor(x / ns) by a multiply (the product's high word is it or one
+        // less): a 64-bit division a sample was a quarter of the kernel
+        const uint64_t inv = ns > 0 ? ~0ull / (uint64_t)ns : 0ull;
         uint32_t gk[kPer];
 #pragma unroll
         for (int r = 0; r < kPer; ++r) {
-            const int64_t i = (int64_t)r * kDrThreads + threadIdx.x;
-            gk[r] = i < ns ? gid_of(i, (i * M) / ns) : 0u;
+            const int i = r * kDrThreads + (int)threadIdx.x;
+            const uint64_t x = (uint64_t)i * (uint64_t)M;
+            uint64_t j = __umul64hi(x, inv);
+            if ((j + 1) * (uint64_t)ns <= x) ++j;
+            gk[r] = i < ns ? gid_of(i, (int64_t)j) : 0u;
         }
 #pragma unroll
         for (int r = 0; r < kPer; ++r) {
-            const int64_t i = (int64_t)r * kDrThreads + threadIdx.x;
+            const int i = r * kDrThreads + (int)threadIdx.x;
             zk[r] = i < ns ? sample_key(c_o_z, scales, gk[r], a) : 0.0f;
         }
     }
-    // the positive keys, clamped, compacted with one shared atomic per warp
-    // and round; their minimum and maximum on the way
-    uint32_t lo_v = 0xffffffffu, hi_v = 0u;
+    // the positive keys, clamped (dropped: all bits set); their count, minimum
+    // and maximum
+    uint32_t v[kPer], lo_v = 0xffffffffu, hi_v = 0u, cnt = 0u;
 #pragma unroll
     for (int r = 0; r < kPer; ++r) {
-        const int64_t i = (int64_t)r * kDrThreads + threadIdx.x;
-        const float z = zk[r];
-        const bool keep = i < ns && z > 0.0f;
-        const unsigned bal = __ballot_sync(0xffffffffu, keep);
-        const int lane = threadIdx.x & 31;
-        int base = 0;
-        if (lane == 0 && bal) base = atomicAdd(&s_n, __popc(bal));
-        base = __shfl_sync(0xffffffffu, base, 0);
+        const bool keep = zk[r] > 0.0f;
+        v[r] = keep ? __float_as_uint(fminf(fmaxf(zk[r], lo_clamp), a.far_plane)) : 0xffffffffu;
         if (keep) {
-            const uint32_t v = __float_as_uint(fminf(fmaxf(z, lo_clamp), a.far_plane));
-            s_v[base + __popc(bal & ((1u << lane) - 1u))] = v;
-            lo_v = min(lo_v, v);
-            hi_v = max(hi_v, v);
+            lo_v = min(lo_v, v[r]);
+            hi_v = max(hi_v, v[r]);
+            ++cnt;
         }
     }
+    lo_v = __reduce_min_sync(0xffffffffu, lo_v);
+    hi_v = __reduce_max_sync(0xffffffffu, hi_v);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) {
+        s_red[0][warp] = lo_v;
+        s_red[1][warp] = hi_v;
+        s_red[2][warp] = cnt;
+    }
+    reinterpret_cast<uint2*>(s_h[0])[threadIdx.x] = make_uint2(0u, 0u);
     __syncthreads();
-    const int n = s_n;
+    lo_v = __reduce_min_sync(0xffffffffu, s_red[0][lane]);
+    hi_v = __reduce_max_sync(0xffffffffu, s_red[1][lane]);
+    const int n = (int)__reduce_add_sync(0xffffffffu, s_red[2][lane]);
     float zmin, zmax;
     if (n == 0) {
         zmin = lo_clamp;
         zmax = a.far_plane;
     } else {
-        // the bits every sample shares (those of the block's min and max)
-        // need no pass: start below the highest bit where samples differ
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        lo_v = __reduce_min_sync(0xffffffffu, lo_v);
-        hi_v = __reduce_max_sync(0xffffffffu, hi_v);
-        if (lane == 0) {
-            s_h[0][warp] = lo_v;
-            s_h[1][warp] = hi_v;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            const int nw = blockDim.x >> 5;
-            lo_v = __reduce_min_sync(0xffffffffu, lane < nw ? s_h[0][lane] : 0xffffffffu);
-            hi_v = __reduce_max_sync(0xffffffffu, lane < nw ? s_h[1][lane] : 0u);
-            if (lane == 0) {
-                const int cp = lo_v == hi_v ? 32 : __clz(lo_v ^ hi_v);
-                const uint32_t top = cp == 32 ? 0xffffffffu : (cp == 0 ? 0u : ~(0xffffffffu >> cp));
-                s_pref[0] = s_pref[1] = lo_v & top;
-                s_k[0] = rank_of(a.p_lo, n);
-                s_k[1] = rank_of(a.p_hi, n);
-                s_low = 32 - cp;  // bits still to select
+        int k = 0;  // warps 0 and 1: the rank left to find, lower and upper
+        if (warp < 2) k = rank_of(warp == 0 ? a.lo : a.hi, n);
+        uint32_t p0 = 0u, p1 = 0u;  // the bits found, of key - lo_v
+        for (int left = 32 - __clz(hi_v - lo_v); left > 0;) {
+            const int w = left < kDrBits ? left : kDrBits;
+            const int shift = left - w;
+            const bool both = p0 == p1;  // one count serves both ranks
+#pragma unroll
+            for (int r = 0; r < kPer; ++r) {
+                const uint32_t u = v[r] - lo_v;
+                const uint32_t top = u >> left;  // left <= 31: both are positive floats' bits
+                const uint32_t dg = (u >> shift) & ((1u << w) - 1u);
+                if (v[r] == 0xffffffffu) continue;
+                if (top == p0) atomicAdd(&s_h[0][dg], 1u);
+                if (!both && top == p1) atomicAdd(&s_h[1][dg], 1u);
             }
-        }
-        __syncthreads();
-        const int low = s_low;
-        uint32_t mask = low >= 32 ? 0u : ~((1u << low) - 1u);
-        // radix select (positive floats: bit order = value order), <= 8 bits a pass
-        for (int hi_bit = low; hi_bit > 0; hi_bit -= 8) {
-            const int shift = hi_bit > 8 ? hi_bit - 8 : 0;
-            const uint32_t dmask = (1u << (hi_bit - shift)) - 1u;
-            for (int d = threadIdx.x; d < 512; d += blockDim.x) s_h[d >> 8][d & 255] = 0u;
             __syncthreads();
-            const uint32_t p0 = s_pref[0], p1 = s_pref[1];
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                const uint32_t v = s_v[i];
-                const uint32_t dg = (v >> shift) & dmask;
-                if ((v & mask) == p0) atomicAdd(&s_h[0][dg], 1u);
-                if ((v & mask) == p1) atomicAdd(&s_h[1][dg], 1u);
+            const uint2 c0 = *reinterpret_cast<const uint2*>(&s_h[0][64 * warp + 2 * lane]);
+            const uint2 c1 = *reinterpret_cast<const uint2*>(&s_h[1][64 * warp + 2 * lane]);
+            const uint32_t g0 = __reduce_add_sync(0xffffffffu, c0.x + c0.y);
+            const uint32_t g1 = __reduce_add_sync(0xffffffffu, c1.x + c1.y);
+            if (lane == 0) {
+                s_red[0][warp] = g0;
+                s_red[1][warp] = both ? g0 : g1;
             }
             __syncthreads();
             if (warp < 2) {
-                uint32_t dsel = 0u;
-                int64_t krem = 0;
-                if (warp_digit_select(s_h[warp], s_k[warp], &dsel, &krem)) {
-                    s_k[warp] = krem;
-                    s_pref[warp] |= dsel << shift;
-                }
+                const uint32_t bin = warp_bin_select(s_h[both ? 0 : warp], s_red[warp][lane], k);
+                if (lane == 0) s_pref[warp] = ((warp == 0 ? p0 : p1) << w) | bin;
             }
-            mask |= dmask << shift;
             __syncthreads();
+            p0 = s_pref[0];
+            p1 = s_pref[1];
+            left = shift;
+            if (left > 0) {
+                reinterpret_cast<uint2*>(s_h[0])[threadIdx.x] = make_uint2(0u, 0u);
+                reinterpret_cast<uint2*>(s_h[1])[threadIdx.x] = make_uint2(0u, 0u);
+                __syncthreads();
+            }
         }
-        const float zlo = __uint_as_float(s_pref[0]);
-        const float zhi = __uint_as_float(s_pref[1]);
+        const float zlo = __uint_as_float(p0 + lo_v);
+        const float zhi = __uint_as_float(p1 + lo_v);
         const float span = fmaxf(zhi - zlo, 1e-6f);
         zmin = fmaxf(a.near_plane, zlo - a.pad * span);
         zmax = fminf(a.far_plane, zhi + a.pad * span);
