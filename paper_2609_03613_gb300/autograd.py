@@ -36,9 +36,13 @@ class Frame:
 class RasterizeFunction(torch.autograd.Function):
     @staticmethod
     def forward(fctx, xy_ab, c_o_z, rgb, frame: Frame):
-        fields = G.projected_fields(frame.projected, frame.n)
-        for name, t in (("xy_ab", xy_ab), ("c_o_z", c_o_z), ("rgb", rgb)):
-            if t.data_ptr() != fields[name].data_ptr() or t.shape != fields[name].shape:
+        # the fields' addresses in the buffer (projected_fields, without the views)
+        buf, off = frame.projected, G.projected_offsets(frame.n)
+        if buf.dtype != torch.uint8 or buf.dim() != 1 or not buf.is_contiguous() or buf.shape[0] < off[-1]:
+            raise G.TileGSError(f"rasterize: the projected buffer must hold {off[-1]} contiguous bytes")
+        base, shape = buf.data_ptr(), (frame.n, 4)
+        for name, t, o in (("xy_ab", xy_ab, off[0]), ("c_o_z", c_o_z, off[1]), ("rgb", rgb, off[2])):
+            if t.data_ptr() != base + o or t.shape != shape:
                 raise G.TileGSError(f"rasterize: {name} must be the projected buffer's own field view")
         img, alpha, _, saved = frame.ctx.rasterize_fwd(frame.projected, frame.n, frame.cam, frame.words,
                                                       frame.offsets, frame.stride, frame.bg, save=True)

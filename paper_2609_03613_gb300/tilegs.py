@@ -58,6 +58,10 @@ class GsCamera(C.Structure):
                 ("near_plane", C.c_float), ("far_plane", C.c_float)]
 
 
+_Mat = C.c_float * 16
+_Bg = C.c_float * 3
+
+
 class GsConfig(C.Structure):
     _fields_ = [("mode", C.c_int32), ("tile_size", C.c_int32), ("K", C.c_int32),
                 ("sample_count", C.c_int32), ("p_lo", C.c_float), ("p_hi", C.c_float),
@@ -180,23 +184,23 @@ def default_config(mode="exact", **kw) -> GsConfig:
 
 def gs_camera(cam) -> GsCamera:
     """Marshal a scenes.Camera (or anything with the same fields)."""
-    c = GsCamera()
-    vm = np.ascontiguousarray(cam.viewmat, np.float32).reshape(-1)
-    for k in range(16):
-        c.viewmat[k] = float(vm[k])
-    c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
-    c.width, c.height = int(cam.width), int(cam.height)
-    c.near_plane, c.far_plane = float(cam.near), float(cam.far)
+    c = GsCamera(_Mat(), float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy), int(cam.width),
+                 int(cam.height), float(cam.near), float(cam.far))
+    c.viewmat[:] = np.ascontiguousarray(cam.viewmat, np.float32).reshape(-1)[:16].tolist()
     return c
 
 
 def _ptr(t) -> int | None:
-    return None if t is None else int(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream():
+    # the handle alone: the Stream object costs six times as much, in each
+    # call of the library
     import torch
-    return torch.cuda.current_stream().cuda_stream
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 @dataclasses.dataclass
@@ -306,7 +310,7 @@ class Context:
         dev = projected.device
         c = gs_camera(cam)
         if m_dev is None:
-            m_dev = torch.zeros(1, dtype=torch.int64, device=dev)
+            m_dev = torch.empty(1, dtype=torch.int64, device=dev)
         if m_cap is None:
             m_cap = max(1024, 4 * n)
         while True:
@@ -337,7 +341,8 @@ class Context:
         T = n_tiles(cam.width, cam.height, int(self.cfg.tile_size))
         words = torch.empty(max(m_cap, 1), dtype=torch.int64, device=dev)
         offsets = torch.empty(T * self.stride + 1, dtype=torch.int32, device=dev)
-        zr = torch.zeros(2, dtype=torch.float32, device=dev)
+        # the binned modes write it
+        zr = (torch.zeros if self.mode == MODE_GLOBAL_SORT else torch.empty)(2, dtype=torch.float32, device=dev)
         c = gs_camera(cam)
         check(lib().gs_sort_or_bin(self.h, _ptr(projected), _ptr(scales), n, C.byref(c), _ptr(isect),
                                    m_cap, _ptr(m_dev), _ptr(words), _ptr(offsets), _ptr(zr), _stream()),
@@ -388,7 +393,7 @@ class Context:
         fT = torch.empty((H, W), dtype=torch.float32, device=dev) if save else None
         te = (torch.empty(n_tiles(W, H, self.cfg.tile_size), dtype=torch.int32, device=dev)
               if save else None)
-        bgv = (C.c_float * 3)(*[float(x) for x in bg])
+        bgv = _Bg(*[float(x) for x in bg])
         c = gs_camera(cam)
         check(lib().gs_rasterize_fwd(self.h, _ptr(projected), n, C.byref(c), _ptr(words), _ptr(offsets),
                                      self.stride if stride is None else int(stride), bgv, _ptr(rgb),
@@ -410,7 +415,7 @@ class Context:
         for t, shape in ((dl_drgb, (cam.height, cam.width, 3)), (dl_dalpha, (cam.height, cam.width))):
             if t is not None and (t.dtype != torch.float32 or not t.is_contiguous() or tuple(t.shape) != shape):
                 raise TileGSError(f"gs_rasterize_bwd: expected a contiguous float32 tensor of shape {shape}")
-        bgv = (C.c_float * 3)(*saved.bg)
+        bgv = _Bg(*saved.bg)
         c = gs_camera(cam)
         check(lib().gs_rasterize_bwd(self.h, _ptr(projected), n, C.byref(c), _ptr(words), _ptr(offsets),
                                      self.stride if stride is None else int(stride), bgv, _ptr(saved.last),
@@ -432,7 +437,7 @@ class Context:
         rgb, alpha, last = out
         s = GsScene(_ptr(sc.means), _ptr(sc.scales), _ptr(sc.quats), _ptr(sc.opacities), _ptr(sc.sh),
                     sc.sh_degree, sc.n)
-        bgv = (C.c_float * 3)(*[float(x) for x in bg])
+        bgv = _Bg(*[float(x) for x in bg])
         c = gs_camera(cam)
         check(lib().gs_render(self.h, C.byref(s), C.byref(c), bgv, _ptr(rgb), _ptr(alpha), _ptr(last),
                               int(flags), _stream()), "gs_render")
@@ -472,7 +477,7 @@ class Context:
         last = torch.empty((H, W), dtype=torch.int32, device=dev)
         fl = torch.empty(T, dtype=torch.uint8, device=dev) if flags else None
         nd = torch.empty(T, dtype=torch.int32, device=dev) if needed else None
-        bgv = (C.c_float * 3)(*[float(x) for x in bg])
+        bgv = _Bg(*[float(x) for x in bg])
         c = gs_camera(cam)
         check(lib().gs_rasterize_fwd_plan(self.h, _ptr(projected), n, C.byref(c), _ptr(words), _ptr(offsets),
                                           self.stride if stride is None else int(stride), bgv, _ptr(rgb),
@@ -561,7 +566,7 @@ class Context:
         last = P(*[_ptr(o[2]) if len(o) > 2 else None for o in outs])
         s = GsScene(_ptr(sc.means), _ptr(sc.scales), _ptr(sc.quats), _ptr(sc.opacities), _ptr(sc.sh),
                     sc.sh_degree, sc.n)
-        bgv = (C.c_float * 3)(*[float(x) for x in bg])
+        bgv = _Bg(*[float(x) for x in bg])
         check(lib().gs_render_batch(self.h, C.byref(s), carr, nv, bgv, rgb, alpha, last, int(flags), _stream()),
               "gs_render_batch")
         return outs
@@ -608,17 +613,30 @@ class Context:
         return int(lib().gs_last_raster_ops(self.h, _stream()))
 
 
+def _align256(b):
+    return (b + 255) & ~255
+
+
+def projected_offsets(n):
+    """Byte offsets of the projected buffer's fields (gs_projected_offset), and
+    the end of the last."""
+    n = int(n)
+    a, r = _align256(16 * n), _align256(8 * n)
+    return 0, a, 2 * a, 3 * a, 3 * a + r, 3 * a + r + 4 * n
+
+
 def projected_fields(projected, n):
     """Views of the projected buffer's fields (float32 / int32 tensors)."""
     import torch
-    L = lib()
-    o = [int(L.gs_projected_offset(n, f)) for f in range(5)]
-    xy_ab = projected[o[0]:o[0] + 16 * n].view(torch.float32).view(n, 4)
-    c_o_z = projected[o[1]:o[1] + 16 * n].view(torch.float32).view(n, 4)
-    rgb = projected[o[2]:o[2] + 16 * n].view(torch.float32).view(n, 4)
-    rect = projected[o[3]:o[3] + 8 * n].view(torch.int32).view(n, 2)
-    radius = projected[o[4]:o[4] + 4 * n].view(torch.int32)
-    return dict(xy_ab=xy_ab, c_o_z=c_o_z, rgb=rgb, rect=rect, radius=radius)
+    n = int(n)
+    xy, co, rgb, rect, radius, end = projected_offsets(n)
+    f = projected[:end].view(torch.float32)
+    if f.shape[0] != end // 4:
+        raise TileGSError(f"projected_fields: {f.shape[0] * 4} bytes, expected {end}")
+    i, o = f.view(torch.int32), f.storage_offset()
+    return dict(xy_ab=f.as_strided((n, 4), (4, 1), o + xy // 4), c_o_z=f.as_strided((n, 4), (4, 1), o + co // 4),
+                rgb=f.as_strided((n, 4), (4, 1), o + rgb // 4), rect=i.as_strided((n, 2), (2, 1), o + rect // 4),
+                radius=i.as_strided((n,), (1,), o + radius // 4))
 
 
 def reciprocal(x):
@@ -672,10 +690,14 @@ def grad_fields(grad, n):
     the projected fields they differentiate: xy_ab {dmx, dmy, da, db},
     c_o_z {dc, dopacity, 0, 0}, rgb {dr, dg, db, 0}."""
     import torch
-    L = lib()
-    o = [int(L.gs_grad2d_offset(n, f)) for f in range(3)]
-    return {k: grad[o[f]:o[f] + 16 * n].view(torch.float32).view(n, 4)
-            for f, k in enumerate(("xy_ab", "c_o_z", "rgb"))}
+    n = int(n)
+    step = _align256(16 * n) // 4  # gs_grad2d_offset
+    end = 2 * step + 4 * n
+    f = grad[:4 * end].view(torch.float32)
+    if f.shape[0] != end:
+        raise TileGSError(f"grad_fields: {f.shape[0] * 4} bytes, expected {4 * end}")
+    o = f.storage_offset()
+    return {k: f.as_strided((n, 4), (4, 1), o + j * step) for j, k in enumerate(("xy_ab", "c_o_z", "rgb"))}
 
 
 def depth_range_noalloc(cfg: GsConfig, projected, scales, n, cam, isect, m_cap, m_dev, zrange):
