@@ -99,78 +99,36 @@ k_group_depth_range(const float4* __restrict__ c_o_z, const GroupViews gv, const
 // The row spans of k_row_spans (tiles.cu) for the group's items: each lane's
 // item and each record's owner look up their view (tile grid, bin splits,
 // difference counts); records carry the item G.
-__global__ void __launch_bounds__(256)
-k_group_row_spans(const uint2* __restrict__ rect, const int32_t* __restrict__ roff, CullArgs ca, const GroupViews gv,
-                  const BinParams* __restrict__ bp, const int64_t* __restrict__ m_dev, int64_t m_cap,
-                  int32_t* __restrict__ D, uint32_t* __restrict__ rs_g, uint32_t* __restrict__ rs_ya,
-                  uint32_t* __restrict__ rs_w, uint32_t* __restrict__ rs_z)
+__global__ void __launch_bounds__(256, kRowBlocks)
+k_group_row_spans(const uint2* __restrict__ rect, const int32_t* __restrict__ roff, CullArgs ca,
+                  const __grid_constant__ GroupViews gv, const BinParams* __restrict__ bp,
+                  const int64_t* __restrict__ m_dev, int64_t m_cap, int32_t* __restrict__ D, RowRecords rs)
 {
+    __shared__ RowOwners s_own[8];
     if (*m_dev > m_cap) return;
     const int64_t n = gv.n * gv.nv;
-    const int64_t g0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
+    const int64_t g0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * 32;
     if (g0 >= n) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t gl = g0 + lane;
-    const bool ok = gl < n;
-    const int32_t my_off = roff[ok ? gl : n];
-    const int32_t base = __shfl_sync(0xffffffffu, my_off, 0);
-    const int32_t end = roff[(g0 + 32) < n ? (g0 + 32) : n];
+    const int64_t gl = g0 + (threadIdx.x & 31);
+    const int32_t off = roff[gl < n ? gl : n], next = roff[gl + 1 < n ? gl + 1 : n];
     uint2 r = make_uint2(0u, 0u);
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f), q = p;
     float margin = 0.0f;
     uint32_t bin = 0u;
-    const int view = ok ? gv.view_of(gl) : 0;
-    if (ok) {
+    int view = 0;
+    if (next > off) {
         r = rect[gl];
-        if ((r.x & 0xffffu) < (r.y & 0xffffu) && (r.x >> 16) < (r.y >> 16)) {
-            p = __ldg(ca.xy_ab + gl);
-            q = __ldg(ca.c_o_z + gl);
-            margin = __ldg(&ca.rgb[gl].w);
-            bin = (uint32_t)bin_split(q.z, bp[view].splits, gv.K[view]);
-        }
+        p = __ldg(ca.xy_ab + gl);
+        q = __ldg(ca.c_o_z + gl);
+        margin = __ldg(&ca.rgb[gl].w);
+        view = gv.view_of(gl);
+        bin = (uint32_t)bin_split(q.z, bp[view].splits, gv.K[view]);
     }
-    const RowGeom mine = row_geom(0.5f * p.z, p.w, 0.5f * q.x, q.w, margin, p.y);
-    const float inv_tile = 1.0f / (float)ca.tile;
-    for (int32_t e0 = base; e0 < end; e0 += 32) {
-        const int32_t e = e0 + lane;
-        int k = 0;
-#pragma unroll
-        for (int s = 16; s > 0; s >>= 1) {
-            const int32_t v = __shfl_sync(0xffffffffu, my_off, (k + s) & 31);
-            if (k + s < 32 && v <= e) k += s;
-        }
-        const uint32_t ra = __shfl_sync(0xffffffffu, r.x, k), rb = __shfl_sync(0xffffffffu, r.y, k);
-        const float mx = __shfl_sync(0xffffffffu, p.x, k);
-        RowGeom g;
-        g.my = __shfl_sync(0xffffffffu, mine.my, k);
-        g.hb = __shfl_sync(0xffffffffu, mine.hb, k);
-        g.inv2ha = __shfl_sync(0xffffffffu, mine.inv2ha, k);
-        g.a4tp = __shfl_sync(0xffffffffu, mine.a4tp, k);
-        g.D = __shfl_sync(0xffffffffu, mine.D, k);
-        g.dymax = __shfl_sync(0xffffffffu, mine.dymax, k);
-        g.ext = __shfl_sync(0xffffffffu, mine.ext, k);
-        g.dyl = __shfl_sync(0xffffffffu, mine.dyl, k);
-        const uint32_t zb = __shfl_sync(0xffffffffu, __float_as_uint(q.z), k);
-        const uint32_t b = __shfl_sync(0xffffffffu, bin, k);
-        const int32_t o = __shfl_sync(0xffffffffu, my_off, k);
-        const int vk = __shfl_sync(0xffffffffu, view, k);
-        if (e < end) {
-            const int tx0 = ra & 0xffff, ty0 = ra >> 16, tx1 = rb & 0xffff;
-            const int ty = ty0 + (e - o);
-            int a, x1;
-            row_span(mx, g, ty, ca.tile, inv_tile, tx0, tx1, &a, &x1);
-            rs_g[e] = (uint32_t)(g0 + k);
-            rs_ya[e] = row_record(ty, a, b);
-            rs_w[e] = (uint32_t)(x1 - a);
-            rs_z[e] = zb;
-            if (x1 > a) {
-                const int W1 = gv.tiles_x[vk] + 1;
-                int32_t* L = D + gv.d_base[vk] + (int64_t)b * gv.tiles_y[vk] * W1;
-                atomicAdd(&L[ty * W1 + a], 1);
-                atomicAdd(&L[ty * W1 + x1], -1);
-            }
-        }
-    }
+    warp_row_spans(s_own[threadIdx.x >> 5], g0, off, next, __shfl_sync(0xffffffffu, off, 0),
+                   __shfl_sync(0xffffffffu, next, 31), r, p, q, margin, bin, view, ca.tile, rs,
+                   [&](uint32_t b, uint32_t v, int ty) {
+                       return D + gv.d_base[v] + ((int64_t)b * gv.tiles_y[v] + ty) * (gv.tiles_x[v] + 1);
+                   });
 }
 
 // One block per (view, bin layer): inclusive prefix along each tile row.
@@ -436,8 +394,7 @@ int group_binning(gs_ctx* gc, const GroupViews* gvp, int32_t flags, int64_t* h_m
     const int64_t warps = (N + 31) / 32;
     if (warps > 0)
         k_group_row_spans<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(pv.rect, roff, ca, gv, s.bp, gc->r_m,
-                                                                       gc->r_m_cap, s.D, s.rs_g, s.rs_ya, s.rs_w,
-                                                                       s.rs_z);
+                                                                       gc->r_m_cap, s.D, RowRecords{s.rs_g, s.rs_ya, s.rs_w, s.rs_z});
     int max_tx = 1, max_k = 1;
     size_t osm = 0;
     for (int v = 0; v < gv.nv; ++v) {

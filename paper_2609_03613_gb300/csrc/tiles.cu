@@ -92,86 +92,42 @@ struct LoadRectRows {
     }
 };
 
-// Warp-cooperative over (Gaussian, row) pairs: a warp owns 32 consecutive
-// Gaussians, whose rows are consecutive records [roff[g0], roff[g0 + 32)).
-// Each lane holds its Gaussian (record, bin); every row record is computed by
-// one lane from the owner's values (shuffled): the row's culled span, the
-// record (gid, row | start, width), and +1 / -1 at the span ends of layer b's
-// row (a per-row difference array).
-__global__ void __launch_bounds__(256)
+// Warp-cooperative over (Gaussian, row) pairs (warp_row_spans): a warp owns 32
+// consecutive Gaussians, whose rows are consecutive records [roff[g0], roff[g0
+// + 32)).  Per record the row's culled span, the record (gid, row | start,
+// width), and +1 / -1 at the span ends of layer b's row (a per-row difference
+// array).
+__global__ void __launch_bounds__(256, kRowBlocks)
 k_row_spans(const uint2* __restrict__ rect, int64_t n, const int32_t* __restrict__ roff, CullArgs ca, int tiles_x,
             const BinParams* __restrict__ bp, int K, const int64_t* __restrict__ m_dev, int64_t m_cap,
-            int32_t* __restrict__ Drow, int64_t layer, uint8_t* __restrict__ gbin, uint32_t* __restrict__ rs_g,
-            uint32_t* __restrict__ rs_ya, uint32_t* __restrict__ rs_w, uint32_t* __restrict__ rs_z)
+            int32_t* __restrict__ Drow, int64_t layer, uint8_t* __restrict__ gbin, RowRecords rs)
 {
     grid_dependency_sync();
     __shared__ float s_split[GS_MAX_K];
+    __shared__ RowOwners s_own[8];
     for (int k = threadIdx.x; k < K - 1; k += blockDim.x) s_split[k] = bp->splits[k];
     __syncthreads();
     if (*m_dev > m_cap) return;
-    const int64_t g0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
+    const int64_t g0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * 32;
     if (g0 >= n) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t gl = g0 + lane;
-    const bool ok = gl < n;
-    const int32_t my_off = roff[ok ? gl : n];
-    const int32_t base = __shfl_sync(0xffffffffu, my_off, 0);
-    const int32_t end = roff[(g0 + 32) < n ? (g0 + 32) : n];
+    const int64_t gl = g0 + (threadIdx.x & 31);
+    const int32_t off = roff[gl < n ? gl : n], next = roff[gl + 1 < n ? gl + 1 : n];
     uint2 r = make_uint2(0u, 0u);
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f), q = p;
     float margin = 0.0f;
     uint32_t bin = 0u;
-    if (ok) {
+    if (next > off) {
         r = rect[gl];
-        if ((r.x & 0xffffu) < (r.y & 0xffffu) && (r.x >> 16) < (r.y >> 16)) {
-            p = __ldg(ca.xy_ab + gl);
-            q = __ldg(ca.c_o_z + gl);
-            margin = __ldg(&ca.rgb[gl].w);
-            bin = (uint32_t)bin_split(q.z, s_split, K);
-            gbin[gl] = (uint8_t)bin;
-        }
+        p = __ldg(ca.xy_ab + gl);
+        q = __ldg(ca.c_o_z + gl);
+        margin = __ldg(&ca.rgb[gl].w);
+        bin = (uint32_t)bin_split(q.z, s_split, K);
+        gbin[gl] = (uint8_t)bin;
     }
-    const RowGeom mine = row_geom(0.5f * p.z, p.w, 0.5f * q.x, q.w, margin, p.y);
-    const float inv_tile = 1.0f / (float)ca.tile;  // exact: tiles are 8, 16 or 32
     const int W1 = tiles_x + 1;
-    for (int32_t e0 = base; e0 < end; e0 += 32) {
-        const int32_t e = e0 + lane;
-        int k = 0;
-#pragma unroll
-        for (int s = 16; s > 0; s >>= 1) {
-            const int32_t v = __shfl_sync(0xffffffffu, my_off, (k + s) & 31);
-            if (k + s < 32 && v <= e) k += s;
-        }
-        const uint32_t ra = __shfl_sync(0xffffffffu, r.x, k), rb = __shfl_sync(0xffffffffu, r.y, k);
-        const float mx = __shfl_sync(0xffffffffu, p.x, k);
-        RowGeom g;
-        g.my = __shfl_sync(0xffffffffu, mine.my, k);
-        g.hb = __shfl_sync(0xffffffffu, mine.hb, k);
-        g.inv2ha = __shfl_sync(0xffffffffu, mine.inv2ha, k);
-        g.a4tp = __shfl_sync(0xffffffffu, mine.a4tp, k);
-        g.D = __shfl_sync(0xffffffffu, mine.D, k);
-        g.dymax = __shfl_sync(0xffffffffu, mine.dymax, k);
-        g.ext = __shfl_sync(0xffffffffu, mine.ext, k);
-        g.dyl = __shfl_sync(0xffffffffu, mine.dyl, k);
-        const uint32_t zb = __shfl_sync(0xffffffffu, __float_as_uint(q.z), k);
-        const uint32_t b = __shfl_sync(0xffffffffu, bin, k);
-        const int32_t o = __shfl_sync(0xffffffffu, my_off, k);
-        if (e < end) {
-            const int tx0 = ra & 0xffff, ty0 = ra >> 16, tx1 = rb & 0xffff;
-            const int ty = ty0 + (e - o);
-            int a, x1;
-            row_span(mx, g, ty, ca.tile, inv_tile, tx0, tx1, &a, &x1);
-            rs_g[e] = (uint32_t)(g0 + k);
-            rs_ya[e] = row_record(ty, a, b);
-            rs_w[e] = (uint32_t)(x1 - a);
-            rs_z[e] = zb;
-            if (x1 > a) {
-                int32_t* L = Drow + b * layer;
-                atomicAdd(&L[ty * W1 + a], 1);
-                atomicAdd(&L[ty * W1 + x1], -1);
-            }
-        }
-    }
+    warp_row_spans(s_own[threadIdx.x >> 5], g0, off, next, __shfl_sync(0xffffffffu, off, 0),
+                   __shfl_sync(0xffffffffu, next, 31), r, p, q, margin, bin, 0, ca.tile, rs,
+                   [&](uint32_t b, uint32_t, int ty) { return Drow + b * layer + ty * W1; });
 }
 
 // One block per layer: inclusive prefix along each row.
@@ -820,8 +776,8 @@ int exact_bins(gs_ctx* ctx, const ProjView& pv, int64_t n, const gs_camera* cam,
         const int64_t warps = (n + 31) / 32;
         if (warps > 0)
             GS_CUDA_TRY(launch_k(ctx, k_row_spans, (unsigned)((warps + 7) / 8), 256, 0, st, pv.rect, n, v.roff, ca, tiles_x, ctx->d_bp, K,
-                                                                     m_dev, m_cap, v.D, rlayer, v.gbin, v.rs_g,
-                                                                     v.rs_ya, v.rs_w, v.rs_z));
+                                                                     m_dev, m_cap, v.D, rlayer, v.gbin,
+                                                                     RowRecords{v.rs_g, v.rs_ya, v.rs_w, v.rs_z}));
         ctx->launches += 1;
         // the per-entry scatter starts its cursors at the offsets
         const bool want_cur = n > 0 && !grouped_path(m_cap, tiles_x, tiles_y, K);
