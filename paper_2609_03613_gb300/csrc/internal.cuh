@@ -556,11 +556,17 @@ struct ScatterPass {
         const int b = (int)(ya >> 24), x0 = (int)((ya >> 12) & 0xfffu);
         const int64_t t0 = (int64_t)(ya & 0xfffu) * tiles_x + x0;
         int lo = -1, hi = -1;
-        for (int j = 0; j < (int)w; ++j)
-            if (keep(t0 + j, b)) {
-                if (lo < 0) lo = j;
-                hi = j;
-            }
+        for (int j0 = 0; j0 < (int)w; j0 += 4) {  // four tiles' plans in flight
+            bool k[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) k[u] = j0 + u < (int)w && keep(t0 + j0 + u, b);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k[u]) {
+                    if (lo < 0) lo = j0 + u;
+                    hi = j0 + u;
+                }
+        }
         if (lo < 0) {
             w = 0u;
             return;

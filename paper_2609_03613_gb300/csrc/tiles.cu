@@ -170,20 +170,26 @@ __device__ __forceinline__ void plan_rows(const ScatterPass& sp, int tiles_x, in
                                           const int32_t* __restrict__ flagged, int32_t* s_row, uint32_t* mask)
 {
     const int words = (tiles_x + 31) / 32;
-    for (int y = threadIdx.x; y < tiles_y; y += blockDim.x) s_row[y] = sp.pass == 1 ? 0 : kNoRow;
+    if (sp.pass == 1) {  // a warp a row (32 atomics on one row's word before)
+        const int lane = threadIdx.x & 31;
+        for (int y = threadIdx.x >> 5; y < tiles_y; y += blockDim.x >> 5) {
+            int m = 0;
+#pragma unroll 8
+            for (int x = lane; x < tiles_x; x += 32) m = max(m, (int)__ldg(sp.plan + (int64_t)y * tiles_x + x));
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) s_row[y] = m;
+        }
+        __syncthreads();
+        return;
+    }
+    for (int y = threadIdx.x; y < tiles_y; y += blockDim.x) s_row[y] = kNoRow;
     if (mask)
         for (int q = threadIdx.x; q < tiles_y * words; q += blockDim.x) mask[q] = 0u;
     __syncthreads();
-    if (sp.pass == 1) {
-#pragma unroll 8
-        for (int t = threadIdx.x; t < tiles_x * tiles_y; t += blockDim.x)
-            atomicMax(&s_row[t / tiles_x], (int)__ldg(sp.plan + t));
-    } else {
-        for (int i = threadIdx.x; i < flagged[0]; i += blockDim.x) {
-            const int t = flagged[1 + i], y = t / tiles_x, x = t - y * tiles_x;
-            atomicMin(&s_row[y], (int)__ldg(sp.plan + t));
-            if (mask) atomicOr(&mask[y * words + (x >> 5)], 1u << (x & 31));
-        }
+    for (int i = threadIdx.x; i < flagged[0]; i += blockDim.x) {
+        const int t = flagged[1 + i], y = t / tiles_x, x = t - y * tiles_x;
+        atomicMin(&s_row[y], (int)__ldg(sp.plan + t));
+        if (mask) atomicOr(&mask[y * words + (x >> 5)], 1u << (x & 31));
     }
     __syncthreads();
 }
@@ -310,6 +316,8 @@ __global__ void k_flagged_cursors(const int32_t* __restrict__ list, const int32_
 // then one block per group holds the cursors of that row's tiles for that bin
 // (tiles_x words) and takes every slot with a shared-memory atomic.
 constexpr int kGroupThreads = 1024;
+template <bool PLANNED>
+constexpr int kGroupIF = PLANNED ? 2 : 8;  // records a thread has in flight
 constexpr int kMaxGroupKeys = 12288;  // (tile row, bin) keys in 48 KB of shared memory
 // reserved entries per tile from which the grouped scatter is used: measured
 // slower at ~3k (1M Gaussians, 1080p: bin stage 0.228 vs 0.210 ms), faster at
@@ -328,17 +336,33 @@ __device__ __forceinline__ void record_slice(int64_t R, int C, int c, int64_t* r
 // key of a row record: (tile row, bin)
 __device__ __forceinline__ int group_key(uint32_t ya, int K) { return (int)(ya & 0xfffu) * K + (int)(ya >> 24); }
 
-// The record word and width at k, the width 0 when the pass drops it.
+// The record words and widths of records k0 + u kGroupThreads, the width 0 when
+// the pass drops one or it lies past r1.  Several in flight: both passes wait
+// on their loads (one a thread and round: count 31 us and
+// write 124, eight 26 and 104; planned passes, whose records mostly drop on the
+// row word, 66 and 66, two 52 and 54).
 template <bool PLANNED>
-__device__ __forceinline__ uint32_t group_record(const uint32_t* __restrict__ rs_ya, const uint32_t* __restrict__ rs_w,
-                                                 int64_t k, const ScatterPass& sp, const int32_t* s_row, int tiles_x,
-                                                 uint32_t& ya)
+__device__ __forceinline__ void group_records(const uint32_t* __restrict__ rs_ya, const uint32_t* __restrict__ rs_w,
+                                              int64_t k0, int64_t r1, const ScatterPass& sp, const int32_t* s_row,
+                                              int tiles_x, uint32_t (&ya)[kGroupIF<PLANNED>], uint32_t (&w)[kGroupIF<PLANNED>])
 {
-    ya = rs_ya[k];
-    if (PLANNED && !plan_row_live(sp, s_row, ya)) return 0u;
-    uint32_t w = rs_w[k];
-    if (PLANNED) sp.trim(ya, w, tiles_x);
-    return w;
+#pragma unroll
+    for (int u = 0; u < kGroupIF<PLANNED>; ++u) {
+        const int64_t k = k0 + u * kGroupThreads;
+        ya[u] = k < r1 ? rs_ya[k] : 0u;
+        w[u] = !PLANNED && k < r1 ? rs_w[k] : 0u;
+    }
+    if constexpr (PLANNED) {
+        // most records are dropped on their row word
+#pragma unroll
+        for (int u = 0; u < kGroupIF<PLANNED>; ++u) {
+            const int64_t k = k0 + u * kGroupThreads;
+            if (k < r1 && plan_row_live(sp, s_row, ya[u])) w[u] = rs_w[k];
+        }
+#pragma unroll
+        for (int u = 0; u < kGroupIF<PLANNED>; ++u)
+            if (w[u] != 0u) sp.trim(ya[u], w[u], tiles_x);
+    }
 }
 
 // pass 1: H[key * C + c] = non-empty records of slice c with that key
@@ -358,9 +382,12 @@ k_group_count(const uint32_t* __restrict__ rs_ya, const uint32_t* __restrict__ r
     if (*m_dev <= m_cap) {
         int64_t r0, r1;
         record_slice(roff[n], C, c, &r0, &r1);
-        for (int64_t k = r0 + threadIdx.x; k < r1; k += blockDim.x) {
-            uint32_t ya;
-            if (group_record<PLANNED>(rs_ya, rs_w, k, sp, s_row, tiles_x, ya) != 0u) atomicAdd(&s_h[group_key(ya, K)], 1);
+        for (int64_t k0 = r0 + threadIdx.x; k0 < r1; k0 += kGroupIF<PLANNED> * kGroupThreads) {
+            uint32_t ya[kGroupIF<PLANNED>], w[kGroupIF<PLANNED>];
+            group_records<PLANNED>(rs_ya, rs_w, k0, r1, sp, s_row, tiles_x, ya, w);
+#pragma unroll
+            for (int u = 0; u < kGroupIF<PLANNED>; ++u)
+                if (w[u] != 0u) atomicAdd(&s_h[group_key(ya[u], K)], 1);
         }
     }
     __syncthreads();
@@ -387,20 +414,30 @@ k_group_write(const uint32_t* __restrict__ rs_g, const uint32_t* __restrict__ rs
     __syncthreads();
     int64_t r0, r1;
     record_slice(roff[n], C, c, &r0, &r1);
-    for (int64_t k = r0 + threadIdx.x; k < r1; k += blockDim.x) {
-        uint32_t ya;
-        const uint32_t w = group_record<PLANNED>(rs_ya, rs_w, k, sp, s_row, tiles_x, ya);
-        if (w == 0u) continue;
-        list[atomicAdd(&s_h[group_key(ya, K)], 1)] = make_uint4(rs_g[k], ya, w, rs_z[k]);
+    for (int64_t k0 = r0 + threadIdx.x; k0 < r1; k0 += kGroupIF<PLANNED> * kGroupThreads) {
+        uint32_t ya[kGroupIF<PLANNED>], w[kGroupIF<PLANNED>], g[kGroupIF<PLANNED>], z[kGroupIF<PLANNED>];
+        group_records<PLANNED>(rs_ya, rs_w, k0, r1, sp, s_row, tiles_x, ya, w);
+#pragma unroll
+        for (int u = 0; u < kGroupIF<PLANNED>; ++u) {
+            if (w[u] == 0u) continue;
+            g[u] = __ldcs(rs_g + k0 + u * kGroupThreads);
+            z[u] = __ldcs(rs_z + k0 + u * kGroupThreads);
+        }
+#pragma unroll
+        for (int u = 0; u < kGroupIF<PLANNED>; ++u)
+            if (w[u] != 0u) list[atomicAdd(&s_h[group_key(ya[u], K)], 1)] = make_uint4(g[u], ya[u], w[u], z[u]);
     }
 }
 
 // one block per (tile row, bin): that bin's cursor of every tile of the row
-// (1024 threads: the groups' sizes vary widely, and the largest bound the
-// kernel's tail); a thread takes a record and walks its span of tiles
-constexpr int kScatterGroupThreads = 1024;
+// (NT = 1024 threads: the groups' sizes vary widely, and the largest bound the
+// kernel's tail: 217 us, with 512 threads 277, for 3M Gaussians seen from
+// inside a cluster; 512 in a planned first pass, most of whose groups are
+// empty: 45 us against 97 at 2560 x 1440); a thread takes a record and walks
+// its span of tiles (two records at a time in flight: 302 us)
 
-__global__ void __launch_bounds__(kScatterGroupThreads)
+template <int NT>
+__global__ void __launch_bounds__(NT)
 k_scatter_groups(const uint4* __restrict__ list, const int32_t* __restrict__ Hs, int C,
                  const int32_t* __restrict__ offsets, int tiles_x, int K, const int64_t* __restrict__ m_dev,
                  int64_t m_cap, uint64_t* __restrict__ words, const ScatterPass sp,
@@ -414,6 +451,9 @@ k_scatter_groups(const uint4* __restrict__ list, const int32_t* __restrict__ Hs,
     const int ty = key / K, b = key - ty * K;
     const int32_t L0 = Hs[(int64_t)key * C], L1 = Hs[(int64_t)(key + 1) * C];
     if (L1 <= L0) return;
+    // the first records are on their way while the cursors are
+    int32_t i = L0 + (int32_t)threadIdx.x;
+    uint4 next = i < L1 ? __ldcs(list + i) : make_uint4(0u, 0u, 0u, 0u);
     int any = 0;
     for (int x = threadIdx.x; x < tiles_x; x += blockDim.x) {
         const int64_t t = (int64_t)ty * tiles_x + x;
@@ -422,8 +462,10 @@ k_scatter_groups(const uint4* __restrict__ list, const int32_t* __restrict__ Hs,
     }
     // a planned pass skips the groups no tile of the row takes in this pass
     if (!__syncthreads_or(any)) return;
-    for (int32_t i = L0 + (int32_t)threadIdx.x; i < L1; i += (int32_t)blockDim.x) {
-        const uint4 rec = list[i];
+    while (i < L1) {
+        const uint4 rec = next;
+        i += NT;
+        if (i < L1) next = __ldcs(list + i);
         const uint64_t word = ((uint64_t)rec.w << 32) | rec.x;
         const int a = (int)((rec.y >> 12) & 0xfffu);
         for (int j = 0; j < (int)rec.z; ++j) {
@@ -633,7 +675,7 @@ static int exact_scatter(gs_ctx* ctx, const ExactScratch& v, int64_t n, int32_t 
         if ((r = scan_impl(ctx, LoadI32{v.H}, (int64_t)nkeys * C, v.Hs, nullptr, st)) != GS_OK) return r;
         GS_CUDA_TRY(launch_k(ctx, sp.pass ? k_group_write<true> : k_group_write<false>, (unsigned)C, kGroupThreads, hsm, st, v.rs_g, v.rs_ya, v.rs_w, v.rs_z, v.roff, n, K, nkeys,
                                                                 m_dev, m_cap, v.Hs, v.list, sp, tiles_x));
-        GS_CUDA_TRY(launch_k(ctx, k_scatter_groups, (unsigned)nkeys, kScatterGroupThreads, (size_t)tiles_x * 4, st, 
+        GS_CUDA_TRY(launch_k(ctx, sp.pass ? k_scatter_groups<512> : k_scatter_groups<1024>, (unsigned)nkeys, sp.pass ? 512 : 1024, (size_t)tiles_x * 4, st, 
             v.list, v.Hs, C, offsets, tiles_x, K, m_dev, m_cap, words, sp, flagged));
         ctx->launches += 2;
     } else {
