@@ -26,42 +26,11 @@
 
 namespace gs {
 
-// A lane's P pixels.  Two: (x, y) and (x + 4, y) of the warp's 8 x 8 block;
-// they share dy and the entry's shared-memory reads, and what is done to both
-// runs on packed float32 pairs (each half rounded as the scalar operation).
-// One: a pixel of the warp's 8 x 4 block, scalar.
+// The lane's pixel h in its warp's block: (x, y) and (x + 4, y), or (x, y).
 template <int P>
-struct Lane;
-template <>
-struct Lane<2> {
-    using V = uint64_t;  // pixel 0 in the low half
-    static __device__ __forceinline__ V same(float v) { return same2(v); }
-    static __device__ __forceinline__ V put(const float (&v)[2]) { return pk2(v[0], v[1]); }
-    static __device__ __forceinline__ void get(V v, float (&o)[2]) { upk2(v, o[0], o[1]); }
-    static __device__ __forceinline__ V fma(V a, V b, V c) { return fma2(a, b, c); }
-    static __device__ __forceinline__ V mul(V a, V b) { return mul2(a, b); }
-    static __device__ __forceinline__ void exp_neg(const float (&q)[2], float (&e)[2])
-    {
-        spec_exp_neg2(q[0], q[1], e[0], e[1]);
-    }
-    static __device__ __forceinline__ float least(const float (&v)[2]) { return fminf(v[0], v[1]); }
-    // the lane's pixel h in its warp's block
-    static __device__ __forceinline__ int x(int lane, int h) { return (lane & 3) + 4 * h; }
-    static __device__ __forceinline__ int y(int lane) { return lane >> 2; }
-};
-template <>
-struct Lane<1> {
-    using V = float;
-    static __device__ __forceinline__ V same(float v) { return v; }
-    static __device__ __forceinline__ V put(const float (&v)[1]) { return v[0]; }
-    static __device__ __forceinline__ void get(V v, float (&o)[1]) { o[0] = v; }
-    static __device__ __forceinline__ V fma(V a, V b, V c) { return fmaf(a, b, c); }
-    static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
-    static __device__ __forceinline__ void exp_neg(const float (&q)[1], float (&e)[1]) { e[0] = spec_exp_core(-q[0]); }
-    static __device__ __forceinline__ float least(const float (&v)[1]) { return v[0]; }
-    static __device__ __forceinline__ int x(int lane, int) { return lane & 7; }
-    static __device__ __forceinline__ int y(int lane) { return lane >> 3; }
-};
+__device__ __forceinline__ int lane_x(int lane, int h) { return P == 2 ? (lane & 3) + 4 * h : lane & 7; }
+template <int P>
+__device__ __forceinline__ int lane_y(int lane) { return P == 2 ? lane >> 2 : lane >> 3; }
 
 // Per-thread compositing state.  A pixel that has stopped (or lies outside the
 // image) has a NaN centre, so that no entry passes it again.
@@ -75,18 +44,6 @@ struct PixelState {
     int live;       // bit h: pixel h is still compositing
     unsigned long long ops;
 };
-
-// q of one staged entry at the lane's pixels.
-template <int P>
-__device__ __forceinline__ void entry_dist(const float4& ga, const float4& gb, const PixelState<P>& st, float (&q)[P])
-{
-    if constexpr (P == 2) {
-        entry_q(ga, gb, st.x[0], st.x[1], st.y, q[0], q[1]);
-    } else {
-        const float dx = ga.x - st.x[0], dy = ga.y - st.y;
-        q[0] = fmaf(dx, fmaf(ga.z, dx, ga.w * dy), (gb.x * dy) * dy);
-    }
-}
 
 // alpha of one entry where the pixel takes it (pass), else 0.  0 <= q <= tau
 // as one unsigned compare of the float bits (negative q and NaN compare above
@@ -206,7 +163,7 @@ __device__ __forceinline__ void composite_batch(int cnt, RasterShared<TILE, P>& 
 #pragma unroll
         for (int j = 0; j < R; ++j) {
             gb[j] = *reinterpret_cast<const float4*>(pb + k[j]);
-            entry_dist<P>(*reinterpret_cast<const float4*>(pa + k[j]), gb[j], st, q[j]);
+            entry_dist(*reinterpret_cast<const float4*>(pa + k[j]), gb[j], st.x, st.y, q[j]);
         }
         if constexpr (SKIP) {
             bool any = false;
@@ -366,10 +323,10 @@ __device__ __forceinline__ void raster_tile(
     const int tx = t % a.tiles_x, ty = t / a.tiles_x;
     const int lane = threadIdx.x & 31;
     const int px0 = tx * TILE + TB::x0(), py0 = ty * TILE + TB::y0();  // the warp's block
-    const int py = py0 + L::y(lane);
+    const int py = py0 + lane_y<P>(lane);
     int inside = 0;
 #pragma unroll
-    for (int h = 0; h < P; ++h) inside |= (py < a.height && px0 + L::x(lane, h) < a.width ? 1 : 0) << h;
+    for (int h = 0; h < P; ++h) inside |= (py < a.height && px0 + lane_x<P>(lane, h) < a.width ? 1 : 0) << h;
 
     // float32 operations of the compositing definition each pixel executes
     // (COUNT builds): 8 per visit (offsets, q, sign test), 17 more when exp is
@@ -402,7 +359,7 @@ __device__ __forceinline__ void raster_tile(
             T[h] = 1.0f;
             C[0][h] = C[1][h] = C[2][h] = 0.0f;
             if ((inside >> h) & 1) {
-                const int64_t p = (int64_t)py * a.width + px0 + L::x(lane, h);
+                const int64_t p = (int64_t)py * a.width + px0 + lane_x<P>(lane, h);
                 // the first pass's state: C in rgb, T in alpha (negative once the
                 // pixel stopped), last
                 const float Ts = out_alpha[p];
@@ -421,7 +378,7 @@ __device__ __forceinline__ void raster_tile(
     }
 #pragma unroll
     for (int h = 0; h < P; ++h)
-        st.x[h] = (st.live >> h) & 1 ? (float)(px0 + L::x(lane, h)) + 0.5f : __uint_as_float(0x7fc00000u);
+        st.x[h] = (st.live >> h) & 1 ? (float)(px0 + lane_x<P>(lane, h)) + 0.5f : __uint_as_float(0x7fc00000u);
     sh.init_pad();
     FwdSpan<TILE, P, COUNT, LAZY, R> span{sh, xy_ab, c_o_z, rgbv, cullmode, tx, ty, st};
     // saving for the backward: the sorted chunks go back into the stream
@@ -512,7 +469,7 @@ __device__ __forceinline__ void raster_tile(
         pair_rows(st.last);
         if (COUNT) pair_rows(st.ntests);
     }
-    const int ox = px0 + (P == 2 ? (lane & 3) + (odd ? 4 : 0) : L::x(lane, 0));
+    const int ox = px0 + (P == 2 ? (lane & 3) + (odd ? 4 : 0) : lane_x<P>(lane, 0));
 #pragma unroll
     for (int h = 0; h < P; ++h) {
         const int oy = P == 2 ? py0 + ((lane >> 2) & ~1) + h : py;

@@ -80,6 +80,50 @@ __device__ __forceinline__ void entry_q(const float4& ga, const float4& gb, floa
     upk2(fma2(dx, fma2(same2(ga.z), dx, same2(ga.w * dy)), same2((gb.x * dy) * dy)), q0, q1);
 }
 
+// Values at a lane's P pixels.  Two, of a row of the warp's 8 x 8 block: they
+// share dy and the entry's shared-memory reads, and what is done to both runs on
+// packed float32 pairs (each half rounded as the scalar operation).  One: a
+// pixel of the warp's 8 x 4 block, scalar.
+template <int P>
+struct Lane;
+template <>
+struct Lane<2> {
+    using V = uint64_t;  // pixel 0 in the low half
+    static __device__ __forceinline__ V same(float v) { return same2(v); }
+    static __device__ __forceinline__ V put(const float (&v)[2]) { return pk2(v[0], v[1]); }
+    static __device__ __forceinline__ void get(V v, float (&o)[2]) { upk2(v, o[0], o[1]); }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return fma2(a, b, c); }
+    static __device__ __forceinline__ V mul(V a, V b) { return mul2(a, b); }
+    static __device__ __forceinline__ void exp_neg(const float (&q)[2], float (&e)[2])
+    {
+        spec_exp_neg2(q[0], q[1], e[0], e[1]);
+    }
+    static __device__ __forceinline__ float least(const float (&v)[2]) { return fminf(v[0], v[1]); }
+};
+template <>
+struct Lane<1> {
+    using V = float;
+    static __device__ __forceinline__ V same(float v) { return v; }
+    static __device__ __forceinline__ V put(const float (&v)[1]) { return v[0]; }
+    static __device__ __forceinline__ void get(V v, float (&o)[1]) { o[0] = v; }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return fmaf(a, b, c); }
+    static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
+    static __device__ __forceinline__ void exp_neg(const float (&q)[1], float (&e)[1]) { e[0] = spec_exp_core(-q[0]); }
+    static __device__ __forceinline__ float least(const float (&v)[1]) { return v[0]; }
+};
+
+// q of one staged entry at the lane's pixels (centres x[h], y).
+template <int P>
+__device__ __forceinline__ void entry_dist(const float4& ga, const float4& gb, const float (&x)[P], float y, float (&q)[P])
+{
+    if constexpr (P == 2) {
+        entry_q(ga, gb, x[0], x[1], y, q[0], q[1]);
+    } else {
+        const float dx = ga.x - x[0], dy = ga.y - y;
+        q[0] = fmaf(dx, fmaf(ga.z, dx, ga.w * dy), (gb.x * dy) * dy);
+    }
+}
+
 struct RasterArgs {
     int width, height, tiles_x, n_tiles, stride;
     float bg0, bg1, bg2;

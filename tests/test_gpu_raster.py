@@ -38,9 +38,10 @@ def test_ragged_sizes_and_pixels_a_lane(w, h, tile):
         assert_image(mode, sc, cam, tile, 64 if mode == "exact" else 1, ref)
 
 
-@pytest.mark.parametrize("w,h", [(640, 608), (641, 608)])
+@pytest.mark.parametrize("w,h", [(384, 608), (385, 608), (640, 608), (641, 608)])
 def test_both_sides_of_the_rule(w, h):
-    # 1520 tiles go by one pixel a lane, 1558 by two: the image, and the ends
+    # 1520 tiles go by one pixel a lane, 1558 by two (the backward's line lies
+    # between 912 and 950): the image, and the ends
     # of the 8 x 8 blocks that the backward starts from (it skips what lies
     # beyond, so a frame's gradients equal those of the stages, which walk on
     # to the tile's end, up to the order of their float32 atomics)
@@ -51,14 +52,16 @@ def test_both_sides_of_the_rule(w, h):
     dC, dA = (torch.from_numpy(x).cuda() for x in scenes.incoming_grads(h, w, seed=3))
     ds = G.DeviceScene.from_numpy(sc)
     ctx = G.Context("exact")
-    ctx.render(ds, cam, flags=G.RENDER_SAVE)
+    kept = ctx.render(ds, cam, flags=G.RENDER_SAVE)  # the backward reads its last-id output
     got = G.grad_fields(ctx.render_bwd(dC, dA), sc.n)
     proj = ctx.project(ds, cam)
     isect, m_cap, m_dev, _ = ctx.tile_intersect(proj, sc.n, cam)
     words, offsets, _ = ctx.sort_or_bin(proj, ds.scales, sc.n, cam, isect, m_cap, m_dev)
     saved = ctx.rasterize_fwd(proj, sc.n, cam, words, offsets, save=True)[3]
     want = G.grad_fields(ctx.rasterize_bwd(proj, sc.n, cam, words, offsets, saved, dC, dA), sc.n)
+    torch.cuda.synchronize()
     assert ctx.error() == 0
+    del kept
     for k in got:
         np.testing.assert_allclose(got[k].cpu(), want[k].cpu(), rtol=1e-5, atol=1e-6 * float(want[k].abs().max()))
 
