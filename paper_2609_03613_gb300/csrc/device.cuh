@@ -193,31 +193,35 @@ struct BucketMap {
     __device__ __forceinline__ int of(uint64_t w) const { return (int)(((uint32_t)(w >> 32) - lo) >> sh); }
 };
 
-// By a block of NT threads: src[0..n) into dst[0..n) in order of 1 << LOG
+// By a block of NT threads (32: by one warp of any block): src[0..n) into dst[0..n) in order of 1 << LOG
 // buckets, boff[q] (q <= 1 << LOG) the start of bucket q.  h: 1 << LOG words
 // of shared memory, red: 2 words a warp.  Returns (block-uniformly) whether
-// every bucket is short.  Ends with a block barrier; src may be global memory
+// every bucket is short.  Ends with a barrier; src may be global memory
 // that is not written meanwhile, n < 65536.
 template <int NT, int LOG>
 __device__ __forceinline__ bool block_buckets(const uint64_t* src, int n, uint64_t* dst, uint32_t* h, uint32_t* red,
                                               uint16_t* boff, BucketMap& map)
 {
     constexpr int NB = 1 << LOG, NW = NT / 32, PER = NB > NT ? NB / NT : 1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, tid = NT == 32 ? lane : (int)threadIdx.x, warp = tid >> 5;
+    auto sync = [] {
+        if constexpr (NT == 32) __syncwarp();
+        else __syncthreads();
+    };
     uint32_t lo = 0xffffffffu, hi = 0u;
-    for (int i = threadIdx.x; i < n; i += NT) {
+    for (int i = tid; i < n; i += NT) {
         const uint32_t z = (uint32_t)(src[i] >> 32);
         lo = min(lo, z);
         hi = max(hi, z);
     }
-    for (int k = threadIdx.x; k < NB; k += NT) h[k] = 0u;
+    for (int k = tid; k < NB; k += NT) h[k] = 0u;
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
     if (lane == 0) {
         red[warp] = lo;
         red[NW + warp] = hi;
     }
-    __syncthreads();
+    sync();
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
         lo = min(lo, red[w]);
@@ -226,12 +230,12 @@ __device__ __forceinline__ bool block_buckets(const uint64_t* src, int n, uint64
     const int bits = 32 - __clz(hi - lo);
     map.lo = lo;
     map.sh = bits > LOG ? bits - LOG : 0;
-    for (int i = threadIdx.x; i < n; i += NT) atomicAdd(&h[map.of(src[i])], 1u);
-    __syncthreads();  // also: red is read
+    for (int i = tid; i < n; i += NT) atomicAdd(&h[map.of(src[i])], 1u);
+    sync();  // also: red is read
     uint32_t c[PER], run = 0u, longest = 0u;
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
-        const int q = (int)threadIdx.x * PER + k;
+        const int q = tid * PER + k;
         c[k] = q < NB ? h[q] : 0u;
         run += c[k];
         longest = max(longest, c[k]);
@@ -243,25 +247,27 @@ __device__ __forceinline__ bool block_buckets(const uint64_t* src, int n, uint64
         if (lane >= d) incl += u;
     }
     if (lane == 31) red[warp] = incl;
-    const bool fits = __syncthreads_or(longest > (uint32_t)kBucketMax) == 0;
+    bool fits;
+    if constexpr (NT == 32) fits = !__any_sync(0xffffffffu, longest > (uint32_t)kBucketMax);
+    else fits = __syncthreads_or(longest > (uint32_t)kBucketMax) == 0;
     uint32_t e = incl - run;
     for (int w = 0; w < warp; ++w) e += red[w];
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
-        const int q = (int)threadIdx.x * PER + k;
+        const int q = tid * PER + k;
         if (q < NB) {
             boff[q] = (uint16_t)e;
             h[q] = e;
             e += c[k];
         }
     }
-    if (threadIdx.x == 0) boff[NB] = (uint16_t)n;
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += NT) {
+    if (tid == 0) boff[NB] = (uint16_t)n;
+    sync();
+    for (int i = tid; i < n; i += NT) {
         const uint64_t w = src[i];
         dst[atomicAdd(&h[map.of(w)], 1u)] = w;
     }
-    __syncthreads();
+    sync();
     return fits;
 }
 

@@ -66,14 +66,8 @@ def test_both_sides_of_the_rule(w, h):
         np.testing.assert_allclose(got[k].cpu(), want[k].cpu(), rtol=1e-5, atol=1e-6 * float(want[k].abs().max()))
 
 
-@pytest.mark.parametrize("depths", ["spread", "equal", "skewed"])
-@pytest.mark.parametrize("tile", [8, 16])
-@pytest.mark.parametrize("count", [128, 129, 256, 257, 512, 513, 2048, 2049, 8191, 8192, 8193])
-def test_segments_at_batch_and_sort_limits(count, tile, depths):
-    # one bin a tile holding `count` entries (all inside one tile, which stops
-    # after some two thousand of them): staged at
-    # rank, in depth buckets in the raster, or sorted before it.  Equal depths
-    # and depths crowded at one end fill a bucket past its limit.
+def one_tile(count, depths):
+    """`count` Gaussians inside one tile, which stops after some two thousand."""
     rng = np.random.default_rng(count)
     cam = scenes.tiny_camera()
     z = rng.uniform(-0.4, 0.4, count)
@@ -82,9 +76,30 @@ def test_segments_at_batch_and_sort_limits(count, tile, depths):
     elif depths == "skewed":
         z = 0.4 - 0.8 * rng.random(count) ** 40
     xy = (132.0 + rng.uniform(-1.0, 1.0, (count, 2)) - cam.cx) * (3.0 - z)[:, None] / cam.fx
-    sc = scenes.Scene(np.column_stack([xy, z]).astype(np.float32), np.full((count, 3), 0.002, np.float32),
-                      np.tile(np.array([1, 0, 0, 0], np.float32), (count, 1)),
-                      np.full(count, 0.0045, np.float32), rng.uniform(0, 1, (count, 1, 3)).astype(np.float32), 0)
+    return cam, scenes.Scene(np.column_stack([xy, z]).astype(np.float32), np.full((count, 3), 0.002, np.float32),
+                             np.tile(np.array([1, 0, 0, 0], np.float32), (count, 1)),
+                             np.full(count, 0.0045, np.float32), rng.uniform(0, 1, (count, 1, 3)).astype(np.float32), 0)
+
+
+@pytest.mark.parametrize("depths", ["spread", "equal", "skewed"])
+@pytest.mark.parametrize("tile", [8, 16])
+@pytest.mark.parametrize("count", [128, 129, 256, 257, 512, 513, 2048, 2049, 8191, 8192, 8193])
+def test_segments_at_batch_and_sort_limits(count, tile, depths):
+    # one bin a tile holding `count` entries: staged at rank, in depth buckets in
+    # the raster, or sorted before it.  Equal depths and depths crowded at one
+    # end fill a bucket past its limit.
+    cam, sc = one_tile(count, depths)
     P, ent, (off, stream), ref = O.render(sc, cam, tile, bg=(0.1, 0.2, 0.3))
     assert np.diff(off).max() == count
     assert_image("exact", sc, cam, tile, 1, ref)
+
+
+@pytest.mark.parametrize("depths", ["spread", "equal", "skewed"])
+@pytest.mark.parametrize("count", [2, 32, 33, 128, 512, 513, 4096, 4097])
+def test_segments_sorted_before_the_raster(count, depths):
+    # the repair outside the raster: a segment sorted in registers, by a warp, by
+    # a block (depth buckets; the network past a full bucket), or as a tail
+    cam, sc = one_tile(count, depths)
+    P, ent, (off, stream), ref = O.render(sc, cam, 16, bg=(0.1, 0.2, 0.3))
+    assert np.diff(off).max() == count
+    assert_image("exact", sc, cam, 16, 1, ref, repair_in_raster=0)
